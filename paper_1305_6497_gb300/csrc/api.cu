@@ -305,6 +305,7 @@ struct dda_target {
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   DevBuf comp, site, tw64, tw32, twdf, perm;  // perm: k_at x|y|z, then pos x|y|z
   DevBuf twzp;  // FP32 z twiddles of the column-pair kernel's plan (when it has one)
+  DevBuf twzr;  // FP32 z twiddles of the register kernel (when it has a plan)
   DevBuf zerr;  // one int: a kernel's bounded wait on a copy ran out
   AxisPlan px{}, py{}, pz{};
   int twoff[3] = {0, 0, 0};
@@ -358,6 +359,7 @@ static OpView<T> make_view(const dda_target* t, const void* ghat, const void* ai
   v.kz_at = pm + t->Lx + t->Ly;
   v.ypos_at = pm + (t->Lx + t->Ly + t->Lz) + t->Lx;
   v.twz_pair = t->twzp.as<float2>();
+  v.twz_reg = t->twzr.as<float4>();
   v.zerr = t->zerr.as<int>();
   v.px = t->px; v.py = t->py; v.pz = t->pz;
   auto magic = [](int d) { return ((1ull << 36) + (unsigned long long)d - 1) / (unsigned long long)d; };
@@ -1397,6 +1399,7 @@ void dda_target_destroy(dda_target* t) {
   t->ws.release_all();
   t->comp.release(); t->site.release(); t->tw64.release(); t->tw32.release(); t->twdf.release();
   t->twzp.release();
+  t->twzr.release();
   t->zerr.release();
   t->perm.release();
   t->g64.release(); t->g32.release(); t->gdf.release(); t->h64.release();
@@ -1521,6 +1524,21 @@ dda_status dda_target_create(int nx, int ny, int nz, const uint8_t* occ, const u
       t->twzp.ensure(sizeof(float2) * tp.size());
       CK(cudaMemcpy(t->twzp.p, tp.data(), sizeof(float2) * tp.size(), cudaMemcpyHostToDevice));
     }
+    // and of the register z kernel: w_L^(j2 (2 k1 + parity)), [k1 < R1][j2 < R2],
+    // both parities side by side (re, im even; re, im odd)
+    int r1 = 0, r2 = 0;
+    if (z_reg_plan(t->Lz, t->nz, &r1, &r2)) {
+      std::vector<float4> tr;
+      const long double two_pi = 6.283185307179586476925286766559L;
+      for (int k = 0; k < r1; ++k)
+        for (int j = 0; j < r2; ++j) {
+          const long double a = -two_pi * (long double)((2LL * j * k) % t->Lz) / t->Lz;
+          const long double b = -two_pi * (long double)(((2LL * k + 1) * j) % t->Lz) / t->Lz;
+          tr.push_back(make_float4((float)cosl(a), (float)sinl(a), (float)cosl(b), (float)sinl(b)));
+        }
+      t->twzr.ensure(sizeof(float4) * tr.size());
+      CK(cudaMemcpy(t->twzr.p, tr.data(), sizeof(float4) * tr.size(), cudaMemcpyHostToDevice));
+    }
   } catch (const CudaFail& f) {
     dda_status s = from_cuda(f);
     dda_target_destroy(t);
@@ -1559,7 +1577,7 @@ int64_t dda_solve_hbm_bytes(const dda_target* t, const dda_solve_params* p) {
 // workspace and its near-field box.
 static int64_t held_bytes(dda_target* t) {
   int64_t b = 0;
-  for (const DevBuf* d : {&t->comp, &t->site, &t->tw64, &t->tw32, &t->twdf, &t->twzp, &t->perm,
+  for (const DevBuf* d : {&t->comp, &t->site, &t->tw64, &t->tw32, &t->twdf, &t->twzp, &t->twzr, &t->perm,
                           &t->g64, &t->g32, &t->gdf, &t->h64})
     b += (int64_t)d->bytes;
   b += t->ws.bytes();
@@ -1593,8 +1611,9 @@ int64_t dda_estimate_solve_bytes(int nx, int ny, int nz, int64_t n_dipoles, int 
   if (solve < 0) return -1;
   const int64_t Lsum = (int64_t)d.Lx + d.Ly + d.Lz;
   // dda_target_create: composition grid, site list, twiddles (FP64, FP32,
-  // double-float) and the frequency/position tables
-  const int64_t created = nbox + 8 * n_dipoles + Lsum * (16 + 8 + 16) + 2 * Lsum * 4 + 3 * 256;
+  // double-float, and the FP32 z kernels' own) and the frequency/position tables
+  const int64_t created = nbox + 8 * n_dipoles + Lsum * (16 + 8 + 16) + 2 * Lsum * 4 +
+                          16 * (int64_t)d.Lz + 3 * 256;
   return created + solve;
 }
 
@@ -2134,7 +2153,8 @@ void apply_schedule(const dda_target* t, MatvecLaunch& L, const std::vector<int>
   L.z_ps = v[3];
   // z staging 2, 3: the column-pair kernel, Ghat through L2 (2) or staged (3);
   // +4: its column tiles moved by TMA
-  L.z_pair = v[4] >= 6 ? 2 : v[4] >= 2 ? 1 : 0;
+  // 8: the two-step register kernel
+  L.z_pair = v[4] == 8 ? 3 : v[4] >= 6 ? 2 : v[4] >= 2 ? 1 : 0;
   L.z_gs = v[4] == 1 || v[4] == 3 || v[4] == 7;
   const int Hz = t->Lz / 2 + 1;
   L.z_smem = (((size_t)t->Lz * L.z_ps * sizeof(C) + 15) & ~(size_t)15) +
@@ -2143,7 +2163,7 @@ void apply_schedule(const dda_target* t, MatvecLaunch& L, const std::vector<int>
 
 std::vector<int> schedule_of(const MatvecLaunch& L) {
   return {L.x_lines, L.y_tile, L.z_tile, L.z_ps,
-          (L.z_pair ? 2 : 0) + (L.z_pair == 2 ? 4 : 0) + (L.z_gs ? 1 : 0),
+          L.z_pair == 3 ? 8 : (L.z_pair ? 2 : 0) + (L.z_pair == 2 ? 4 : 0) + (L.z_gs ? 1 : 0),
           L.x_threads, L.y_threads, L.z_threads};
 }
 }  // namespace
@@ -2304,20 +2324,23 @@ dda_status dda_set_schedule(dda_target* t, int precision, const int* in8) {
   const bool f64 = precision == DDA_PREC_FP64;
   const size_t cs = f64 ? sizeof(double2) : sizeof(float2);
   if (xl < 1 || xl > 64 || yt < 1 || yt > 64 || (zt != 2 && zt != 4 && zt != 8 && zt != 16) ||
-      zp < 3 * zt || zp > 3 * zt + 8 || zg < 0 || zg > 7 || zg == 4 || zg == 5)
+      zp < 3 * zt || zp > 3 * zt + 8 || zg < 0 || zg > 8 || zg == 4 || zg == 5)
     return fail(DDA_ERR_INVALID_ARG, "schedule: x lines 1..64, y tile 1..64, z tile 2/4/8/16, "
-                                     "z pitch 3*tile..3*tile+8, z staging 0, 1, 2, 3, 6 or 7");
-  if (zg >= 2 && (f64 || !z_pair_applies(t->Lz, t->Lx, zt) || in8[7] != kZPairThreads))
+                                     "z pitch 3*tile..3*tile+8, z staging 0, 1, 2, 3, 6, 7 or 8");
+  if (zg == 8 && (f64 || zt != kZRegTile || !z_reg_plan(t->Lz, t->nz, nullptr, nullptr)))
+    return fail(DDA_ERR_INVALID_ARG, "schedule: z staging 8 (register z kernel) needs FP32, z tile "
+                                     "8 and an even Lz with a two-factor plan");
+  if (zg >= 2 && zg != 8 && (f64 || !z_pair_applies(t->Lz, t->Lx, zt) || in8[7] != kZPairThreads))
     return fail(DDA_ERR_INVALID_ARG, "schedule: z staging 2/3/6/7 (column-pair z kernel) needs "
                                      "FP32, an even Lx, Lz of 64, 128, 288 or 512, tile 4 or 8 "
                                      "and 384 threads");
-  if (zg >= 6 && !z_pair_tma_applies(t->Lz, t->Lx, t->nz, zt))
+  if ((zg == 6 || zg == 7) && !z_pair_tma_applies(t->Lz, t->Lx, t->nz, zt))
     return fail(DDA_ERR_INVALID_ARG, "schedule: z staging 6/7 (TMA tiles) needs nz <= 256");
   for (int i = 5; i < 8; ++i) {
     // the FP32 z pass of a compiled radix plan (and the column-pair one) takes
     // up to 384 threads
     const int tmax =
-        (i == 7 && !f64 && (z_fixed_applies(t->pz, zt) || zg >= 2)) ? 384 : 256;
+        (i == 7 && !f64 && (z_fixed_applies(t->pz, zt) || (zg >= 2 && zg != 8))) ? 384 : 256;
     if (in8[i] < 32 || in8[i] > tmax || in8[i] % 32)
       return fail(DDA_ERR_INVALID_ARG, "schedule: threads per CTA must be a multiple of 32 in "
                                        "32..256 (FP32 z pass of a compiled plan: ..384)");
@@ -2327,7 +2350,7 @@ dda_status dda_set_schedule(dda_target* t, int precision, const int* in8) {
   // a compiled-plan z kernel uses its own pitch, 3 tile (+1 below 128 B rows)
   const int zpc = (!f64 && z_fixed_applies(t->pz, zt))
                       ? std::max(zp, 3 * zt + (zt * (int)cs < 128 ? 1 : 0)) : zp;
-  const size_t zsm = zg >= 2 ? zpair_smem_bytes(t->Lz, zt, zg == 3 || zg == 7)
+  const size_t zsm = zg == 8 ? 0 : zg >= 2 ? zpair_smem_bytes(t->Lz, zt, zg == 3 || zg == 7)
                              : (((size_t)t->Lz * zpc * cs + 15) & ~(size_t)15) +
                                    (zg ? (size_t)6 * (t->Lz / 2 + 1) * zt * cs : 0);
   if (xinv > 200 * 1024 || ysm > 200 * 1024 || zsm > 200 * 1024)

@@ -8,8 +8,9 @@
 //    z pass transforms along z, multiplies by the Green tensor transform and
 //    transforms back in place, and the inverse y and x passes shrink back;
 //  - Green tensor transform: one octant [Lz/2+1][Ly/2+1][Lx/2+1][6] complex
-//    (components xx, xy, xz, yy, yz, zz side by side), the rest follows from
-//    the parity of each component in each axis.
+//    (components xx, xy, xz, yy, yz, zz side by side; FP32:
+//    [Ly/2+1][Lx/2+1][3][Lz/2+1][2], pairs of components with hz fastest), the
+//    rest follows from the parity of each component in each axis.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -151,6 +152,13 @@ __host__ __device__ __forceinline__ int fast_div(int q, unsigned long long m) {
   return (int)(((unsigned long long)q * m) >> 36);
 }
 
+// Element (complex) of component c (xx, xy, xz, yy, yz, zz) at octant point
+// (hz, hy, hx) of the FP32 Green transform.
+__host__ __device__ __forceinline__ int64_t ghat_f32_offset(int Hx, int Hz, int hz, int hy, int hx,
+                                                            int c) {
+  return ((((int64_t)hy * Hx + hx) * 3 + (c >> 1)) * Hz + hz) * 2 + (c & 1);
+}
+
 // Everything a matvec kernel needs about one target's operator.
 template <typename T> struct OpView {
   using C = cplx_t<T>;
@@ -159,7 +167,8 @@ template <typename T> struct OpView {
   int Hx, Hy, Hz;                 // octant sizes L/2 + 1
   int64_t nbox;                   // nx*ny*nz
   const uint8_t* comp;            // [nbox] 0 = vacant, else composition 1..ncomp
-  const C* ghat;                  // [Hz][Hy][Hx][6], already divided by Lx*Ly*Lz
+  const C* ghat;                  // octant, already divided by Lx*Ly*Lz: [Hz][Hy][Hx][6],
+                                  // FP32 [Hy][Hx][3][Hz][2] (see ghat_f32_offset)
   const C* ainv;                  // [R][ncomp+1][3] alpha^{-1} per RHS and lattice axis
                                   // (the polarizability tensor's diagonal), entry 0 unused
   int ncomp1;                     // ncomp + 1
@@ -167,6 +176,7 @@ template <typename T> struct OpView {
   const int* kx_at; const int* ky_at; const int* kz_at;  // frequency held at each
                                                           // digit-reversed position
   const int* ypos_at;             // position holding each y frequency (inverse of ky_at)
+  const float4* twz_reg;          // z twiddles of the register kernel (FP32), or null
   const float2* twz_pair;         // z twiddles of the column-pair kernel's plan (FP32), or null
   int* zerr;                      // set to 1 by a kernel whose bounded wait on a copy ran out
   unsigned long long div_nx, div_ny, div_nz, div_Lx;     // fast_div magics

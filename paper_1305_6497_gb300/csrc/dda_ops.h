@@ -25,7 +25,8 @@ struct MatvecLaunch {
   int y_tile, y_threads; size_t y_smem;
   int z_tile, z_ps, z_threads; size_t z_smem;
   bool z_gs;   // Ghat tile staged in shared memory
-  int z_pair;  // FP32: the column-pair z kernel (k_fft_z_pairs); 2: with TMA tiles
+  int z_pair;  // FP32: the column-pair z kernel (k_fft_z_pairs); 2: with TMA tiles;
+               // 3: the two-step register kernel (k_fft_z_reg)
 };
 
 template <typename T> MatvecLaunch plan_matvec(const OpView<T>& op);
@@ -108,6 +109,13 @@ bool z_pair_applies(int Lz, int Lx, int tile);
 constexpr int kZPairThreads = 384;
 // Dynamic shared memory of the column-pair z kernel (with the Ghat tile if gs).
 size_t zpair_smem_bytes(int Lz, int tile, bool gs);
+// The two-step register z kernel (FP32, zpass_reg.cuh) covers z length Lz of a box
+// of nz planes: Lz even, Lz / 2 = R1 R2 in its list of plans (R1, R2 returned
+// unless null) and (R1 - 1) R2 <= nz <= Lz / 2, so that only the last of a thread's
+// R1 rows can lie beyond the box (of the smooth lengths up to 512 this leaves out
+// the boxes of 163 to 167 planes).
+bool z_reg_plan(int Lz, int nz, int* R1, int* R2);
+constexpr int kZRegTile = 8;
 // The column-pair kernel's TMA variant applies as well: nz <= 256 (a box
 // dimension), 2 nz <= Lz, and a driver that encodes tensor maps.
 bool z_pair_tma_applies(int Lz, int Lx, int nz, int tile);

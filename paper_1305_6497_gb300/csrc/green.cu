@@ -298,7 +298,8 @@ __global__ void k_green_octant(int Lx, int Ly, int Lz, const int* __restrict__ p
     const double2 v = full[c * M + ((int64_t)posz[hz] * Ly + posy[hy]) * Lx + posx[hx]];
     const double2 w = make_double2(v.x * inv, v.y * inv);
     g64[6 * o + c] = w;  // the six components of a point side by side
-    if (g32) g32[6 * o + c] = make_float2((float)w.x, (float)w.y);
+    if (g32)
+      g32[ghat_f32_offset(Hx, Hz, hz, hy, hx, c)] = make_float2((float)w.x, (float)w.y);
   }
 }
 

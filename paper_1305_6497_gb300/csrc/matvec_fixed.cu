@@ -9,6 +9,7 @@
 
 #include "matvec_impl.cuh"
 #include "zpass_pair.cuh"
+#include "zpass_reg.cuh"
 
 namespace dda {
 
@@ -149,9 +150,32 @@ bool encode_zpair_map(CUtensorMap* map, const float2* scratch, int Lx, int Ly, i
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// the two-step register kernel, instantiated in zpass_reg_*.cu
+bool z_reg_plan(int Lz, int nz, int* R1, int* R2) {
+  if (Lz % 2) return false;
+  switch (Lz / 2) {
+#define DDA_ZREG_PLAN(A, B) \
+  case (A) * (B):           \
+    if (R1) *R1 = (A);      \
+    if (R2) *R2 = (B);      \
+    return nz <= (A) * (B) && nz >= ((A) - 1) * (B);
+    DDA_ZREG_ALL(DDA_ZREG_PLAN)
+#undef DDA_ZREG_PLAN
+  }
+  return false;
+}
+
+static bool launch_z_reg_any(const OpView<float>& op, int R, float2* buf, const int* active,
+                             cudaStream_t st) {
+  return launch_z_reg_part0(op, R, buf, active, st) || launch_z_reg_part1(op, R, buf, active, st) ||
+         launch_z_reg_part2(op, R, buf, active, st) || launch_z_reg_part3(op, R, buf, active, st) ||
+         launch_z_reg_part4(op, R, buf, active, st) || launch_z_reg_part5(op, R, buf, active, st);
+}
+
 bool launch_z_fixed(const OpView<float>& op, const MatvecLaunch& L, int R, float2* scratch,
                     const int* active, cudaStream_t st) {
   bool done = false;
+  if (L.z_pair == 3) return op.twz_reg && op.Lz % 2 == 0 && launch_z_reg_any(op, R, scratch, active, st);
   if (L.z_pair) {
     if (!z_pair_applies(op.Lz, op.Lx, L.z_tile) || !op.twz_pair) return false;
     dispatch_length(op.Lz, PairPlans{}, [&](auto plan) {
@@ -312,6 +336,8 @@ cudaError_t configure_fixed_kernels() {
     ok(set_smem((const void*)k_fft_x_inv<float, XOUT_QT, P>));
   };
   xcfg(P16x8{}); xcfg(P16x4{}); xcfg(P16x8x4{}); xcfg(P8x4x3{});
+  ok(configure_z_reg_part0()); ok(configure_z_reg_part1()); ok(configure_z_reg_part2());
+  ok(configure_z_reg_part3()); ok(configure_z_reg_part4()); ok(configure_z_reg_part5());
   return e;
 }
 

@@ -342,8 +342,18 @@ template <typename C> struct ZIO {
   }
 };
 
-// The six components of Ghat at octant point o are stored together,
-// ghat[6 o .. 6 o + 5] = xx, xy, xz, yy, yz, zz (48 B in FP32, 96 B in FP64).
+// The six components of Ghat at an octant point, xx, xy, xz, yy, yz, zz: side by
+// side in FP64 and double-float ([hz][hy][hx][6]); in FP32 three 16-byte pieces
+// (xx xy | xz yy | yz zz) ghat_piece_f32(op) elements apart, each piece a plane
+// with hz fastest ([hy][hx][3][hz][2]), so that threads at neighbouring z
+// frequencies of one column read neighbouring 16-byte words.
+template <typename T>
+__device__ __forceinline__ const cplx_t<T>* ghat_at(const OpView<T>& op, int hz, int hy, int hx) {
+  if constexpr (std::is_same<T, float>::value)
+    return op.ghat + ghat_f32_offset(op.Hx, op.Hz, hz, hy, hx, 0);
+  else
+    return op.ghat + 6 * (((int64_t)hz * op.Hy + hy) * op.Hx + hx);
+}
 template <typename T> struct G6;
 template <> struct G6<float> {
   static __device__ __forceinline__ void load_smem(const float2* g, float2 (&v)[6]) {
@@ -353,9 +363,9 @@ template <> struct G6<float> {
     v[2] = make_float2(b.x, b.y); v[3] = make_float2(b.z, b.w);
     v[4] = make_float2(c.x, c.y); v[5] = make_float2(c.z, c.w);
   }
-  static __device__ __forceinline__ void load(const float2* g, float2 (&v)[6]) {
+  static __device__ __forceinline__ void load(const float2* g, int Hz, float2 (&v)[6]) {
     const float4* q = reinterpret_cast<const float4*>(g);
-    const float4 a = __ldg(q), b = __ldg(q + 1), c = __ldg(q + 2);
+    const float4 a = __ldg(q), b = __ldg(q + Hz), c = __ldg(q + 2 * Hz);
     v[0] = make_float2(a.x, a.y); v[1] = make_float2(a.z, a.w);
     v[2] = make_float2(b.x, b.y); v[3] = make_float2(b.z, b.w);
     v[4] = make_float2(c.x, c.y); v[5] = make_float2(c.z, c.w);
@@ -371,7 +381,7 @@ template <> struct G6<df64> {
       v[i].y = df64(a.z, a.w);
     }
   }
-  static __device__ __forceinline__ void load(const df64c* g, df64c (&v)[6]) {
+  static __device__ __forceinline__ void load(const df64c* g, int, df64c (&v)[6]) {
 #pragma unroll
     for (int i = 0; i < 6; ++i) v[i] = ldc(g + i);
   }
@@ -381,7 +391,7 @@ template <> struct G6<double> {
 #pragma unroll
     for (int i = 0; i < 6; ++i) v[i] = g[i];
   }
-  static __device__ __forceinline__ void load(const double2* g, double2 (&v)[6]) {
+  static __device__ __forceinline__ void load(const double2* g, int, double2 (&v)[6]) {
 #pragma unroll
     for (int i = 0; i < 6; ++i) v[i] = __ldg(g + i);
   }
@@ -448,7 +458,7 @@ __device__ __forceinline__ void z_mid(cplx_t<T>* s, int ps, int ncol, int col0, 
           G6<T>::load_smem(gs + 6 * (hz * TILE + t), g);
         } else {
           const int hx = fx ? op.Lx - kx : kx;
-          G6<T>::load(op.ghat + 6 * (((int64_t)hz * op.Hy + hy) * op.Hx + hx), g);
+          G6<T>::load(ghat_at<T>(op, hz, hy, hx), op.Hz, g);
         }
         spectral_mul<T, CROSS>(g, fx, fy, fz, q + i * ps, TILE);
       }
@@ -474,15 +484,14 @@ __device__ __forceinline__ void ghat_tile_async(const OpView<T>& op, cplx_t<T>* 
                                                 int ncol, int hy) {
   constexpr int CH = 6 * (int)sizeof(cplx_t<T>) / 16;  // 16-byte chunks per point
   const int n = op.Hz * TILE * CH;
-  const int64_t plane = (int64_t)op.Hy * op.Hx;
   for (int e = threadIdx.x; e < n; e += blockDim.x) {
     const int ch = e % CH, pt = e / CH;
     const int t = pt % TILE, hz = pt / TILE;
     if (t < ncol) {
       const int kx = op.kx_at[col0 + t];
       const int hx = kx > (op.Lx >> 1) ? op.Lx - kx : kx;
-      const char* src = reinterpret_cast<const char*>(
-          op.ghat + 6 * (hz * plane + (int64_t)hy * op.Hx + hx)) + 16 * ch;
+      const int64_t piece = std::is_same<T, float>::value ? 16 * (int64_t)op.Hz : 16;
+      const char* src = reinterpret_cast<const char*>(ghat_at<T>(op, hz, hy, hx)) + piece * ch;
       char* dst = reinterpret_cast<char*>(gs + 6 * (hz * TILE + t)) + 16 * ch;
       cp_async<16>(dst, src);
     }
@@ -539,7 +548,7 @@ k_fft_z_mul(OpView<T> op, cplx_t<T>* __restrict__ buf, int ps, const int* __rest
       const bool fx = kx > (Lx >> 1);
       C g[6];
       if (GS) G6<T>::load_smem(gs + 6 * t, g);
-      else G6<T>::load(op.ghat + 6 * ((int64_t)hy * op.Hx + (fx ? Lx - kx : kx)), g);
+      else G6<T>::load(ghat_at<T>(op, 0, hy, fx ? Lx - kx : kx), op.Hz, g);
       spectral_mul<T, CROSS>(g, fx, fy, false, s + t, TILE);
     }
     __syncthreads();
@@ -656,7 +665,7 @@ k_fft_z_mul_p(OpView<float> op, float2* __restrict__ buf, const int* __restrict_
             G6<float>::load_smem(gs + 6 * (hz * TILE + t), g);
           } else {
             const int hx = fx ? Lx - kx : kx;
-            G6<float>::load(op.ghat + 6 * (((int64_t)hz * op.Hy + hy) * op.Hx + hx), g);
+            G6<float>::load(ghat_at<float>(op, hz, hy, hx), op.Hz, g);
           }
           spectral_mul<float, false>(g, fx, fy, fz, q + i * PS, TILE);
         }
@@ -992,6 +1001,15 @@ MatvecLaunch plan_matvec(const OpView<T>& op) {
     const size_t d = ((size_t)op.Lz * pitch(tt) * sizeof(C) + 15) & ~(size_t)15;
     return d + (gsm ? (size_t)6 * op.Hz * tt * sizeof(C) : 0);
   };
+  // FP32 with a two-step plan: the register kernel, faster than every other at
+  // all sizes measured (zpass_reg.cuh); its tile, pitch and threads are its own
+  if (std::is_same<T, float>::value && z_reg_plan(op.Lz, op.nz, nullptr, nullptr)) {
+    L.z_pair = 3;
+    L.z_tile = kZRegTile;
+    L.z_ps = 3 * kZRegTile;
+    L.z_threads = 256;
+    return L;
+  }
   int tz = tz_min;
   L.z_gs = zbytes(tz, true) <= 64 * 1024;
   if (!L.z_gs)

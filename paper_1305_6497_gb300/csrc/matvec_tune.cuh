@@ -131,7 +131,7 @@ cudaError_t autotune_matvec(const OpView<T>& op, MatvecLaunch& L, int R, const c
         if (tt < bt) { bt = tt; best = c; }
       }
   }
-  // z pass
+  // z pass (the register kernel is the starting point where it has a plan)
   {
     float bt = time_pass<T>(op, best, 2, R, x, y, scratch, st, e0, e1, reps, ks, part, fold);
     for (int tile : {2, 4, 8, 16})

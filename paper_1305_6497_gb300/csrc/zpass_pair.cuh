@@ -228,14 +228,13 @@ __device__ __forceinline__ void ghat_tile_pairs_async(const OpView<float>& op, f
                                                       int col0, int ncol, int hy) {
   const int stride = zpair_gstride(op.Hz, TILE);
   const int n = op.Hz * TILE * 3;  // 16-byte chunks: 3 per point
-  const int64_t plane = (int64_t)op.Hy * op.Hx;
   for (int e = threadIdx.x; e < n; e += blockDim.x) {
     const int ch = e % 3, pt = e / 3;
     const int hz = pt % op.Hz, t = pt / op.Hz;
     if (t < ncol) {
       const int kx = op.kx_at[col0 + t];
       const int hx = kx > (op.Lx >> 1) ? op.Lx - kx : kx;
-      const float2* src = op.ghat + 6 * (hz * plane + (int64_t)hy * op.Hx + hx) + 2 * ch;
+      const float2* src = ghat_at<float>(op, hz, hy, hx) + (int64_t)2 * op.Hz * ch;
       cp_async<16>(gs + t * stride + 6 * hz + 2 * ch, src);
     }
   }
@@ -434,7 +433,7 @@ k_fft_z_pairs(OpView<float> op, float2* __restrict__ buf, int R, const int* __re
           if (GS) {
             G6<float>::load_smem(gs + (2 * tp2 + e) * gstride + 6 * hz, g);
           } else {
-            G6<float>::load(op.ghat + 6 * (((int64_t)hz * op.Hy + hy) * op.Hx + hxm[e]), g);
+            G6<float>::load(ghat_at<float>(op, hz, hy, hxm[e]), op.Hz, g);
           }
           spectral_mul<float, false>(g, fxm[e], fy, fz, e ? bb : a, 1);
         }

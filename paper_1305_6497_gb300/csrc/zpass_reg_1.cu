@@ -1,0 +1,6 @@
+// Instances of the two-step register z pass (zpass_reg.cuh), part 1.
+#include "zpass_reg.cuh"
+
+namespace dda {
+DDA_ZREG_DEFINE(1)
+}  // namespace dda

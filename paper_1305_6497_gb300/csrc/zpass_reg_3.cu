@@ -1,0 +1,6 @@
+// Instances of the two-step register z pass (zpass_reg.cuh), part 3.
+#include "zpass_reg.cuh"
+
+namespace dda {
+DDA_ZREG_DEFINE(3)
+}  // namespace dda

@@ -1,0 +1,80 @@
+"""The two-step register z kernel (z kind 8, the FP32 default): the same product
+as the general one-tile kernel and the FP64 one, at the edges of its plans."""
+import numpy as np
+import pytest
+
+from dda_inputs import targets as tg
+from dda_inputs import workloads as W
+from oracle import dda as O
+
+pytestmark = pytest.mark.gpu
+
+# z extents at both ends of a plan (full lines, and the shortest box of a length),
+# plans whose first step leaves part of a warp idle (9, 11, 26), 4 and 8 column
+# tiles, odd Lx (no asynchronous copies), fewer columns than a tile, odd Ly
+SHAPES = [(2, 3, 9), (3, 5, 11), (13, 8, 12), (8, 13, 16), (14, 9, 26), (9, 11, 32), (10, 7, 33),
+          (7, 10, 64), (13, 6, 76), (5, 9, 96), (12, 5, 97), (6, 7, 128), (3, 9, 129),
+          (10, 4, 144), (5, 6, 168), (13, 4, 162), (4, 6, 200), (5, 4, 216), (4, 5, 225),
+          (6, 4, 251), (5, 5, 256)]
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+def test_register_z_kernel_matches(shape):
+    from paper_1305_6497_gb300 import binding as B
+    occ, comp = tg.rect_prism(*shape)
+    flat, pos = O.site_positions(occ)
+    x = O.box_to_sites(W.random_polarization(occ, 11)[0], flat)
+    t = B.Target(occ, comp, [1.5 + 0.1j], method="GKDLDR")
+    kh, e = np.array([0.36, 0.48, 0.8]), [0.8, -0.6, 0]
+    sch = t.schedule("fp32") if t.matvec(0.4, x, kh, e, "fp32") is not None else None
+    assert sch["z_stage_ghat"] == 8
+    y8 = t.matvec(0.4, x, kh, e, "fp32")
+    y64 = t.matvec(0.4, x, kh, e, "fp64")
+    t.set_schedule(dict(sch, z_tile=4, z_pitch=13, z_stage_ghat=0, z_threads=128), "fp32")
+    y0 = t.matvec(0.4, x, kh, e, "fp32")
+    # six transforms of at most nine radix-2 levels, each rounding to 2^-24
+    tol = 6 * 9 * 2.0 ** -24
+    top = np.abs(y64).max()
+    assert np.abs(y8 - y64).max() <= tol * top
+    assert np.abs(y8 - y0).max() <= 2 * tol * top
+    rows = np.arange(0, len(flat), max(1, len(flat) // 40))
+    ainv = O.site_alpha_inverse(comp.reshape(-1)[flat], [1.5 + 0.1j], "GKDLDR", 0.4, kh)
+    ref = O.matvec_direct(x, pos, ainv, 0.4, "GKDLDR", rows=rows)
+    assert np.abs(y8[rows] - ref).max() <= tol * top
+    t.set_schedule(sch, "fp32")
+    assert t.schedule("fp32")["z_stage_ghat"] == 8
+    assert np.array_equal(t.matvec(0.4, x, kh, e, "fp32"), y8)
+    t.close()
+
+
+def test_batches_and_frozen_right_hand_sides():
+    """Several right-hand sides, some converged before others, with one and with
+    several passes per CTA."""
+    from paper_1305_6497_gb300 import binding as B
+    for shape, n_orient in (((9, 12, 11), 3), ((40, 64, 64), 5)):
+        w = W.small_ellipsoid(*shape, m=1.5 + 0.1j, kd=0.3, method="LDR", n_orient=n_orient, seed=9)
+        t = B.Target(w.occ, w.comp, w.m, method="LDR")
+        kw = dict(yhat=w.yhat, npol=2, tol=1e-9, precision="fp32_refined")
+        a = t.solve(w.kd, w.khat, w.e01, **kw)
+        assert t.schedule("fp32")["z_stage_ghat"] == 8 and a["status"] == B.DDA_OK
+        t.set_schedule(dict(t.schedule("fp32"), z_tile=4, z_pitch=13, z_stage_ghat=0,
+                            z_threads=128), "fp32")
+        b = t.solve(w.kd, w.khat, w.e01, **kw)
+        assert np.all(np.abs(b["Qext"] / a["Qext"] - 1) < 1e-7)
+        assert np.abs(b["P"] - a["P"]).max() <= 1e-7 * np.abs(a["P"]).max()
+        t.close()
+
+
+def test_register_z_kernel_is_refused_where_it_has_no_plan():
+    from paper_1305_6497_gb300 import binding as B
+    for nz in (13, 125, 165):      # odd Lz, no two-factor plan, two rows beyond the box
+        occ, comp = tg.rect_prism(4, 3, nz)
+        t = B.Target(occ, comp, [1.5 + 0.1j], method="CM")
+        x = np.ones((t.num_dipoles, 3), np.complex128)
+        y = t.matvec(0.3, x, precision="fp32")
+        assert np.abs(y - t.matvec(0.3, x, precision="fp64")).max() <= 4e-6 * np.abs(y).max()
+        s = t.schedule("fp32")
+        assert s["z_stage_ghat"] != 8
+        with pytest.raises(B.DDAError):
+            t.set_schedule(dict(s, z_tile=8, z_pitch=24, z_stage_ghat=8), "fp32")
+        t.close()
