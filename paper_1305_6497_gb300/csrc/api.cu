@@ -10,6 +10,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/dda.h"
@@ -305,7 +306,8 @@ struct dda_target {
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   DevBuf comp, site, tw64, tw32, twdf, perm;  // perm: k_at x|y|z, then pos x|y|z
   DevBuf twzp;  // FP32 z twiddles of the column-pair kernel's plan (when it has one)
-  DevBuf twzr;  // FP32 z twiddles of the register kernel (when it has a plan)
+  DevBuf twr;   // FP32 twiddles of the register passes, x | y | z (axes with a plan)
+  int twroff[3] = {-1, -1, -1};
   DevBuf zerr;  // one int: a kernel's bounded wait on a copy ran out
   AxisPlan px{}, py{}, pz{};
   int twoff[3] = {0, 0, 0};
@@ -354,12 +356,18 @@ static OpView<T> make_view(const dda_target* t, const void* ghat, const void* ai
   v.twy = tb + t->twoff[1];
   v.twz = tb + t->twoff[2];
   const int* pm = t->perm.as<int>();
-  v.kx_at = pm;
+  // k_at x | y | z, positions x | y | z, then the identity (natural order)
+  const int* id = pm + 2 * (t->Lx + t->Ly + t->Lz);
+  const bool f32 = std::is_same<T, float>::value;
+  v.kx_at = f32 && t->L32.x_reg ? id : pm;
   v.ky_at = pm + t->Lx;
   v.kz_at = pm + t->Lx + t->Ly;
   v.ypos_at = pm + (t->Lx + t->Ly + t->Lz) + t->Lx;
   v.twz_pair = t->twzp.as<float2>();
-  v.twz_reg = t->twzr.as<float4>();
+  const float4* tr = t->twr.as<float4>();
+  v.twx_reg = t->twroff[0] < 0 ? nullptr : tr + t->twroff[0];
+  v.twy_reg = t->twroff[1] < 0 ? nullptr : tr + t->twroff[1];
+  v.twz_reg = t->twroff[2] < 0 ? nullptr : tr + t->twroff[2];
   v.zerr = t->zerr.as<int>();
   v.px = t->px; v.py = t->py; v.pz = t->pz;
   auto magic = [](int d) { return ((1ull << 36) + (unsigned long long)d - 1) / (unsigned long long)d; };
@@ -1329,7 +1337,8 @@ static void ensure_workspace(dda_target* t, int R, dda_precision prec, int ndir)
   }
   const int rows = 3 * t->nz * t->ny;
   const int nblk = std::max({reduce_blocks(3 * t->nbox), (rows + t->L32.x_lines - 1) / t->L32.x_lines,
-                             (rows + t->L64.x_lines - 1) / t->L64.x_lines});
+                             (rows + t->L64.x_lines - 1) / t->L64.x_lines,
+                             t->L32.x_reg ? x_reg_blocks(t->Lx, rows) : 1});
   const int fblk = std::min(reduce_blocks(t->nbox), 304);
   w.partials.ensure((size_t)std::max((int64_t)8 * R * nblk, (int64_t)12 * (ndir + 1) * fblk) * 8);
   w.ks.ensure(sizeof(KState) * R);
@@ -1399,7 +1408,7 @@ void dda_target_destroy(dda_target* t) {
   t->ws.release_all();
   t->comp.release(); t->site.release(); t->tw64.release(); t->tw32.release(); t->twdf.release();
   t->twzp.release();
-  t->twzr.release();
+  t->twr.release();
   t->zerr.release();
   t->perm.release();
   t->g64.release(); t->g32.release(); t->gdf.release(); t->h64.release();
@@ -1509,6 +1518,7 @@ dda_status dda_target_create(int nx, int ny, int nz, const uint8_t* occ, const u
     CK(cudaMemcpy(t->tw32.p, t32.data(), sizeof(float2) * t32.size(), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(t->twdf.p, tdf.data(), sizeof(float4) * tdf.size(), cudaMemcpyHostToDevice));
     kat.insert(kat.end(), posall.begin(), posall.end());
+    for (int i = 0; i < std::max({t->Lx, t->Ly, t->Lz}); ++i) kat.push_back(i);  // natural order
     t->perm.ensure(sizeof(int) * kat.size());
     CK(cudaMemcpy(t->perm.p, kat.data(), sizeof(int) * kat.size(), cudaMemcpyHostToDevice));
     t->zerr.ensure(sizeof(int));
@@ -1524,20 +1534,25 @@ dda_status dda_target_create(int nx, int ny, int nz, const uint8_t* occ, const u
       t->twzp.ensure(sizeof(float2) * tp.size());
       CK(cudaMemcpy(t->twzp.p, tp.data(), sizeof(float2) * tp.size(), cudaMemcpyHostToDevice));
     }
-    // and of the register z kernel: w_L^(j2 (2 k1 + parity)), [k1 < R1][j2 < R2],
-    // both parities side by side (re, im even; re, im odd)
-    int r1 = 0, r2 = 0;
-    if (z_reg_plan(t->Lz, t->nz, &r1, &r2)) {
-      std::vector<float4> tr;
+    // and of the register passes: w_L^(j2 (2 k1 + parity)), [k1 < R1][j2 < R2], both
+    // parities side by side (re, im even; re, im odd)
+    std::vector<float4> tr;
+    auto reg_twiddles = [&](int axis, int L, int r1, int r2) {
       const long double two_pi = 6.283185307179586476925286766559L;
+      t->twroff[axis] = (int)tr.size();
       for (int k = 0; k < r1; ++k)
         for (int j = 0; j < r2; ++j) {
-          const long double a = -two_pi * (long double)((2LL * j * k) % t->Lz) / t->Lz;
-          const long double b = -two_pi * (long double)(((2LL * k + 1) * j) % t->Lz) / t->Lz;
+          const long double a = -two_pi * (long double)((2LL * j * k) % L) / L;
+          const long double b = -two_pi * (long double)(((2LL * k + 1) * j) % L) / L;
           tr.push_back(make_float4((float)cosl(a), (float)sinl(a), (float)cosl(b), (float)sinl(b)));
         }
-      t->twzr.ensure(sizeof(float4) * tr.size());
-      CK(cudaMemcpy(t->twzr.p, tr.data(), sizeof(float4) * tr.size(), cudaMemcpyHostToDevice));
+    };
+    int r1 = 0, r2 = 0;
+    if (x_reg_plan(t->Lx, t->nx, &r1, &r2)) reg_twiddles(0, t->Lx, r1, r2);
+    if (z_reg_plan(t->Lz, t->nz, &r1, &r2)) reg_twiddles(2, t->Lz, r1, r2);
+    if (!tr.empty()) {
+      t->twr.ensure(sizeof(float4) * tr.size());
+      CK(cudaMemcpy(t->twr.p, tr.data(), sizeof(float4) * tr.size(), cudaMemcpyHostToDevice));
     }
   } catch (const CudaFail& f) {
     dda_status s = from_cuda(f);
@@ -1577,7 +1592,7 @@ int64_t dda_solve_hbm_bytes(const dda_target* t, const dda_solve_params* p) {
 // workspace and its near-field box.
 static int64_t held_bytes(dda_target* t) {
   int64_t b = 0;
-  for (const DevBuf* d : {&t->comp, &t->site, &t->tw64, &t->tw32, &t->twdf, &t->twzp, &t->twzr, &t->perm,
+  for (const DevBuf* d : {&t->comp, &t->site, &t->tw64, &t->tw32, &t->twdf, &t->twzp, &t->twr, &t->perm,
                           &t->g64, &t->g32, &t->gdf, &t->h64})
     b += (int64_t)d->bytes;
   b += t->ws.bytes();
@@ -1613,7 +1628,7 @@ int64_t dda_estimate_solve_bytes(int nx, int ny, int nz, int64_t n_dipoles, int 
   // dda_target_create: composition grid, site list, twiddles (FP64, FP32,
   // double-float, and the FP32 z kernels' own) and the frequency/position tables
   const int64_t created = nbox + 8 * n_dipoles + Lsum * (16 + 8 + 16) + 2 * Lsum * 4 +
-                          16 * (int64_t)d.Lz + 3 * 256;
+                          4 * std::max({d.Lx, d.Ly, d.Lz}) + 8 * (int64_t)d.Lz + 8 * Lsum + 3 * 256;
   return created + solve;
 }
 
@@ -2141,6 +2156,8 @@ void tune_store_locked(const std::string& key, const std::vector<int>& v) {
 template <typename T>
 void apply_schedule(const dda_target* t, MatvecLaunch& L, const std::vector<int>& v) {
   using C = cplx_t<T>;
+  const int kind = v[4] & 15;
+  L.x_reg = (v[4] & 16) != 0;
   L.x_threads = v[5];
   L.y_threads = v[6];
   L.z_threads = v[7];
@@ -2153,9 +2170,9 @@ void apply_schedule(const dda_target* t, MatvecLaunch& L, const std::vector<int>
   L.z_ps = v[3];
   // z staging 2, 3: the column-pair kernel, Ghat through L2 (2) or staged (3);
   // +4: its column tiles moved by TMA
-  // 8: the two-step register kernel
-  L.z_pair = v[4] == 8 ? 3 : v[4] >= 6 ? 2 : v[4] >= 2 ? 1 : 0;
-  L.z_gs = v[4] == 1 || v[4] == 3 || v[4] == 7;
+  // 8: the two-step register kernel; +16: the register x passes
+  L.z_pair = kind == 8 ? 3 : kind >= 6 ? 2 : kind >= 2 ? 1 : 0;
+  L.z_gs = kind == 1 || kind == 3 || kind == 7;
   const int Hz = t->Lz / 2 + 1;
   L.z_smem = (((size_t)t->Lz * L.z_ps * sizeof(C) + 15) & ~(size_t)15) +
              (L.z_gs ? (size_t)6 * Hz * L.z_tile * sizeof(C) : 0);
@@ -2163,7 +2180,8 @@ void apply_schedule(const dda_target* t, MatvecLaunch& L, const std::vector<int>
 
 std::vector<int> schedule_of(const MatvecLaunch& L) {
   return {L.x_lines, L.y_tile, L.z_tile, L.z_ps,
-          L.z_pair == 3 ? 8 : (L.z_pair ? 2 : 0) + (L.z_pair == 2 ? 4 : 0) + (L.z_gs ? 1 : 0),
+          (L.z_pair == 3 ? 8 : (L.z_pair ? 2 : 0) + (L.z_pair == 2 ? 4 : 0) + (L.z_gs ? 1 : 0)) +
+              (L.x_reg ? 16 : 0),
           L.x_threads, L.y_threads, L.z_threads};
 }
 }  // namespace
@@ -2320,13 +2338,17 @@ dda_status dda_autotune(dda_target* t, double kd, int n_rhs) {
 dda_status dda_set_schedule(dda_target* t, int precision, const int* in8) {
   g_last_error.clear();
   if (!t || !in8) return fail(DDA_ERR_INVALID_ARG, "null argument");
-  const int xl = in8[0], yt = in8[1], zt = in8[2], zp = in8[3], zg = in8[4];
+  const int xl = in8[0], yt = in8[1], zt = in8[2], zp = in8[3];
+  const int zg = in8[4] < 0 || in8[4] > 31 ? -1 : in8[4] & 15;  // z kind; +16: register x passes
   const bool f64 = precision == DDA_PREC_FP64;
   const size_t cs = f64 ? sizeof(double2) : sizeof(float2);
   if (xl < 1 || xl > 64 || yt < 1 || yt > 64 || (zt != 2 && zt != 4 && zt != 8 && zt != 16) ||
       zp < 3 * zt || zp > 3 * zt + 8 || zg < 0 || zg > 8 || zg == 4 || zg == 5)
     return fail(DDA_ERR_INVALID_ARG, "schedule: x lines 1..64, y tile 1..64, z tile 2/4/8/16, "
                                      "z pitch 3*tile..3*tile+8, z staging 0, 1, 2, 3, 6, 7 or 8");
+  if ((in8[4] & 16) && (f64 || !x_reg_plan(t->Lx, t->nx, nullptr, nullptr)))
+    return fail(DDA_ERR_INVALID_ARG, "schedule: the register x passes (z staging + 16) need FP32 "
+                                     "and an even Lx with a two-factor plan");
   if (zg == 8 && (f64 || zt != kZRegTile || !z_reg_plan(t->Lz, t->nz, nullptr, nullptr)))
     return fail(DDA_ERR_INVALID_ARG, "schedule: z staging 8 (register z kernel) needs FP32, z tile "
                                      "8 and an even Lz with a two-factor plan");

@@ -27,6 +27,8 @@ struct MatvecLaunch {
   bool z_gs;   // Ghat tile staged in shared memory
   int z_pair;  // FP32: the column-pair z kernel (k_fft_z_pairs); 2: with TMA tiles;
                // 3: the two-step register kernel (k_fft_z_reg)
+  bool x_reg;  // FP32: the x passes in two register transforms (xpass_reg.cuh), which
+               // keep their spectra in natural order (kx_at is the identity)
 };
 
 template <typename T> MatvecLaunch plan_matvec(const OpView<T>& op);
@@ -116,6 +118,9 @@ size_t zpair_smem_bytes(int Lz, int tile, bool gs);
 // the boxes of 163 to 167 planes).
 bool z_reg_plan(int Lz, int nz, int* R1, int* R2);
 constexpr int kZRegTile = 8;
+// The same for the x passes (xpass_reg.cuh), and their CTAs per right-hand side.
+bool x_reg_plan(int Lx, int nx, int* R1, int* R2);
+int x_reg_blocks(int Lx, int rows);
 // The column-pair kernel's TMA variant applies as well: nz <= 256 (a box
 // dimension), 2 nz <= Lz, and a driver that encodes tensor maps.
 bool z_pair_tma_applies(int Lz, int Lx, int nz, int tile);

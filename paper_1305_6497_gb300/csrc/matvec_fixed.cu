@@ -10,6 +10,7 @@
 #include "matvec_impl.cuh"
 #include "zpass_pair.cuh"
 #include "zpass_reg.cuh"
+#include "xpass_reg.cuh"
 
 namespace dda {
 
@@ -163,6 +164,51 @@ bool z_reg_plan(int Lz, int nz, int* R1, int* R2) {
 #undef DDA_ZREG_PLAN
   }
   return false;
+}
+
+// the register x passes, instantiated in xpass_reg_*.cu
+bool x_reg_plan(int Lx, int nx, int* R1, int* R2) {
+  if (Lx % 2) return false;
+  switch (Lx / 2) {
+#define DDA_XREG_PLAN(A, B) \
+  case (A) * (B):           \
+    if (R1) *R1 = (A);      \
+    if (R2) *R2 = (B);      \
+    return nx <= (A) * (B) && nx >= ((A) - 1) * (B);
+    DDA_XREG_ALL(DDA_XREG_PLAN)
+#undef DDA_XREG_PLAN
+  }
+  return false;
+}
+
+int x_reg_blocks(int Lx, int rows) {
+  switch (Lx / 2) {
+#define DDA_XREG_BLOCKS(A, B) \
+  case (A) * (B): return x_reg_grid(rows, XRegCfg<A, B>::LW);
+    DDA_XREG_ALL(DDA_XREG_BLOCKS)
+#undef DDA_XREG_BLOCKS
+  }
+  return 0;
+}
+
+bool launch_x_fwd_reg_any(int mode, const OpView<float>& op, int R, const float2* x, float2* buf,
+                          const int* active, XinArgs<float> xa, cudaStream_t st) {
+  if (!op.twx_reg || op.Lx % 2) return false;
+#define DDA_XREG_TRY(P) launch_x_fwd_reg_part##P(mode, op, R, x, buf, active, xa, st)
+  return DDA_XREG_TRY(0) || DDA_XREG_TRY(1) || DDA_XREG_TRY(2) || DDA_XREG_TRY(3) ||
+         DDA_XREG_TRY(4) || DDA_XREG_TRY(5) || DDA_XREG_TRY(6) || DDA_XREG_TRY(7);
+#undef DDA_XREG_TRY
+}
+
+bool launch_x_inv_reg_any(int mode, const OpView<float>& op, int R, const float2* buf,
+                          const float2* x, float2* y, const int* active, const float2* rhat,
+                          double* partials, cudaStream_t st, FoldArgs fold) {
+  if (!op.twx_reg || op.Lx % 2) return false;
+  const XInvArgs a{buf, x, y, rhat, partials, fold};
+#define DDA_XREG_TRY(P) launch_x_inv_reg_part##P(mode, op, R, a, active, st)
+  return DDA_XREG_TRY(0) || DDA_XREG_TRY(1) || DDA_XREG_TRY(2) || DDA_XREG_TRY(3) ||
+         DDA_XREG_TRY(4) || DDA_XREG_TRY(5) || DDA_XREG_TRY(6) || DDA_XREG_TRY(7);
+#undef DDA_XREG_TRY
 }
 
 static bool launch_z_reg_any(const OpView<float>& op, int R, float2* buf, const int* active,
@@ -338,6 +384,9 @@ cudaError_t configure_fixed_kernels() {
   xcfg(P16x8{}); xcfg(P16x4{}); xcfg(P16x8x4{}); xcfg(P8x4x3{});
   ok(configure_z_reg_part0()); ok(configure_z_reg_part1()); ok(configure_z_reg_part2());
   ok(configure_z_reg_part3()); ok(configure_z_reg_part4()); ok(configure_z_reg_part5());
+  ok(configure_x_reg_part0()); ok(configure_x_reg_part1()); ok(configure_x_reg_part2());
+  ok(configure_x_reg_part3()); ok(configure_x_reg_part4()); ok(configure_x_reg_part5());
+  ok(configure_x_reg_part6()); ok(configure_x_reg_part7());
   return e;
 }
 

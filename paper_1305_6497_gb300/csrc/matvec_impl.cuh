@@ -732,6 +732,13 @@ bool launch_x_inv_fixed(const OpView<float>& op, const MatvecLaunch& L, int R,
                         const float2* scratch, const float2* x, float2* y, const int* active,
                         const float2* rhat, double* partials, cudaStream_t st, FoldArgs fold);
 cudaError_t configure_fixed_kernels();
+// The register x passes (xpass_reg.cuh), by prologue / epilogue mode; false,
+// launching nothing, without a plan for the x length.
+bool launch_x_fwd_reg_any(int mode, const OpView<float>& op, int R, const float2* x, float2* buf,
+                          const int* active, XinArgs<float> xa, cudaStream_t st);
+bool launch_x_inv_reg_any(int mode, const OpView<float>& op, int R, const float2* buf,
+                          const float2* x, float2* y, const int* active, const float2* rhat,
+                          double* partials, cudaStream_t st, FoldArgs fold);
 
 // One y pass (forward: ny -> Ly rows, inverse: Ly -> ny rows) with the
 // schedule's tile (a compiled radix plan where one matches).
@@ -943,6 +950,7 @@ static void launch_x_fwd_pass(const OpView<T>& op, const MatvecLaunch& L, int R,
                               const io_t<T>* x, cplx_t<T>* scratch, const int* active,
                               XinArgs<T> xa, cudaStream_t st) {
   if constexpr (std::is_same<T, float>::value) {
+    if (L.x_reg && launch_x_fwd_reg_any(XIN, op, R, x, scratch, active, xa, st)) return;
     if (launch_x_fwd_fixed<XIN>(op, L, R, x, scratch, active, xa, st)) return;
   }
   const int rows = 3 * op.nz * op.ny;
@@ -958,6 +966,8 @@ static void launch_x_inv_pass(const OpView<T>& op, const MatvecLaunch& L, int R,
                               const int* active, const io_t<T>* rhat, double* partials,
                               cudaStream_t st, FoldArgs fold = FoldArgs()) {
   if constexpr (std::is_same<T, float>::value && XOUT != XOUT_FIELD) {
+    if (L.x_reg && launch_x_inv_reg_any(XOUT, op, R, scratch, x, y, active, rhat, partials, st, fold))
+      return;
     if (launch_x_inv_fixed<XOUT>(op, L, R, scratch, x, y, active, rhat, partials, st, fold))
       return;
   }
@@ -982,6 +992,7 @@ MatvecLaunch plan_matvec(const OpView<T>& op) {
   L.x_lines = nl;
   L.x_threads = 256;
   L.x_smem = (size_t)op.Lx * (nl + 1) * sizeof(C);
+  L.x_reg = std::is_same<T, float>::value && x_reg_plan(op.Lx, op.nx, nullptr, nullptr);
   L.xinv_smem = x_inv_smem_bytes(op.Lx, nl, op.nx, sizeof(C));  // + x, rhat, composition
   // y pass: a tile of 128 B of columns (16 FP32 / 8 FP64 complex), 256 threads
   int ty = 128 / (int)sizeof(C);
@@ -1125,6 +1136,7 @@ cudaError_t launch_field(const OpView<T>& op, const MatvecLaunch& L, int R,
 template <typename T>
 int matvec_partial_blocks(const OpView<T>& op, const MatvecLaunch& L) {
   const int rows = 3 * op.nz * op.ny;
+  if (L.x_reg) return x_reg_blocks(op.Lx, rows);
   return (rows + L.x_lines - 1) / L.x_lines;
 }
 

@@ -109,6 +109,7 @@ cudaError_t autotune_matvec(const OpView<T>& op, MatvecLaunch& L, int R, const c
       for (int th : {64, 96, 128, 192, 256}) {
         MatvecLaunch c = best;
         fill_x<T>(op, c, nl);
+        c.x_reg = false;
         c.x_threads = th;
         if (c.xinv_smem > kMax || nl > 3 * op.nz * op.ny) continue;
         const float tt = time_pass<T>(op, c, 0, R, x, y, scratch, st, e0, e1, reps, ks, part, fold) +

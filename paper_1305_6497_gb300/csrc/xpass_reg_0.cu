@@ -1,0 +1,6 @@
+// Instances of the register x passes (xpass_reg.cuh), part 0.
+#include "xpass_reg.cuh"
+
+namespace dda {
+DDA_XREG_DEFINE(0)
+}  // namespace dda

@@ -1,0 +1,6 @@
+// Instances of the register x passes (xpass_reg.cuh), part 7.
+#include "xpass_reg.cuh"
+
+namespace dda {
+DDA_XREG_DEFINE(7)
+}  // namespace dda

@@ -1,5 +1,6 @@
-"""The two-step register z kernel (z kind 8, the FP32 default): the same product
-as the general one-tile kernel and the FP64 one, at the edges of its plans."""
+"""The two-step register passes (z kind 8, + 16 for the x passes; the FP32 default):
+the same product as the general kernels and the FP64 one, at the edges of their
+plans."""
 import numpy as np
 import pytest
 
@@ -27,7 +28,7 @@ def test_register_z_kernel_matches(shape):
     t = B.Target(occ, comp, [1.5 + 0.1j], method="GKDLDR")
     kh, e = np.array([0.36, 0.48, 0.8]), [0.8, -0.6, 0]
     sch = t.schedule("fp32") if t.matvec(0.4, x, kh, e, "fp32") is not None else None
-    assert sch["z_stage_ghat"] == 8
+    assert sch["z_stage_ghat"] & 15 == 8
     y8 = t.matvec(0.4, x, kh, e, "fp32")
     y64 = t.matvec(0.4, x, kh, e, "fp64")
     t.set_schedule(dict(sch, z_tile=4, z_pitch=13, z_stage_ghat=0, z_threads=128), "fp32")
@@ -42,8 +43,47 @@ def test_register_z_kernel_matches(shape):
     ref = O.matvec_direct(x, pos, ainv, 0.4, "GKDLDR", rows=rows)
     assert np.abs(y8[rows] - ref).max() <= tol * top
     t.set_schedule(sch, "fp32")
-    assert t.schedule("fp32")["z_stage_ghat"] == 8
+    assert t.schedule("fp32")["z_stage_ghat"] & 15 == 8
     assert np.array_equal(t.matvec(0.4, x, kh, e, "fp32"), y8)
+    t.close()
+
+
+# x extents at the ends of the plans, several rows per warp, a last warp with fewer
+# rows than it holds, one composition byte per site unaligned
+X_SHAPES = [(9, 3, 2), (10, 5, 3), (11, 4, 5), (15, 7, 3), (17, 5, 4), (26, 3, 5), (28, 5, 3),
+            (33, 6, 3), (42, 3, 4), (51, 4, 3), (64, 7, 5), (73, 3, 2), (82, 5, 3), (91, 2, 5),
+            (101, 3, 4), (114, 4, 3), (126, 3, 5), (129, 5, 2), (136, 3, 3), (145, 2, 4),
+            (151, 3, 3), (161, 3, 2), (168, 2, 3), (189, 3, 3), (193, 2, 2), (204, 3, 2),
+            (217, 2, 3), (226, 3, 2), (251, 2, 3), (256, 3, 3)]
+
+
+@pytest.mark.parametrize("shape", X_SHAPES)
+def test_register_x_passes_match(shape):
+    from paper_1305_6497_gb300 import binding as B
+    w = W.two_material_brick(*shape, seed=5)
+    flat, pos = O.site_positions(w.occ)
+    x = O.box_to_sites(W.random_polarization(w.occ, 12)[0], flat)
+    kh, e = np.array([0.36, 0.48, 0.8]), [0.8, -0.6, 0]
+    t = B.Target(w.occ, w.comp, w.m, method="GKDLDR")
+    y = t.matvec(0.4, x, kh, e, "fp32")
+    s = t.schedule("fp32")
+    assert s["z_stage_ghat"] & 16
+    y64 = t.matvec(0.4, x, kh, e, "fp64")
+    tol = 6 * 9 * 2.0 ** -24
+    top = np.abs(y64).max()
+    assert np.abs(y - y64).max() <= tol * top
+    t.set_schedule(dict(s, z_stage_ghat=s["z_stage_ghat"] - 16), "fp32")
+    assert not t.schedule("fp32")["z_stage_ghat"] & 16
+    assert np.abs(t.matvec(0.4, x, kh, e, "fp32") - y).max() <= 2 * tol * top
+    # the fused prologues and epilogues of every method against the general passes
+    for solver in ("bicgstab", "qmr", "bicgstab2", "gpbicg", "petrkp"):
+        q = []
+        for z in (s["z_stage_ghat"], s["z_stage_ghat"] - 16):
+            t.set_schedule(dict(s, z_stage_ghat=z), "fp32")
+            q.append(t.solve(0.4, kh, e, npol=2, tol=1e-9, max_iter=4000, precision="fp32_refined",
+                             solver=solver))
+        assert q[0]["status"] == B.DDA_OK
+        assert np.abs(q[0]["P"] - q[1]["P"]).max() <= 1e-7 * np.abs(q[1]["P"]).max(), solver
     t.close()
 
 
@@ -56,7 +96,7 @@ def test_batches_and_frozen_right_hand_sides():
         t = B.Target(w.occ, w.comp, w.m, method="LDR")
         kw = dict(yhat=w.yhat, npol=2, tol=1e-9, precision="fp32_refined")
         a = t.solve(w.kd, w.khat, w.e01, **kw)
-        assert t.schedule("fp32")["z_stage_ghat"] == 8 and a["status"] == B.DDA_OK
+        assert t.schedule("fp32")["z_stage_ghat"] & 15 == 8 and a["status"] == B.DDA_OK
         t.set_schedule(dict(t.schedule("fp32"), z_tile=4, z_pitch=13, z_stage_ghat=0,
                             z_threads=128), "fp32")
         b = t.solve(w.kd, w.khat, w.e01, **kw)
@@ -74,7 +114,7 @@ def test_register_z_kernel_is_refused_where_it_has_no_plan():
         y = t.matvec(0.3, x, precision="fp32")
         assert np.abs(y - t.matvec(0.3, x, precision="fp64")).max() <= 4e-6 * np.abs(y).max()
         s = t.schedule("fp32")
-        assert s["z_stage_ghat"] != 8
+        assert s["z_stage_ghat"] & 15 != 8
         with pytest.raises(B.DDAError):
             t.set_schedule(dict(s, z_tile=8, z_pitch=24, z_stage_ghat=8), "fp32")
         t.close()
