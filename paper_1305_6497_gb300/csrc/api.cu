@@ -360,9 +360,9 @@ static OpView<T> make_view(const dda_target* t, const void* ghat, const void* ai
   const int* id = pm + 2 * (t->Lx + t->Ly + t->Lz);
   const bool f32 = std::is_same<T, float>::value;
   v.kx_at = f32 && t->L32.x_reg ? id : pm;
-  v.ky_at = pm + t->Lx;
+  v.ky_at = f32 && t->L32.y_reg ? id : pm + t->Lx;
   v.kz_at = pm + t->Lx + t->Ly;
-  v.ypos_at = pm + (t->Lx + t->Ly + t->Lz) + t->Lx;
+  v.ypos_at = f32 && t->L32.y_reg ? id : pm + (t->Lx + t->Ly + t->Lz) + t->Lx;
   v.twz_pair = t->twzp.as<float2>();
   const float4* tr = t->twr.as<float4>();
   v.twx_reg = t->twroff[0] < 0 ? nullptr : tr + t->twroff[0];
@@ -1364,6 +1364,7 @@ static void configure(dda_target* t) {
   t->L32 = plan_matvec<float>(v32);
   t->L64 = plan_matvec<double>(v64);
   CK(configure_matvec_kernels<float>(t->L32));
+  CK(configure_reg_kernels(t->Lx, t->Ly, t->Lz));
   CK(configure_matvec_kernels<double>(t->L64));
   CK(configure_matvec_kernels_df());
   t->kernels_configured = true;
@@ -1549,6 +1550,7 @@ dda_status dda_target_create(int nx, int ny, int nz, const uint8_t* occ, const u
     };
     int r1 = 0, r2 = 0;
     if (x_reg_plan(t->Lx, t->nx, &r1, &r2)) reg_twiddles(0, t->Lx, r1, r2);
+    if (x_reg_plan(t->Ly, t->ny, &r1, &r2)) reg_twiddles(1, t->Ly, r1, r2);
     if (z_reg_plan(t->Lz, t->nz, &r1, &r2)) reg_twiddles(2, t->Lz, r1, r2);
     if (!tr.empty()) {
       t->twr.ensure(sizeof(float4) * tr.size());
@@ -2158,6 +2160,7 @@ void apply_schedule(const dda_target* t, MatvecLaunch& L, const std::vector<int>
   using C = cplx_t<T>;
   const int kind = v[4] & 15;
   L.x_reg = (v[4] & 16) != 0;
+  L.y_reg = (v[4] & 32) != 0;
   L.x_threads = v[5];
   L.y_threads = v[6];
   L.z_threads = v[7];
@@ -2170,7 +2173,7 @@ void apply_schedule(const dda_target* t, MatvecLaunch& L, const std::vector<int>
   L.z_ps = v[3];
   // z staging 2, 3: the column-pair kernel, Ghat through L2 (2) or staged (3);
   // +4: its column tiles moved by TMA
-  // 8: the two-step register kernel; +16: the register x passes
+  // 8: the two-step register kernel; +16, +32: the register x and y passes
   L.z_pair = kind == 8 ? 3 : kind >= 6 ? 2 : kind >= 2 ? 1 : 0;
   L.z_gs = kind == 1 || kind == 3 || kind == 7;
   const int Hz = t->Lz / 2 + 1;
@@ -2181,7 +2184,7 @@ void apply_schedule(const dda_target* t, MatvecLaunch& L, const std::vector<int>
 std::vector<int> schedule_of(const MatvecLaunch& L) {
   return {L.x_lines, L.y_tile, L.z_tile, L.z_ps,
           (L.z_pair == 3 ? 8 : (L.z_pair ? 2 : 0) + (L.z_pair == 2 ? 4 : 0) + (L.z_gs ? 1 : 0)) +
-              (L.x_reg ? 16 : 0),
+              (L.x_reg ? 16 : 0) + (L.y_reg ? 32 : 0),
           L.x_threads, L.y_threads, L.z_threads};
 }
 }  // namespace
@@ -2339,7 +2342,7 @@ dda_status dda_set_schedule(dda_target* t, int precision, const int* in8) {
   g_last_error.clear();
   if (!t || !in8) return fail(DDA_ERR_INVALID_ARG, "null argument");
   const int xl = in8[0], yt = in8[1], zt = in8[2], zp = in8[3];
-  const int zg = in8[4] < 0 || in8[4] > 31 ? -1 : in8[4] & 15;  // z kind; +16: register x passes
+  const int zg = in8[4] < 0 || in8[4] > 63 ? -1 : in8[4] & 15;  // z kind; +16, +32: register x, y passes
   const bool f64 = precision == DDA_PREC_FP64;
   const size_t cs = f64 ? sizeof(double2) : sizeof(float2);
   if (xl < 1 || xl > 64 || yt < 1 || yt > 64 || (zt != 2 && zt != 4 && zt != 8 && zt != 16) ||
@@ -2349,6 +2352,9 @@ dda_status dda_set_schedule(dda_target* t, int precision, const int* in8) {
   if ((in8[4] & 16) && (f64 || !x_reg_plan(t->Lx, t->nx, nullptr, nullptr)))
     return fail(DDA_ERR_INVALID_ARG, "schedule: the register x passes (z staging + 16) need FP32 "
                                      "and an even Lx with a two-factor plan");
+  if ((in8[4] & 32) && (f64 || !x_reg_plan(t->Ly, t->ny, nullptr, nullptr)))
+    return fail(DDA_ERR_INVALID_ARG, "schedule: the register y passes (z staging + 32) need FP32 "
+                                     "and an even Ly with a two-factor plan");
   if (zg == 8 && (f64 || zt != kZRegTile || !z_reg_plan(t->Lz, t->nz, nullptr, nullptr)))
     return fail(DDA_ERR_INVALID_ARG, "schedule: z staging 8 (register z kernel) needs FP32, z tile "
                                      "8 and an even Lz with a two-factor plan");

@@ -29,6 +29,7 @@ struct MatvecLaunch {
                // 3: the two-step register kernel (k_fft_z_reg)
   bool x_reg;  // FP32: the x passes in two register transforms (xpass_reg.cuh), which
                // keep their spectra in natural order (kx_at is the identity)
+  bool y_reg;  // the same for the y passes (ypass_reg.cuh); plans as for x
 };
 
 template <typename T> MatvecLaunch plan_matvec(const OpView<T>& op);
@@ -121,6 +122,7 @@ constexpr int kZRegTile = 8;
 // The same for the x passes (xpass_reg.cuh), and their CTAs per right-hand side.
 bool x_reg_plan(int Lx, int nx, int* R1, int* R2);
 int x_reg_blocks(int Lx, int rows);
+cudaError_t configure_reg_kernels(int Lx, int Ly, int Lz);
 // The column-pair kernel's TMA variant applies as well: nz <= 256 (a box
 // dimension), 2 nz <= Lz, and a driver that encodes tensor maps.
 bool z_pair_tma_applies(int Lz, int Lx, int nz, int tile);

@@ -11,6 +11,7 @@
 #include "zpass_pair.cuh"
 #include "zpass_reg.cuh"
 #include "xpass_reg.cuh"
+#include "ypass_reg.cuh"
 
 namespace dda {
 
@@ -191,6 +192,21 @@ int x_reg_blocks(int Lx, int rows) {
   return 0;
 }
 
+// Shared-memory limits of the register passes of one target's grid.
+cudaError_t configure_reg_kernels(int Lx, int Ly, int Lz) {
+  cudaError_t e = cudaSuccess;
+  auto ok = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
+  const int hx = Lx % 2 ? 0 : Lx / 2, hy = Ly % 2 ? 0 : Ly / 2, hz = Lz % 2 ? 0 : Lz / 2;
+  ok(configure_z_reg_part0(hz)); ok(configure_z_reg_part1(hz)); ok(configure_z_reg_part2(hz));
+  ok(configure_z_reg_part3(hz)); ok(configure_z_reg_part4(hz)); ok(configure_z_reg_part5(hz));
+  ok(configure_x_reg_part0(hx)); ok(configure_x_reg_part1(hx)); ok(configure_x_reg_part2(hx));
+  ok(configure_x_reg_part3(hx)); ok(configure_x_reg_part4(hx)); ok(configure_x_reg_part5(hx));
+  ok(configure_x_reg_part6(hx)); ok(configure_x_reg_part7(hx));
+  ok(configure_y_reg_part0(hy)); ok(configure_y_reg_part1(hy)); ok(configure_y_reg_part2(hy));
+  ok(configure_y_reg_part3(hy));
+  return e;
+}
+
 bool launch_x_fwd_reg_any(int mode, const OpView<float>& op, int R, const float2* x, float2* buf,
                           const int* active, XinArgs<float> xa, cudaStream_t st) {
   if (!op.twx_reg || op.Lx % 2) return false;
@@ -275,6 +291,12 @@ bool launch_z_fixed(const OpView<float>& op, const MatvecLaunch& L, int R, float
 bool launch_y_fixed(bool inv, const OpView<float>& op, const MatvecLaunch& L, int R,
                     float2* scratch, const int* active, cudaStream_t st) {
   bool done = false;
+  // the register y passes, instantiated in ypass_reg_*.cu
+  if (L.y_reg && op.twy_reg && op.Ly % 2 == 0) {
+#define DDA_YREG_TRY(P) launch_y_reg_part##P(inv, op, R, scratch, active, st)
+    if (DDA_YREG_TRY(0) || DDA_YREG_TRY(1) || DDA_YREG_TRY(2) || DDA_YREG_TRY(3)) return true;
+#undef DDA_YREG_TRY
+  }
   dispatch_plan(op.py, YPlans{}, [&](auto plan) {
     using P = decltype(plan);
     const dim3 gy((op.Lx + L.y_tile - 1) / L.y_tile, 3 * op.nz, R);
@@ -382,11 +404,6 @@ cudaError_t configure_fixed_kernels() {
     ok(set_smem((const void*)k_fft_x_inv<float, XOUT_QT, P>));
   };
   xcfg(P16x8{}); xcfg(P16x4{}); xcfg(P16x8x4{}); xcfg(P8x4x3{});
-  ok(configure_z_reg_part0()); ok(configure_z_reg_part1()); ok(configure_z_reg_part2());
-  ok(configure_z_reg_part3()); ok(configure_z_reg_part4()); ok(configure_z_reg_part5());
-  ok(configure_x_reg_part0()); ok(configure_x_reg_part1()); ok(configure_x_reg_part2());
-  ok(configure_x_reg_part3()); ok(configure_x_reg_part4()); ok(configure_x_reg_part5());
-  ok(configure_x_reg_part6()); ok(configure_x_reg_part7());
   return e;
 }
 

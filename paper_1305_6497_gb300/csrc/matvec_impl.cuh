@@ -993,6 +993,7 @@ MatvecLaunch plan_matvec(const OpView<T>& op) {
   L.x_threads = 256;
   L.x_smem = (size_t)op.Lx * (nl + 1) * sizeof(C);
   L.x_reg = std::is_same<T, float>::value && x_reg_plan(op.Lx, op.nx, nullptr, nullptr);
+  L.y_reg = std::is_same<T, float>::value && x_reg_plan(op.Ly, op.ny, nullptr, nullptr);
   L.xinv_smem = x_inv_smem_bytes(op.Lx, nl, op.nx, sizeof(C));  // + x, rhat, composition
   // y pass: a tile of 128 B of columns (16 FP32 / 8 FP64 complex), 256 threads
   int ty = 128 / (int)sizeof(C);

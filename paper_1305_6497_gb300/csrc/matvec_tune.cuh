@@ -125,6 +125,7 @@ cudaError_t autotune_matvec(const OpView<T>& op, MatvecLaunch& L, int R, const c
       for (int th : {64, 96, 128, 192, 256}) {
         MatvecLaunch c = best;
         fill_y<T>(op, c, tile);
+        c.y_reg = false;
         c.y_threads = th;
         if (c.y_smem > kMax) continue;
         const float tt = time_pass<T>(op, c, 1, R, x, y, scratch, st, e0, e1, reps, ks, part, fold) +

@@ -13,6 +13,15 @@
 //
 // Shared memory: [row][k1][j2] 16-byte (even, odd) pairs, k1 rows an odd number of
 // pairs apart, so that step 2's half-warps (k1, parity) hit distinct banks.
+//
+// What bounds it: HBM on grids larger than L2 (256^3 box: the update of p and its
+// transform move 4.8 GB in 651 us, all of the measured copy rate), load latency on
+// smaller ones.  The kernels that keep lines in shared memory ran a third of the
+// warps, each CTA waiting for its slowest stage.  Forward / inverse pass, two
+// right-hand sides, before and now: 256^3 box 1135 / 1319 -> 651 / 1079 us, 128^3
+// 164 / 202 -> 88 / 123, 64^3 29 / 43 -> 18 / 26, 100x75x135 98 / 121 -> 48 / 85,
+// 16^3 17 / 26 -> 6.5 / 12 us.  The error of a product against 64 bits is 5.9e-8
+// where it was 5.7e-8 (RMS).
 #pragma once
 
 #include "fft_reg.cuh"
@@ -340,7 +349,7 @@ struct XInvArgs {
                                    cudaStream_t st);                                         \
   bool launch_x_inv_reg_part##PART(int mode, const OpView<float>& op, int R,                  \
                                    const XInvArgs& a, const int* active, cudaStream_t st);   \
-  cudaError_t configure_x_reg_part##PART();
+  cudaError_t configure_x_reg_part##PART(int half);
 DDA_XREG_DECLARE(0) DDA_XREG_DECLARE(1) DDA_XREG_DECLARE(2) DDA_XREG_DECLARE(3)
 DDA_XREG_DECLARE(4) DDA_XREG_DECLARE(5) DDA_XREG_DECLARE(6) DDA_XREG_DECLARE(7)
 
@@ -366,7 +375,7 @@ void x_inv_reg_mode(int mode, const OpView<float>& op, int R, const XInvArgs& a,
 }
 #define DDA_XREG_FWD(A, B) case (A) * (B): x_fwd_reg_mode<A, B>(mode, op, R, x, buf, active, xa, st); return true;
 #define DDA_XREG_INV(A, B) case (A) * (B): x_inv_reg_mode<A, B>(mode, op, R, a, active, st); return true;
-#define DDA_XREG_CONFIG(A, B) if (e == cudaSuccess) e = configure_x_reg<A, B>();
+#define DDA_XREG_CONFIG(A, B) case (A) * (B): return configure_x_reg<A, B>();
 #define DDA_XREG_DEFINE(PART)                                                                \
   bool launch_x_fwd_reg_part##PART(int mode, const OpView<float>& op, int R, const float2* x, \
                                    float2* buf, const int* active, XinArgs<float> xa,        \
@@ -379,10 +388,9 @@ void x_inv_reg_mode(int mode, const OpView<float>& op, int R, const XInvArgs& a,
     switch (op.Lx / 2) { DDA_XREG_PART##PART(DDA_XREG_INV) }                                 \
     return false;                                                                            \
   }                                                                                          \
-  cudaError_t configure_x_reg_part##PART() {                                                 \
-    cudaError_t e = cudaSuccess;                                                             \
-    DDA_XREG_PART##PART(DDA_XREG_CONFIG)                                                     \
-    return e;                                                                                \
+  cudaError_t configure_x_reg_part##PART(int half) {                                           \
+    switch (half) { DDA_XREG_PART##PART(DDA_XREG_CONFIG) }                                     \
+    return cudaSuccess;                                                                        \
   }
 
 }  // namespace dda

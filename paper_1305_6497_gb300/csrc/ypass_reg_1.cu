@@ -1,0 +1,6 @@
+// Instances of the register y passes (ypass_reg.cuh), part 1.
+#include "ypass_reg.cuh"
+
+namespace dda {
+DDA_YREG_DEFINE(1)
+}  // namespace dda

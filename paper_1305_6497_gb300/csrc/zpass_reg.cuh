@@ -308,22 +308,21 @@ void launch_z_reg(const OpView<float>& op, int R, float2* buf, const int* active
 #define DDA_ZREG_DECLARE(PART)                                                                 \
   bool launch_z_reg_part##PART(const OpView<float>& op, int R, float2* buf, const int* active, \
                                cudaStream_t st);                                               \
-  cudaError_t configure_z_reg_part##PART();
+  cudaError_t configure_z_reg_part##PART(int half);
 DDA_ZREG_DECLARE(0) DDA_ZREG_DECLARE(1) DDA_ZREG_DECLARE(2)
 DDA_ZREG_DECLARE(3) DDA_ZREG_DECLARE(4) DDA_ZREG_DECLARE(5)
 
 #define DDA_ZREG_LAUNCH(A, B) case (A) * (B): launch_z_reg<A, B>(op, R, buf, active, st); return true;
-#define DDA_ZREG_CONFIG(A, B) if (e == cudaSuccess) e = configure_z_reg<A, B>();
+#define DDA_ZREG_CONFIG(A, B) case (A) * (B): return configure_z_reg<A, B>();
 #define DDA_ZREG_DEFINE(PART)                                                                  \
   bool launch_z_reg_part##PART(const OpView<float>& op, int R, float2* buf, const int* active, \
                                cudaStream_t st) {                                              \
     switch (op.Lz / 2) { DDA_ZREG_PART##PART(DDA_ZREG_LAUNCH) }                                \
     return false;                                                                              \
   }                                                                                            \
-  cudaError_t configure_z_reg_part##PART() {                                                   \
-    cudaError_t e = cudaSuccess;                                                               \
-    DDA_ZREG_PART##PART(DDA_ZREG_CONFIG)                                                       \
-    return e;                                                                                  \
+  cudaError_t configure_z_reg_part##PART(int half) {                                           \
+    switch (half) { DDA_ZREG_PART##PART(DDA_ZREG_CONFIG) }                                     \
+    return cudaSuccess;                                                                        \
   }
 
 }  // namespace dda

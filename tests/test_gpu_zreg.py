@@ -1,4 +1,4 @@
-"""The two-step register passes (z kind 8, + 16 for the x passes; the FP32 default):
+"""The two-step register passes (z kind 8, + 16 for the x and + 32 for the y passes; the FP32 default):
 the same product as the general kernels and the FP64 one, at the edges of their
 plans."""
 import numpy as np
@@ -55,6 +55,30 @@ X_SHAPES = [(9, 3, 2), (10, 5, 3), (11, 4, 5), (15, 7, 3), (17, 5, 4), (26, 3, 5
             (101, 3, 4), (114, 4, 3), (126, 3, 5), (129, 5, 2), (136, 3, 3), (145, 2, 4),
             (151, 3, 3), (161, 3, 2), (168, 2, 3), (189, 3, 3), (193, 2, 2), (204, 3, 2),
             (217, 2, 3), (226, 3, 2), (251, 2, 3), (256, 3, 3)]
+
+
+@pytest.mark.parametrize("nx,ny", [(3, 9), (2, 10), (9, 11), (5, 16), (17, 26), (9, 33),
+                                   (4, 64), (5, 73), (9, 82), (3, 101), (17, 128), (3, 129),
+                                   (5, 136), (2, 145), (9, 150), (3, 168), (2, 189), (5, 193),
+                                   (9, 204), (2, 225), (3, 240), (9, 251), (2, 256)])
+def test_register_y_passes_match(nx, ny):
+    """Column tiles with one column, a partial tile and several tiles."""
+    from paper_1305_6497_gb300 import binding as B
+    occ, comp = tg.rect_prism(nx, ny, 4)
+    flat, pos = O.site_positions(occ)
+    x = O.box_to_sites(W.random_polarization(occ, 13)[0], flat)
+    t = B.Target(occ, comp, [1.5 + 0.1j], method="CM")
+    y = t.matvec(0.4, x, precision="fp32")
+    s = t.schedule("fp32")
+    assert s["z_stage_ghat"] & 32
+    y64 = t.matvec(0.4, x, precision="fp64")
+    tol = 6 * 9 * 2.0 ** -24
+    top = np.abs(y64).max()
+    assert np.abs(y - y64).max() <= tol * top
+    for kind in (s["z_stage_ghat"] - 32, s["z_stage_ghat"] & 15):
+        t.set_schedule(dict(s, z_stage_ghat=kind), "fp32")
+        assert np.abs(t.matvec(0.4, x, precision="fp32") - y).max() <= 2 * tol * top
+    t.close()
 
 
 @pytest.mark.parametrize("shape", X_SHAPES)
