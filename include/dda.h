@@ -431,12 +431,12 @@ int64_t dda_target_num_dipoles(const dda_target* t);
 /* Upper bound on the device bytes dda_solve(t, params) allocates on the target
  * besides its creation arrays and a Green transform it already holds: the
  * solve's workspace and, when the transform for (kd, method) is not built
- * yet, its transient build grids (admission control); -1 on bad arguments. */
+ * yet, the transform's octant (admission control); -1 on bad arguments. */
 int64_t dda_solve_hbm_bytes(const dda_target* t, const dda_solve_params* params);
 
 /* Upper bound on the device bytes a NEW target of this shape holds at the
  * peak of its first dda_solve(params): creation arrays, the kept Green
- * transform, its transient build grids and the workspace.  Host-only (no
+ * transform and the workspace (in which the transform is built).  Host-only (no
  * device work, no allocation), so a scheduler can admit a request before the
  * target exists.  method: dda_pol_method.  -1 on bad arguments. */
 int64_t dda_estimate_solve_bytes(int nx, int ny, int nz, int64_t n_dipoles, int ncomp,

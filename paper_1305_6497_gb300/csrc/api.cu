@@ -375,49 +375,31 @@ static OpView<T> make_view(const dda_target* t, const void* ghat, const void* ai
   return v;
 }
 
-// Fill a tensor on the full grid (kind: see launch_green_fill), transform it
-// (FP64, unpruned) and keep one octant in g64 (and g32 when given).
-static void build_transform(dda_target* t, double kd, int kind, DevBuf& g64, DevBuf* g32) {
-  const int64_t M = (int64_t)t->Lx * t->Ly * t->Lz;
+// Transform of G or h (kind: see launch_green_transform) into g64 (and g32, gdf
+// when given).  The transform's scratch is the FP64 spectral scratch of the
+// workspace: every matvec writes that before it reads it, and for one right-hand
+// side it is about twice as big, so a target that has solved once (a spectrum's
+// next wavelength) allocates nothing here.
+static void build_transform(dda_target* t, double kd, int kind, DevBuf& g64, DevBuf* g32,
+                            DevBuf* gdf) {
   const int64_t H = octant_size(t);
-  DevBuf full, tmp;
-  try {
-    full.ensure(sizeof(double2) * 6 * M);
-    tmp.ensure(sizeof(double2) * 6 * M);
-    g64.ensure(sizeof(double2) * 6 * H);
-    if (g32) g32->ensure(sizeof(float2) * 6 * H);
-    CK(launch_green_fill(t->nx, t->ny, t->nz, t->Lx, t->Ly, t->Lz, kd, kind,
-                         full.as<double2>(), t->stream));
-    // the full grid seen as a "box" of 2 RHS x 3 components: nothing is pruned
-    OpView<double> op = make_view<double>(t, nullptr, nullptr, t->tw64.p);
-    op.nx = t->Lx; op.ny = t->Ly; op.nz = t->Lz;
-    op.nbox = M;
-    op.comp = nullptr;
-    auto magic = [](int d) { return ((1ull << 36) + (unsigned long long)d - 1) / (unsigned long long)d; };
-    op.div_nx = magic(op.nx); op.div_ny = magic(op.ny); op.div_nz = magic(op.nz);
-    MatvecLaunch L = plan_matvec<double>(op);
-    CK(configure_matvec_kernels<double>(L));
-    CK(launch_fft3d_full(op, L, 6, full.as<double2>(), tmp.as<double2>(), t->stream));
-    const int* pos = t->perm.as<int>() + (t->Lx + t->Ly + t->Lz);
-    CK(launch_green_octant(t->Lx, t->Ly, t->Lz, pos, pos + t->Lx, pos + t->Lx + t->Ly,
-                           tmp.as<double2>(), g64.as<double2>(),
-                           g32 ? g32->as<float2>() : nullptr, t->stream));
-    CK(cudaStreamSynchronize(t->stream));
-  } catch (...) {
-    full.release();
-    tmp.release();
-    throw;
-  }
-  full.release();
-  tmp.release();
+  t->ws.scr64.ensure(green_scratch_bytes(t->nz, t->Lx, t->Ly));
+  g64.ensure(sizeof(double2) * 6 * H);
+  if (g32) g32->ensure(sizeof(float2) * 6 * H);
+  if (gdf) gdf->ensure(sizeof(df64c) * 6 * H);
+  const OpView<double> op = make_view<double>(t, nullptr, nullptr, t->tw64.p);
+  const int* pos = t->perm.as<int>() + (t->Lx + t->Ly + t->Lz);
+  CK(launch_green_transform(op, pos, pos + t->Lx, pos + t->Lx + t->Ly, kd, kind,
+                            t->ws.scr64.as<double2>(), g64.as<double2>(),
+                            g32 ? g32->as<float2>() : nullptr, gdf ? gdf->as<df64c>() : nullptr,
+                            t->stream));
+  CK(cudaStreamSynchronize(t->stream));
 }
 
 static void build_green(dda_target* t, double kd, int filtered) {
   if (t->have_green && t->green_kd == kd && t->green_filtered == filtered) return;
   t->have_green = false;
-  build_transform(t, kd, filtered, t->g64, &t->g32);
-  t->gdf.ensure(sizeof(df64c) * 6 * (size_t)octant_size(t));
-  CK(launch_split_df(6 * octant_size(t), t->g64.as<double2>(), t->gdf.as<df64c>(), t->stream));
+  build_transform(t, kd, filtered, t->g64, &t->g32, &t->gdf);
   t->have_green = true;
   t->green_kd = kd;
   t->green_filtered = filtered;
@@ -426,7 +408,7 @@ static void build_green(dda_target* t, double kd, int filtered) {
 static void build_magnetic(dda_target* t, double kd, int filtered) {
   if (t->have_h && t->h_kd == kd && t->h_filtered == filtered) return;
   t->have_h = false;
-  build_transform(t, kd, filtered | 2, t->h64, nullptr);
+  build_transform(t, kd, filtered | 2, t->h64, nullptr, nullptr);
   t->have_h = true;
   t->h_kd = kd;
   t->h_filtered = filtered;
@@ -1583,8 +1565,10 @@ int64_t dda_solve_hbm_bytes(const dda_target* t, const dda_solve_params* p) {
   b += (int64_t)nextra * 3 * t->nbox * R * (p->precision == DDA_PREC_FP64 ? 16 : 8);
   const int filtered = t->method == DDA_POL_FCD ? 1 : 0;
   if (!(t->have_green && t->green_kd == p->kd && t->green_filtered == filtered)) {
-    const int64_t M = (int64_t)t->Lx * t->Ly * t->Lz;
-    b += 2 * 6 * M * 16;                            // transient setup grids
+    // the build works in the FP64 spectral scratch, counted above (on the smallest
+    // grids it needs a little more)
+    const int64_t scr = 3 * (int64_t)t->nz * t->Ly * t->Lx * R * 16;
+    b += std::max((int64_t)0, (int64_t)green_scratch_bytes(t->nz, t->Lx, t->Ly) - scr);
     b += 6 * octant_size(t) * (16 + 8 + 16);        // the kept octant (FP64, FP32, df)
   }
   return b;
@@ -1671,10 +1655,10 @@ dda_status dda_matvec(dda_target* t, double kd, const double* khat, const double
   try {
     CK(cudaSetDevice(t->device));
     const int filtered = t->method == DDA_POL_FCD ? 1 : 0;
-    build_green(t, kd, filtered);
     const bool dfp = precision == DDA_PREC_DF64;
     const bool f32 = precision != DDA_PREC_FP64 && !dfp;
     ensure_workspace(t, 1, f32 ? DDA_PREC_FP32 : DDA_PREC_FP64, 0);
+    build_green(t, kd, filtered);
     configure(t);
     Workspace& w = t->ws;
     std::vector<double2> ai(3 * (t->ncomp + 1));
@@ -1765,13 +1749,13 @@ dda_status dda_solve(dda_target* t, const dda_solve_params* p, dda_solve_result*
     CK(cudaSetDevice(t->device));
     cudaStream_t st = t->stream;
     const int filtered = t->method == DDA_POL_FCD ? 1 : 0;
+    ensure_workspace(t, R, p->precision, p->n_dirs);
     CK(cudaEventRecord(t->ev0, st));
     build_green(t, kd, filtered);
     CK(cudaEventRecord(t->ev1, st));
     CK(cudaEventSynchronize(t->ev1));
     float setup_ms = 0.f;
     CK(cudaEventElapsedTime(&setup_ms, t->ev0, t->ev1));
-    ensure_workspace(t, R, p->precision, p->n_dirs);
     configure(t);
     Workspace& w = t->ws;
     const long long launches0 = launch_count();
@@ -2222,8 +2206,8 @@ dda_status dda_nearfield(dda_target* t, const dda_solve_params* p, const double*
     if (s != DDA_OK) return s;
     dda_target* f = t->nf;
     cudaStream_t st = f->stream;
-    build_green(f, p->kd, t->method == DDA_POL_FCD ? 1 : 0);
     ensure_workspace(f, R, DDA_PREC_FP64, 0);
+    build_green(f, p->kd, t->method == DDA_POL_FCD ? 1 : 0);
     Workspace& w = f->ws;
     const int64_t N = f->N, nb = f->nbox;
     // dipoles of the solved target, in the extended box
@@ -2297,8 +2281,8 @@ dda_status dda_autotune(dda_target* t, double kd, int n_rhs) {
   if (s != DDA_OK) return s;
   try {
     CK(cudaSetDevice(t->device));
-    build_green(t, kd, t->method == DDA_POL_FCD ? 1 : 0);
     ensure_workspace(t, n_rhs, DDA_PREC_FP32_REFINED, 0);  // FP32 and FP64 matvec buffers
+    build_green(t, kd, t->method == DDA_POL_FCD ? 1 : 0);
     Workspace& w = t->ws;
     for (int prec = 0; prec < 2; ++prec) {
       const std::string key = tune_key(t, prec, n_rhs);

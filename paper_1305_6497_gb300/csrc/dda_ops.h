@@ -64,28 +64,17 @@ cudaError_t launch_matvec_df(const OpView<df64>& op, const MatvecLaunch& L, int 
                              const double2* x, double2* y, df64c* scratch, const int* active,
                              cudaStream_t st, const cudaEvent_t* ev = nullptr);
 cudaError_t configure_matvec_kernels_df();
-// Ghat octant FP64 -> df64 (n complex values)
-cudaError_t launch_split_df(int64_t n, const double2* in, df64c* out, cudaStream_t st);
-
-// x pass forward only (box rows -> spectral rows), used by the setup transforms.
-template <typename T>
-cudaError_t launch_x_fwd(const OpView<T>& op, const MatvecLaunch& L, int R,
-                         const cplx_t<T>* x, cplx_t<T>* out, cudaStream_t st);
 
 // ---- Green tensor ----------------------------------------------------------
-// Fill the 6 components of G on the full FFT grid (FP64), parity-mirrored.
-// kind: bit 0 = filtered (FCD) scalar Green function; bit 1 = the magnetic
-// vector h (B = h x P) in components 0..2 instead of G (3..5 stay zero).
-cudaError_t launch_green_fill(int nx, int ny, int nz, int Lx, int Ly, int Lz, double kd,
-                              int kind, double2* grid6, cudaStream_t st);
-// Forward 3-D FFT of `count` full grids in place (FP64, unpruned).
-cudaError_t launch_fft3d_full(const OpView<double>& op, const MatvecLaunch& L, int count,
-                              double2* grids, double2* tmp, cudaStream_t st);
-// Copy the octant of the transformed grids (frequency k of an axis sits at
-// position pos[k]), scaled by 1/(Lx Ly Lz), to FP64 and FP32 (g32 may be null).
-cudaError_t launch_green_octant(int Lx, int Ly, int Lz, const int* posx, const int* posy,
-                                const int* posz, const double2* grid6, double2* g64,
-                                float2* g32, cudaStream_t st);
+// Transform of G for wavenumber kd on the octant, divided by Lx Ly Lz: FP64, and
+// FP32 and double-float where given (null: not written).  kind: bit 0 = filtered
+// (FCD) scalar Green function; bit 1 = the magnetic vector h (B = h x P) in
+// components 0..2 (3..5 zero) instead of G.  posx .. posz: position holding each
+// frequency; scratch: green_scratch_bytes.
+size_t green_scratch_bytes(int nz, int Lx, int Ly);
+cudaError_t launch_green_transform(const OpView<double>& op, const int* posx, const int* posy,
+                                   const int* posz, double kd, int kind, double2* scratch,
+                                   double2* g64, float2* g32, df64c* gdf, cudaStream_t st);
 
 // ---- Krylov / vector kernels -----------------------------------------------
 struct KState {

@@ -160,157 +160,179 @@ __device__ void magnetic_vector(double dx, double dy, double dz, double k, int f
   out[2] = cscale(m, dz / r);
 }
 
-// One thread per non-negative offset (dx, dy, dz) in the box; writes the up to
-// 8 mirrored grid points with the parity signs.  grid6: [6][Lz][Ly][Lx], zeroed.
-__global__ void k_green_fill(int nx, int ny, int nz, int Lx, int Ly, int Lz, double k,
-                             int filtered, double2* __restrict__ grid6) {
-  const int64_t nb = (int64_t)nx * ny * nz;
-  const int64_t M = (int64_t)Lx * Ly * Lz;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nb;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int dx = (int)(i % nx);
-    const int64_t q = i / nx;
-    const int dy = (int)(q % ny), dz = (int)(q / ny);
-    if (dx == 0 && dy == 0 && dz == 0) continue;
-    double2 g[6];
-    const bool mag = (filtered & 2) != 0;
-    if (mag) {
-      magnetic_vector((double)dx, (double)dy, (double)dz, k, filtered & 1, g);
-      g[3] = g[4] = g[5] = make_double2(0.0, 0.0);
-    } else {
-      green_tensor((double)dx, (double)dy, (double)dz, k, filtered & 1, g);
-    }
-    // parity of each component under the reflection of x, y, z: G xx..zz, or
-    // h_x, h_y, h_z (odd in their own axis) for the magnetic vector
-    const int pg[6][3] = {{0, 0, 0}, {1, 1, 0}, {1, 0, 1}, {0, 0, 0}, {0, 1, 1}, {0, 0, 0}};
-    const int ph[6][3] = {{1, 0, 0}, {0, 1, 0}, {0, 0, 1}, {0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
-    const int (*par)[3] = mag ? ph : pg;
-    for (int mz = 0; mz < 2; ++mz) {
-      if (mz && dz == 0) continue;
-      const int iz = mz ? Lz - dz : dz;
-      for (int my = 0; my < 2; ++my) {
-        if (my && dy == 0) continue;
-        const int iy = my ? Ly - dy : dy;
-        for (int mx = 0; mx < 2; ++mx) {
-          if (mx && dx == 0) continue;
-          const int ix = mx ? Lx - dx : dx;
-          const int64_t o = ((int64_t)iz * Ly + iy) * Lx + ix;
-#pragma unroll
-          for (int c = 0; c < 6; ++c) {
-            const int flips = (mx & par[c][0]) + (my & par[c][1]) + (mz & par[c][2]);
-            double2 v = g[c];
-            if (flips & 1) { v.x = -v.x; v.y = -v.y; }
-            grid6[c * M + o] = v;
-          }
-        }
-      }
-    }
-  }
+// Parity of each component under the reflection of x, y, z: G xx, xy, xz, yy, yz,
+// zz, or h_x, h_y, h_z (odd in their own axis) for the magnetic vector.
+__device__ __forceinline__ bool green_odd(bool mag, int c, int axis) {
+  if (mag) return c == axis;
+  // xy: x, y; xz: x, z; yz: y, z
+  return c == 1 ? axis != 2 : c == 2 ? axis != 1 : c == 4 ? axis != 0 : false;
 }
 
-cudaError_t launch_green_fill(int nx, int ny, int nz, int Lx, int Ly, int Lz, double kd,
-                              int filtered, double2* grid6, cudaStream_t st) {
-  const int64_t M = (int64_t)Lx * Ly * Lz;
-  cudaError_t e = cudaMemsetAsync(grid6, 0, sizeof(double2) * 6 * M, st);
-  if (e != cudaSuccess) return e;
-  const int64_t nb = (int64_t)nx * ny * nz;
-  int blocks = (int)((nb + 255) / 256);
-  if (blocks > 152 * 16) blocks = 152 * 16;
-  k_green_fill<<<blocks, 256, 0, st>>>(nx, ny, nz, Lx, Ly, Lz, kd, filtered, grid6);
-  note_launch();
-  return cudaGetLastError();
-}
+// The transform of G on the periodic grid, from the octant of offsets alone.  G is
+// even or odd in each axis, so a line of the grid is its first n values and their
+// mirror images, its transform is even or odd too, and lines that are mirror
+// images of each other need not be transformed: along x the ny nz lines of the
+// octant, along y the Hx = Lx/2 + 1 kept frequencies of nz planes, along z the
+// Hx Hy kept columns -- a quarter of the full grid's lines on each axis, and one
+// array [6][nz][Hy][Hx] instead of two of the full grid.  A mirrored line is put
+// together in shared memory and transformed like a full grid's, so the kept values
+// are those of the full transform, bit for bit.
+//
+// What bounds it: FP64 arithmetic.  Build for a new wavelength, before (two full
+// grids, allocated and freed each time) and now: 256^3 box 171 -> 41 ms,
+// 100x75x135 12.7 -> 3.0, 64^3 2.5 -> 0.59, 70x54x54 2.5 -> 0.59, 16^3 0.35 -> 0.06.
 
-// Generic strided transform (used for the unpruned setup transforms along y and z).
-// Lines are columns of a row-major plane: element (p, col) at base + p*row_stride + col.
-template <typename T, bool INV>
-__global__ void __launch_bounds__(512) k_fft_strided(cplx_t<T>* __restrict__ buf, AxisPlan P, const cplx_t<T>* tw,
-                              int64_t ncols, int64_t row_stride, int64_t plane_stride,
-                              int tile) {
-  using C = cplx_t<T>;
+// x pass: rows (y < ny, z < nz), six components a row; the tensor is evaluated
+// here.  buf [6][nz][Hy][Hx], rows y < ny.  Shared memory: L x (6 rows) lines.
+__global__ void __launch_bounds__(256)
+k_green_x(int nx, int ny, int nz, AxisPlan P, const double2* __restrict__ tw,
+          const int* __restrict__ pos, int Hx, int Hy, double k, int kind, int per,
+          double2* __restrict__ buf) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* s = reinterpret_cast<C*>(smem_raw);
-  const int64_t col0 = (int64_t)blockIdx.x * tile;
-  const int ncol = (int)min((int64_t)tile, ncols - col0);
-  C* base = buf + (int64_t)blockIdx.y * plane_stride + col0;
-  const int L = P.L;
-  for (int e = threadIdx.x; e < L * tile; e += blockDim.x) {
-    const int p = e / tile, t = e - p * tile;
-    s[p * tile + t] = t < ncol ? base[p * row_stride + t] : mk<C>(0, 0);
+  double2* s = reinterpret_cast<double2*>(smem_raw);
+  const int L = P.L, nl = 6 * per;
+  const bool mag = (kind & 2) != 0;
+  const int row0 = blockIdx.x * per, rows = ny * nz;
+  const double2 zero = make_double2(0.0, 0.0);
+  // positions nx .. L - nx hold no offset
+  for (int e = threadIdx.x; e < (L - 2 * nx + 1) * nl; e += blockDim.x) s[nx * nl + e] = zero;
+  for (int e = threadIdx.x; e < nx * per; e += blockDim.x) {
+    const int q = e / nx, dx = e - q * nx, row = row0 + q;
+    const int dz = row / ny, dy = row - dz * ny;
+    double2 g[6] = {zero, zero, zero, zero, zero, zero};
+    if (row < rows && (dx | dy | dz) != 0) {
+      if (mag) magnetic_vector((double)dx, (double)dy, (double)dz, k, kind & 1, g);
+      else green_tensor((double)dx, (double)dy, (double)dz, k, kind & 1, g);
+    }
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+      s[dx * nl + 6 * q + c] = g[c];
+      if (dx > 0)
+        s[(L - dx) * nl + 6 * q + c] =
+            green_odd(mag, c, 0) ? make_double2(-g[c].x, -g[c].y) : g[c];
+    }
   }
   __syncthreads();
-  fft_smem<C, INV>(s, tile, tile, P, tw);
-  for (int e = threadIdx.x; e < L * tile; e += blockDim.x) {
+  fft_smem<double2, false>(s, nl, nl, P, tw);
+  for (int e = threadIdx.x; e < Hx * nl; e += blockDim.x) {
+    const int line = e / Hx, h = e - line * Hx;
+    const int q = line / 6, c = line - 6 * q, row = row0 + q;
+    if (row >= rows) continue;
+    const int z = row / ny, y = row - z * ny;
+    buf[(((int64_t)c * nz + z) * Hy + y) * Hx + h] = s[pos[h] * nl + line];
+  }
+}
+
+// One line of the y or z pass in shared memory: n values and their mirror images.
+__device__ __forceinline__ void green_mirror(double2* s, int tile, int t, int p, int L, double2 v,
+                                             bool odd) {
+  s[p * tile + t] = v;
+  if (p > 0) s[(L - p) * tile + t] = odd ? make_double2(-v.x, -v.y) : v;
+}
+
+// y pass, in place: ny rows of each (component, z) plane in, Hy rows out.
+// grid: (column tiles, 6 nz)
+__global__ void __launch_bounds__(512)
+k_green_y(int ny, int nz, AxisPlan P, const double2* __restrict__ tw, const int* __restrict__ pos,
+          int Hx, int Hy, int kind, int tile, double2* __restrict__ buf) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double2* s = reinterpret_cast<double2*>(smem_raw);
+  const int L = P.L, col0 = blockIdx.x * tile, ncol = min(tile, Hx - col0);
+  const int c = blockIdx.y / nz;
+  const bool odd = green_odd((kind & 2) != 0, c, 1);
+  double2* base = buf + (int64_t)blockIdx.y * Hy * Hx + col0;
+  const double2 zero = make_double2(0.0, 0.0);
+  for (int e = threadIdx.x; e < (L - 2 * ny + 1) * tile; e += blockDim.x) s[ny * tile + e] = zero;
+  for (int e = threadIdx.x; e < ny * tile; e += blockDim.x) {
     const int p = e / tile, t = e - p * tile;
-    if (t < ncol) base[p * row_stride + t] = s[p * tile + t];
+    green_mirror(s, tile, t, p, L, t < ncol ? base[(int64_t)p * Hx + t] : zero, odd);
+  }
+  __syncthreads();
+  fft_smem<double2, false>(s, tile, tile, P, tw);
+  for (int e = threadIdx.x; e < Hy * tile; e += blockDim.x) {
+    const int h = e / tile, t = e - h * tile;
+    if (t < ncol) base[(int64_t)h * Hx + t] = s[pos[h] * tile + t];
   }
 }
 
-static cudaError_t strided_pass(double2* buf, const AxisPlan& P, const double2* tw,
-                                int64_t ncols, int64_t row_stride, int64_t plane_stride,
-                                int nplanes, cudaStream_t st) {
-  int tile = 8;
-  while (tile > 1 && (size_t)tile * P.L * sizeof(double2) > 64 * 1024) tile >>= 1;
-  int th = ((tile * P.L / 4 + 31) / 32) * 32;
-  th = th < 64 ? 64 : (th > 512 ? 512 : th);
-  const size_t smem = (size_t)tile * P.L * sizeof(double2);
-  cudaError_t e = cudaFuncSetAttribute(k_fft_strided<double, false>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
-  if (e != cudaSuccess) return e;
-  dim3 g((unsigned)((ncols + tile - 1) / tile), nplanes);
-  k_fft_strided<double, false><<<g, th, smem, st>>>(buf, P, tw, ncols, row_stride,
-                                                     plane_stride, tile);
-                                                     note_launch();
-  return cudaGetLastError();
-}
-
-// Forward unpruned 3-D transform of `count` (a multiple of 3) grids
-// [count][Lz][Ly][Lx] into tmp.  `op` describes the full grid as its box
-// (nx = Lx, ny = Ly, nz = Lz), so the x pass prunes nothing.
-cudaError_t launch_fft3d_full(const OpView<double>& op, const MatvecLaunch& L, int count,
-                              double2* grids, double2* tmp, cudaStream_t st) {
-  cudaError_t e = launch_x_fwd<double>(op, L, count / 3, grids, tmp, st);
-  if (e != cudaSuccess) return e;
-  const int64_t Lx = op.Lx, Ly = op.Ly, Lz = op.Lz;
-  // y: columns x of each (grid, z) plane
-  e = strided_pass(tmp, op.py, op.twy, Lx, Lx, Ly * Lx, (int)(count * Lz), st);
-  if (e != cudaSuccess) return e;
-  // z: columns (y, x) of each grid
-  return strided_pass(tmp, op.pz, op.twz, Ly * Lx, Ly * Lx, Lz * Ly * Lx, count, st);
-}
-
-// The forward transforms leave frequency k of each axis at position pos[k].
-__global__ void k_green_octant(int Lx, int Ly, int Lz, const int* __restrict__ posx,
-                               const int* __restrict__ posy, const int* __restrict__ posz,
-                               const double2* __restrict__ full, double2* __restrict__ g64,
-                               float2* __restrict__ g32) {
-  const int Hx = Lx / 2 + 1, Hy = Ly / 2 + 1, Hz = Lz / 2 + 1;
-  const int64_t H = (int64_t)Hx * Hy * Hz;
-  const int64_t M = (int64_t)Lx * Ly * Lz;
-  const double inv = 1.0 / (double)M;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < 6 * H;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int c = (int)(i / H);
-    const int64_t o = i - c * H;
-    const int hx = (int)(o % Hx);
-    const int64_t q = o / Hx;
-    const int hy = (int)(q % Hy), hz = (int)(q / Hy);
-    const double2 v = full[c * M + ((int64_t)posz[hz] * Ly + posy[hy]) * Lx + posx[hx]];
-    const double2 w = make_double2(v.x * inv, v.y * inv);
-    g64[6 * o + c] = w;  // the six components of a point side by side
+// z pass: nz planes in, the octant out, scaled by 1/(Lx Ly Lz): FP64, and FP32 and
+// double-float where given.  grid: (6, column tiles of Hx Hy), the components of a
+// tile neighbours, since they share the lines they are written to.
+__global__ void __launch_bounds__(512)
+k_green_z(int nz, AxisPlan P, const double2* __restrict__ tw, const int* __restrict__ pos, int Hx,
+          int Hy, int kind, int tile, int64_t first, double scale, const double2* __restrict__ buf,
+          double2* __restrict__ g64, float2* __restrict__ g32, df64c* __restrict__ gdf) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double2* s = reinterpret_cast<double2*>(smem_raw);
+  const int L = P.L, Hz = L / 2 + 1, c = blockIdx.x;
+  const int64_t plane = (int64_t)Hx * Hy, col0 = first + (int64_t)blockIdx.y * tile;
+  const int ncol = (int)min((int64_t)tile, plane - col0);
+  const bool odd = green_odd((kind & 2) != 0, c, 2);
+  const double2* base = buf + (int64_t)c * nz * plane + col0;
+  const double2 zero = make_double2(0.0, 0.0);
+  for (int e = threadIdx.x; e < (L - 2 * nz + 1) * tile; e += blockDim.x) s[nz * tile + e] = zero;
+  for (int e = threadIdx.x; e < nz * tile; e += blockDim.x) {
+    const int p = e / tile, t = e - p * tile;
+    green_mirror(s, tile, t, p, L, t < ncol ? base[p * plane + t] : zero, odd);
+  }
+  __syncthreads();
+  fft_smem<double2, false>(s, tile, tile, P, tw);
+  for (int e = threadIdx.x; e < Hz * tile; e += blockDim.x) {
+    const int hz = e / tile, t = e - hz * tile;
+    if (t >= ncol) continue;
+    const double2 v = s[pos[hz] * tile + t];
+    const double2 w = make_double2(v.x * scale, v.y * scale);
+    const int64_t col = col0 + t, o = 6 * (hz * plane + col) + c;
+    g64[o] = w;
+    if (gdf) gdf[o] = from_io<df64c>(w);
     if (g32)
-      g32[ghat_f32_offset(Hx, Hz, hz, hy, hx, c)] = make_float2((float)w.x, (float)w.y);
+      g32[ghat_f32_offset(Hx, Hz, hz, (int)(col / Hx), (int)(col % Hx), c)] =
+          make_float2((float)w.x, (float)w.y);
   }
 }
 
-cudaError_t launch_green_octant(int Lx, int Ly, int Lz, const int* posx, const int* posy,
-                                const int* posz, const double2* grid6, double2* g64,
-                                float2* g32, cudaStream_t st) {
-  const int64_t H = (int64_t)(Lx / 2 + 1) * (Ly / 2 + 1) * (Lz / 2 + 1);
-  int blocks = (int)((6 * H + 255) / 256);
-  if (blocks > 152 * 16) blocks = 152 * 16;
-  k_green_octant<<<blocks, 256, 0, st>>>(Lx, Ly, Lz, posx, posy, posz, grid6, g64, g32);
+size_t green_scratch_bytes(int nz, int Lx, int Ly) {
+  return sizeof(double2) * 6 * (size_t)nz * (Ly / 2 + 1) * (Lx / 2 + 1);
+}
+
+cudaError_t launch_green_transform(const OpView<double>& op, const int* posx, const int* posy,
+                                   const int* posz, double kd, int kind, double2* scratch,
+                                   double2* g64, float2* g32, df64c* gdf, cudaStream_t st) {
+  const int Hx = op.Lx / 2 + 1, Hy = op.Ly / 2 + 1;
+  const size_t kLimit = 200 * 1024;
+  const void* ks[] = {(const void*)k_green_x, (const void*)k_green_y, (const void*)k_green_z};
+  for (const void* k : ks) {
+    const cudaError_t e =
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLimit);
+    if (e != cudaSuccess) return e;
+  }
+  const int rows = op.ny * op.nz;
+  int per = 1;  // rows of a CTA: up to 48 KB
+  while (per < 8 && (size_t)12 * per * op.Lx * sizeof(double2) <= 48 * 1024) per *= 2;
+  k_green_x<<<(rows + per - 1) / per, 256, (size_t)6 * per * op.Lx * sizeof(double2), st>>>(
+      op.nx, op.ny, op.nz, op.px, op.twx, posx, Hx, Hy, kd, kind, per, scratch);
   note_launch();
+  auto shape = [](int L, int& tile, int& th) {
+    tile = 8;
+    while (tile > 1 && (size_t)tile * L * sizeof(double2) > 64 * 1024) tile >>= 1;
+    th = ((tile * L / 4 + 31) / 32) * 32;
+    th = th < 64 ? 64 : (th > 512 ? 512 : th);
+  };
+  int tile, th;
+  shape(op.Ly, tile, th);
+  k_green_y<<<dim3((Hx + tile - 1) / tile, 6 * op.nz), th, (size_t)tile * op.Ly * sizeof(double2), st>>>(
+      op.ny, op.nz, op.py, op.twy, posy, Hx, Hy, kind, tile, scratch);
+  note_launch();
+  shape(op.Lz, tile, th);
+  const int64_t plane = (int64_t)Hx * Hy, tiles = (plane + tile - 1) / tile;
+  // grid.y is limited to 65535 tiles a launch
+  for (int64_t t0 = 0; t0 < tiles; t0 += 65535) {
+    const int nt = (int)(tiles - t0 < 65535 ? tiles - t0 : 65535);
+    k_green_z<<<dim3(6, nt), th, (size_t)tile * op.Lz * sizeof(double2), st>>>(
+        op.nz, op.pz, op.twz, posz, Hx, Hy, kind, tile, t0 * tile,
+        1.0 / ((double)op.Lx * op.Ly * op.Lz), scratch, g64, g32, gdf);
+    note_launch();
+  }
   return cudaGetLastError();
 }
 

@@ -29,9 +29,6 @@ template cudaError_t launch_matvec<double>(const OpView<double>&, const MatvecLa
 template cudaError_t launch_field<double>(const OpView<double>&, const MatvecLaunch&, int,
                                           const double2*, double2*, double2*, cudaStream_t,
                                           bool);
-template cudaError_t launch_x_fwd<double>(const OpView<double>&, const MatvecLaunch&, int,
-                                          const double2*, double2*, cudaStream_t);
-
 template cudaError_t launch_matvec_rv<double>(const OpView<double>&, const MatvecLaunch&, int,
                                             const double2*, double2*, const double2*, double2*, double*,
                                             const int*, cudaStream_t, const cudaEvent_t*);

@@ -1183,12 +1183,4 @@ cudaError_t launch_matvec_q(const OpView<T>& op, const MatvecLaunch& L, int R,
                                           nullptr, partials, fold);
 }
 
-template <typename T>
-cudaError_t launch_x_fwd(const OpView<T>& op, const MatvecLaunch& L, int R,
-                         const cplx_t<T>* x, cplx_t<T>* out, cudaStream_t st) {
-  launch_x_fwd_pass<T, XIN_PLAIN>(op, L, R, x, out, nullptr, XinArgs<T>{}, st);
-  note_launch();
-  return cudaGetLastError();
-}
-
 }  // namespace dda
