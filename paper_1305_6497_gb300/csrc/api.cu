@@ -306,6 +306,7 @@ struct dda_target {
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   DevBuf comp, site, tw64, tw32, twdf, perm;  // perm: k_at x|y|z, then pos x|y|z
   DevBuf twzp;  // FP32 z twiddles of the column-pair kernel's plan (when it has one)
+  DevBuf tww, twd;  // z twiddles of zpass_wide.cuh, double-float and FP64 (with a plan)
   DevBuf twr;   // FP32 twiddles of the register passes, x | y | z (axes with a plan)
   int twroff[3] = {-1, -1, -1};
   DevBuf zerr;  // one int: a kernel's bounded wait on a copy ran out
@@ -368,6 +369,8 @@ static OpView<T> make_view(const dda_target* t, const void* ghat, const void* ai
   v.twx_reg = t->twroff[0] < 0 ? nullptr : tr + t->twroff[0];
   v.twy_reg = t->twroff[1] < 0 ? nullptr : tr + t->twroff[1];
   v.twz_reg = t->twroff[2] < 0 ? nullptr : tr + t->twroff[2];
+  if (std::is_same<T, df64>::value) v.tw_wide = t->tww.as<cplx_t<T>>();
+  if (std::is_same<T, double>::value) v.tw_wide = t->twd.as<cplx_t<T>>();
   v.zerr = t->zerr.as<int>();
   v.px = t->px; v.py = t->py; v.pz = t->pz;
   auto magic = [](int d) { return ((1ull << 36) + (unsigned long long)d - 1) / (unsigned long long)d; };
@@ -1348,7 +1351,7 @@ static void configure(dda_target* t) {
   CK(configure_matvec_kernels<float>(t->L32));
   CK(configure_reg_kernels(t->Lx, t->Ly, t->Lz));
   CK(configure_matvec_kernels<double>(t->L64));
-  CK(configure_matvec_kernels_df());
+  CK(configure_matvec_kernels_df(t->Lz));
   t->kernels_configured = true;
 }
 
@@ -1392,6 +1395,8 @@ void dda_target_destroy(dda_target* t) {
   t->comp.release(); t->site.release(); t->tw64.release(); t->tw32.release(); t->twdf.release();
   t->twzp.release();
   t->twr.release();
+  t->tww.release();
+  t->twd.release();
   t->zerr.release();
   t->perm.release();
   t->g64.release(); t->g32.release(); t->gdf.release(); t->h64.release();
@@ -1538,6 +1543,26 @@ dda_status dda_target_create(int nx, int ny, int nz, const uint8_t* occ, const u
       t->twr.ensure(sizeof(float4) * tr.size());
       CK(cudaMemcpy(t->twr.p, tr.data(), sizeof(float4) * tr.size(), cudaMemcpyHostToDevice));
     }
+    // [parity][k1][j2] in double-float (the refinement's residual passes) and FP64
+    if (z_wide_plan(t->Lz, t->nz, &r1, &r2)) {
+      std::vector<float4> td;
+      std::vector<double2> tq;
+      const long double two_pi = 6.283185307179586476925286766559L;
+      for (int p = 0; p < 2; ++p)
+        for (int k = 0; k < r1; ++k)
+          for (int j = 0; j < r2; ++j) {
+            const long double a = -two_pi * (long double)(((2LL * k + p) * j) % t->Lz) / t->Lz;
+            const long double re = cosl(a), im = sinl(a);
+            const float rh = (float)re, ih = (float)im;
+            td.push_back(make_float4(rh, (float)(re - (long double)rh), ih,
+                                     (float)(im - (long double)ih)));
+            tq.push_back(make_double2((double)re, (double)im));
+          }
+      t->twd.ensure(sizeof(double2) * tq.size());
+      CK(cudaMemcpy(t->twd.p, tq.data(), sizeof(double2) * tq.size(), cudaMemcpyHostToDevice));
+      t->tww.ensure(sizeof(float4) * td.size());
+      CK(cudaMemcpy(t->tww.p, td.data(), sizeof(float4) * td.size(), cudaMemcpyHostToDevice));
+    }
   } catch (const CudaFail& f) {
     dda_status s = from_cuda(f);
     dda_target_destroy(t);
@@ -1578,7 +1603,7 @@ int64_t dda_solve_hbm_bytes(const dda_target* t, const dda_solve_params* p) {
 // workspace and its near-field box.
 static int64_t held_bytes(dda_target* t) {
   int64_t b = 0;
-  for (const DevBuf* d : {&t->comp, &t->site, &t->tw64, &t->tw32, &t->twdf, &t->twzp, &t->twr, &t->perm,
+  for (const DevBuf* d : {&t->comp, &t->site, &t->tw64, &t->tw32, &t->twdf, &t->twzp, &t->twr, &t->tww, &t->twd, &t->perm,
                           &t->g64, &t->g32, &t->gdf, &t->h64})
     b += (int64_t)d->bytes;
   b += t->ws.bytes();
@@ -1614,7 +1639,7 @@ int64_t dda_estimate_solve_bytes(int nx, int ny, int nz, int64_t n_dipoles, int 
   // dda_target_create: composition grid, site list, twiddles (FP64, FP32,
   // double-float, and the FP32 z kernels' own) and the frequency/position tables
   const int64_t created = nbox + 8 * n_dipoles + Lsum * (16 + 8 + 16) + 2 * Lsum * 4 +
-                          4 * std::max({d.Lx, d.Ly, d.Lz}) + 8 * (int64_t)d.Lz + 8 * Lsum + 3 * 256;
+                          4 * std::max({d.Lx, d.Ly, d.Lz}) + 40 * (int64_t)d.Lz + 8 * Lsum + 3 * 256;
   return created + solve;
 }
 
@@ -2339,9 +2364,10 @@ dda_status dda_set_schedule(dda_target* t, int precision, const int* in8) {
   if ((in8[4] & 32) && (f64 || !x_reg_plan(t->Ly, t->ny, nullptr, nullptr)))
     return fail(DDA_ERR_INVALID_ARG, "schedule: the register y passes (z staging + 32) need FP32 "
                                      "and an even Ly with a two-factor plan");
-  if (zg == 8 && (f64 || zt != kZRegTile || !z_reg_plan(t->Lz, t->nz, nullptr, nullptr)))
-    return fail(DDA_ERR_INVALID_ARG, "schedule: z staging 8 (register z kernel) needs FP32, z tile "
-                                     "8 and an even Lz with a two-factor plan");
+  if (zg == 8 && (f64 ? zt != 4 || !z_wide_plan(t->Lz, t->nz, nullptr, nullptr)
+                      : zt != kZRegTile || !z_reg_plan(t->Lz, t->nz, nullptr, nullptr)))
+    return fail(DDA_ERR_INVALID_ARG, "schedule: z staging 8 (register z kernel) needs z tile 8 "
+                                     "(FP64: 4) and an even Lz with a two-factor plan");
   if (zg >= 2 && zg != 8 && (f64 || !z_pair_applies(t->Lz, t->Lx, zt) || in8[7] != kZPairThreads))
     return fail(DDA_ERR_INVALID_ARG, "schedule: z staging 2/3/6/7 (column-pair z kernel) needs "
                                      "FP32, an even Lx, Lz of 64, 128, 288 or 512, tile 4 or 8 "

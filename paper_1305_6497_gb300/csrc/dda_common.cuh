@@ -179,6 +179,7 @@ template <typename T> struct OpView {
   const float4* twz_reg;          // z twiddles of the register kernel (FP32), or null
   const float4* twx_reg;          // x, y twiddles of the register passes (FP32), or null
   const float4* twy_reg;
+  const C* tw_wide;               // z twiddles of the 16-byte register kernel, or null
   const float2* twz_pair;         // z twiddles of the column-pair kernel's plan (FP32), or null
   int* zerr;                      // set to 1 by a kernel whose bounded wait on a copy ran out
   unsigned long long div_nx, div_ny, div_nz, div_Lx;     // fast_div magics

@@ -26,7 +26,7 @@ struct MatvecLaunch {
   int z_tile, z_ps, z_threads; size_t z_smem;
   bool z_gs;   // Ghat tile staged in shared memory
   int z_pair;  // FP32: the column-pair z kernel (k_fft_z_pairs); 2: with TMA tiles;
-               // 3: the two-step register kernel (k_fft_z_reg)
+               // 3: the two-step register kernel (k_fft_z_reg; FP64: k_fft_z_wide)
   bool x_reg;  // FP32: the x passes in two register transforms (xpass_reg.cuh), which
                // keep their spectra in natural order (kx_at is the identity)
   bool y_reg;  // the same for the y passes (ypass_reg.cuh); plans as for x
@@ -63,7 +63,10 @@ cudaError_t launch_field(const OpView<T>& op, const MatvecLaunch& L, int R,
 cudaError_t launch_matvec_df(const OpView<df64>& op, const MatvecLaunch& L, int R,
                              const double2* x, double2* y, df64c* scratch, const int* active,
                              cudaStream_t st, const cudaEvent_t* ev = nullptr);
-cudaError_t configure_matvec_kernels_df();
+cudaError_t configure_matvec_kernels_df(int Lz);
+// The register z kernel of the FP64 and double-float passes (zpass_wide.cuh) covers z length
+// Lz of a box of nz planes (as z_reg_plan).
+bool z_wide_plan(int Lz, int nz, int* R1, int* R2);
 
 // ---- Green tensor ----------------------------------------------------------
 // Transform of G for wavenumber kd on the octant, divided by Lx Ly Lz: FP64, and

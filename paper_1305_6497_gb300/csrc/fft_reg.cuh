@@ -1,6 +1,6 @@
 // DFTs of up to 20 points in registers, on scalar values or on packed pairs.
 //
-// The element type V is float, double, or f32p: two FP32 numbers in one 64-bit
+// The element type V is float, double, double-float, or f32p: two FP32 numbers in one 64-bit
 // register pair, worked on by the packed instructions {add,sub,mul,fma}.rn.f32x2.
 // On this part a packed instruction occupies the FP32 pipe as long as two scalar
 // ones (60 lanes per clock and SM measured, against 118), but takes one issue slot
@@ -47,6 +47,21 @@ __device__ __forceinline__ f32p vfma(f32p a, f32p b, f32p c) {
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
   return r;
 }
+__device__ __forceinline__ df64 vadd(df64 a, df64 b) { return a + b; }
+__device__ __forceinline__ df64 vsub(df64 a, df64 b) { return a - b; }
+__device__ __forceinline__ df64 vmul(df64 a, df64 b) { return a * b; }
+// a b + c with one renormalisation: the product's leading part, its error (exact by
+// FMA) and the low-order terms; 15 instructions against 18 of a product and a sum
+__device__ __forceinline__ df64 vfma(df64 a, df64 b, df64 c) {
+  const float p = __fmul_rn(a.hi, b.hi);
+  float e = __fmaf_rn(a.hi, b.hi, -p);
+  e = __fmaf_rn(a.hi, b.lo, e);
+  e = __fmaf_rn(a.lo, b.hi, e);
+  const float s = __fadd_rn(p, c.hi), bb = __fsub_rn(s, p);
+  const float r = __fadd_rn(__fsub_rn(p, __fsub_rn(s, bb)), __fsub_rn(c.hi, bb));
+  return df_fast2sum(s, __fadd_rn(r, __fadd_rn(e, c.lo)));
+}
+__device__ __forceinline__ df64 vneg(df64 a) { return -a; }
 __device__ __forceinline__ float vadd(float a, float b) { return a + b; }
 __device__ __forceinline__ float vsub(float a, float b) { return a - b; }
 __device__ __forceinline__ float vmul(float a, float b) { return a * b; }
@@ -57,8 +72,17 @@ __device__ __forceinline__ double vmul(double a, double b) { return a * b; }
 __device__ __forceinline__ double vfma(double a, double b, double c) { return fma(a, b, c); }
 
 template <typename V> __device__ __forceinline__ V vconst(double c) { return (V)c; }
+template <> __device__ __forceinline__ df64 vconst<df64>(double c) { return df64(c); }
 template <> __device__ __forceinline__ f32p vconst<f32p>(double c) {
   return pk_make((float)c, (float)c);
+}
+
+// c - a / 2 (exact scaling)
+__device__ __forceinline__ f32p vsub_half(f32p c, f32p a) { return vfma(vconst<f32p>(-0.5), a, c); }
+__device__ __forceinline__ float vsub_half(float c, float a) { return fmaf(-0.5f, a, c); }
+__device__ __forceinline__ double vsub_half(double c, double a) { return fma(-0.5, a, c); }
+__device__ __forceinline__ df64 vsub_half(df64 c, df64 a) {
+  return c + df64(-0.5f * a.hi, -0.5f * a.lo);
 }
 
 template <typename V> struct cv { V re, im; };
@@ -83,6 +107,26 @@ template <typename V> __device__ __forceinline__ cv<V> cvmul(cv<V> a, cv<V> b) {
 template <typename V> __device__ __forceinline__ cv<V> cvmulc(cv<V> a, cv<V> b) {
   return {vfma(a.re, b.re, vmul(a.im, b.im)), vfma(a.re, b.im, vmul(vneg(a.im), b.re))};
 }
+// Double-float products: both products of a part are split exactly, their leading
+// parts added with the sum's error, everything else in one low-order sum -- 19
+// instructions a part where two products and a sum take 25, and one rounding less.
+__device__ __forceinline__ df64 df_dot2(df64 a, df64 b, df64 c, df64 d) {  // a b + c d
+  const float p = __fmul_rn(a.hi, b.hi), q = __fmul_rn(c.hi, d.hi);
+  float e = __fadd_rn(__fmaf_rn(a.hi, b.hi, -p), __fmaf_rn(c.hi, d.hi, -q));
+  e = __fmaf_rn(a.hi, b.lo, e);
+  e = __fmaf_rn(a.lo, b.hi, e);
+  e = __fmaf_rn(c.hi, d.lo, e);
+  e = __fmaf_rn(c.lo, d.hi, e);
+  const float s = __fadd_rn(p, q), bb = __fsub_rn(s, p);
+  const float r = __fadd_rn(__fsub_rn(p, __fsub_rn(s, bb)), __fsub_rn(q, bb));
+  return df_fast2sum(s, __fadd_rn(r, e));
+}
+template <> __device__ __forceinline__ cv<df64> cvmul(cv<df64> a, cv<df64> b) {
+  return {df_dot2(a.re, b.re, vneg(a.im), b.im), df_dot2(a.re, b.im, a.im, b.re)};
+}
+template <> __device__ __forceinline__ cv<df64> cvmulc(cv<df64> a, cv<df64> b) {
+  return {df_dot2(a.re, b.re, a.im, b.im), df_dot2(a.re, b.im, vneg(a.im), b.re)};
+}
 // a b + c
 template <typename V> __device__ __forceinline__ cv<V> cvmad(cv<V> a, cv<V> b, cv<V> c) {
   return {vfma(vneg(a.im), b.im, vfma(a.re, b.re, c.re)), vfma(a.re, b.im, vfma(a.im, b.re, c.im))};
@@ -94,6 +138,10 @@ __device__ __forceinline__ cv<V> cvrot(cv<V> a, double c, double s) {
   return {vfma(cc, a.re, vmul(sp, a.im)), vfma(cc, a.im, vmul(sn, a.re))};
 }
 
+template <bool INV> __device__ __forceinline__ cv<df64> cvrot(cv<df64> a, double c, double s) {
+  const df64 cc(c), sp(INV ? -s : s), sn(INV ? s : -s);
+  return {df_dot2(cc, a.re, sp, a.im), df_dot2(cc, a.im, sn, a.re)};
+}
 // On packed pairs the rotations by constants run on the two halves: a scalar
 // multiply takes its constant as an immediate, a packed one needs it twice in a
 // register pair, which costs more moves than the packing saves issue slots.
@@ -158,10 +206,10 @@ __device__ __forceinline__ void rdft4(cv<V>& a0, cv<V>& a1, cv<V>& a2, cv<V>& a3
 }
 template <bool INV, typename V>
 __device__ __forceinline__ void rdft3(cv<V>& a0, cv<V>& a1, cv<V>& a2) {
-  const V mh = vconst<V>(-0.5), s = vconst<V>(INV ? -cx_sin(1, 3) : cx_sin(1, 3)),
+  const V s = vconst<V>(INV ? -cx_sin(1, 3) : cx_sin(1, 3)),
           sn = vconst<V>(INV ? cx_sin(1, 3) : -cx_sin(1, 3));
   const cv<V> t = cvadd(a1, a2), d = cvsub(a1, a2);
-  const cv<V> u{vfma(mh, t.re, a0.re), vfma(mh, t.im, a0.im)};
+  const cv<V> u{vsub_half(a0.re, t.re), vsub_half(a0.im, t.im)};
   a0 = cvadd(a0, t);
   a1 = {vfma(s, d.im, u.re), vfma(sn, d.re, u.im)};  // u - i s d
   a2 = {vfma(sn, d.im, u.re), vfma(s, d.re, u.im)};  // u + i s d
@@ -228,8 +276,8 @@ __device__ __forceinline__ void rdft_ct(cv<V> (&a)[A * B]) {
         a[B * ka + jb] = t[ka];
       } else if constexpr (4 * num == A * B) {
         // -i (forward), +i (inverse)
-        if (INV) a[B * ka + jb] = {vsub(vconst<V>(0.0), t[ka].im), t[ka].re};
-        else a[B * ka + jb] = {t[ka].im, vsub(vconst<V>(0.0), t[ka].re)};
+        if (INV) a[B * ka + jb] = {vneg(t[ka].im), t[ka].re};
+        else a[B * ka + jb] = {t[ka].im, vneg(t[ka].re)};
       } else {
         constexpr double c = cx_cos(num, A * B), s = cx_sin(num, A * B);
         a[B * ka + jb] = cvrot<INV>(t[ka], c, s);

@@ -19,6 +19,7 @@
 // the three compile in parallel.
 #pragma once
 
+#include <algorithm>
 #include <type_traits>
 
 #include "dda_ops.h"
@@ -740,6 +741,12 @@ bool launch_x_inv_reg_any(int mode, const OpView<float>& op, int R, const float2
                           const float2* x, float2* y, const int* active, const float2* rhat,
                           double* partials, cudaStream_t st, FoldArgs fold);
 
+// The register z pass on FP64 and double-float values (zpass_wide.cuh); false,
+// launching nothing, without a plan for the z length.
+template <typename T>
+bool launch_z_wide_any(bool cross, const OpView<T>& op, int R, cplx_t<T>* buf, const int* active,
+                       cudaStream_t st);
+
 // One y pass (forward: ny -> Ly rows, inverse: Ly -> ny rows) with the
 // schedule's tile (a compiled radix plan where one matches).
 template <typename T, bool INV>
@@ -757,7 +764,8 @@ template <typename T, bool CROSS>
 static void launch_z_pass(const OpView<T>& op, const MatvecLaunch& L, int R,
                           cplx_t<T>* scratch, const int* active, cudaStream_t st) {
   if constexpr (std::is_same<T, df64>::value) {
-    // double-float passes use one z variant (4 columns, Ghat from global
+    if (!CROSS && launch_z_wide_any<df64>(false, op, R, scratch, active, st)) return;
+    // lengths without a plan have one variant (4 columns, Ghat from global
     // memory): the arithmetic is ~10x the FP32 code, so fewer instantiations
     // keep the build short
     dim3 gz((op.Lx + 3) / 4, op.Ly, R);
@@ -765,6 +773,9 @@ static void launch_z_pass(const OpView<T>& op, const MatvecLaunch& L, int R,
                                                                       active);
   } else {
     dim3 gz((op.Lx + L.z_tile - 1) / L.z_tile, op.Ly, R);
+    if constexpr (std::is_same<T, double>::value) {
+      if (L.z_pair == 3 && launch_z_wide_any<double>(CROSS, op, R, scratch, active, st)) return;
+    }
     if constexpr (std::is_same<T, float>::value && !CROSS) {
       if (launch_z_fixed(op, L, R, scratch, active, st)) return;
     }
@@ -989,8 +1000,12 @@ MatvecLaunch plan_matvec(const OpView<T>& op) {
   int nl = 16;
   while (nl > 1 && (size_t)nl * (op.Lx + 1) * sizeof(C) > 36 * 1024) nl >>= 1;
   while (nl < 64 && (size_t)(2 * nl) * (op.Lx + 1) * sizeof(C) <= 36 * 1024) nl <<= 1;
+  // small grids: fewer lines per CTA (at least 4) until two CTAs per SM have some, and
+  // no more threads than the lines have 8-point butterflies
+  const int rows = 3 * op.nz * op.ny;
+  while (nl > 4 && rows / nl < 304) nl >>= 1;
   L.x_lines = nl;
-  L.x_threads = 256;
+  L.x_threads = std::min(256, std::max(64, (nl * op.Lx / 8 + 31) / 32 * 32));
   L.x_smem = (size_t)op.Lx * (nl + 1) * sizeof(C);
   L.x_reg = std::is_same<T, float>::value && x_reg_plan(op.Lx, op.nx, nullptr, nullptr);
   L.y_reg = std::is_same<T, float>::value && x_reg_plan(op.Ly, op.ny, nullptr, nullptr);
@@ -1020,6 +1035,19 @@ MatvecLaunch plan_matvec(const OpView<T>& op) {
     L.z_tile = kZRegTile;
     L.z_ps = 3 * kZRegTile;
     L.z_threads = 256;
+    return L;
+  }
+  // FP64, bound by FP64 arithmetic: the register kernel (zpass_wide.cuh) for short
+  // lines, where the one-tile kernel's stages have too few butterflies to fill warps
+  // (16^3 box 44 us against 28, 33x29x24 216 against 139, 32^3 214 against 174); from
+  // 48 on the two are level (48^3 623 against 629, 64^3 1375 against 1379) and at 128
+  // the one-tile kernel leads (3010 against 3180)
+  if (std::is_same<T, double>::value && op.Lz <= 80 &&
+      z_wide_plan(op.Lz, op.nz, nullptr, nullptr)) {
+    L.z_pair = 3;
+    L.z_tile = 4;
+    L.z_ps = 12;
+    L.z_threads = 192;
     return L;
   }
   int tz = tz_min;
