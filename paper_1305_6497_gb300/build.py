@@ -21,7 +21,7 @@ INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 SOURCES = ["api.cu", "matvec_f32.cu", "matvec_f64.cu", "matvec_df.cu", "krylov.cu",
            "bicgstab2.cu", "gpbicg.cu", "green.cu", "observables.cu", "scattering.cu",
            "matvec_fixed.cu"] + \
-          [f"zpass_reg_{k}.cu" for k in range(6)] + [f"xpass_reg_{k}.cu" for k in range(8)] + \
+          [f"zpass_reg_{k}.cu" for k in range(6)] + [f"xpass_reg_{k}.cu" for k in range(9)] + \
           [f"ypass_reg_{k}.cu" for k in range(4)] + [f"zpass_wide_{k}.cu" for k in range(6)]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "--expt-relaxed-constexpr",

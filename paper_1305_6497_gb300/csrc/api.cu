@@ -1522,15 +1522,16 @@ dda_status dda_target_create(int nx, int ny, int nz, const uint8_t* occ, const u
       t->twzp.ensure(sizeof(float2) * tp.size());
       CK(cudaMemcpy(t->twzp.p, tp.data(), sizeof(float2) * tp.size(), cudaMemcpyHostToDevice));
     }
-    // and of the register passes: w_L^(j2 (2 k1 + parity)), [k1 < R1][j2 < R2], both
-    // parities side by side (re, im even; re, im odd)
+    // and of the register passes, [k1 < R1][j2 < R2]: w_L^(j2 (2 k1 + parity)), both
+    // parities side by side (re, im even; re, im odd), or w_L^(j2 k1) for odd L
     std::vector<float4> tr;
     auto reg_twiddles = [&](int axis, int L, int r1, int r2) {
       const long double two_pi = 6.283185307179586476925286766559L;
       t->twroff[axis] = (int)tr.size();
       for (int k = 0; k < r1; ++k)
         for (int j = 0; j < r2; ++j) {
-          const long double a = -two_pi * (long double)((2LL * j * k) % L) / L;
+          const long long even = L % 2 ? (long long)j * k : 2LL * j * k;
+          const long double a = -two_pi * (long double)(even % L) / L;
           const long double b = -two_pi * (long double)(((2LL * k + 1) * j) % L) / L;
           tr.push_back(make_float4((float)cosl(a), (float)sinl(a), (float)cosl(b), (float)sinl(b)));
         }
@@ -2360,14 +2361,14 @@ dda_status dda_set_schedule(dda_target* t, int precision, const int* in8) {
                                      "z pitch 3*tile..3*tile+8, z staging 0, 1, 2, 3, 6, 7 or 8");
   if ((in8[4] & 16) && (f64 || !x_reg_plan(t->Lx, t->nx, nullptr, nullptr)))
     return fail(DDA_ERR_INVALID_ARG, "schedule: the register x passes (z staging + 16) need FP32 "
-                                     "and an even Lx with a two-factor plan");
+                                     "and an Lx with a two-factor plan");
   if ((in8[4] & 32) && (f64 || !x_reg_plan(t->Ly, t->ny, nullptr, nullptr)))
     return fail(DDA_ERR_INVALID_ARG, "schedule: the register y passes (z staging + 32) need FP32 "
-                                     "and an even Ly with a two-factor plan");
+                                     "and an Ly with a two-factor plan");
   if (zg == 8 && (f64 ? zt != 4 || !z_wide_plan(t->Lz, t->nz, nullptr, nullptr)
                       : zt != kZRegTile || !z_reg_plan(t->Lz, t->nz, nullptr, nullptr)))
     return fail(DDA_ERR_INVALID_ARG, "schedule: z staging 8 (register z kernel) needs z tile 8 "
-                                     "(FP64: 4) and an even Lz with a two-factor plan");
+                                     "(FP64: 4) and an Lz with a two-factor plan");
   if (zg >= 2 && zg != 8 && (f64 || !z_pair_applies(t->Lz, t->Lx, zt) || in8[7] != kZPairThreads))
     return fail(DDA_ERR_INVALID_ARG, "schedule: z staging 2/3/6/7 (column-pair z kernel) needs "
                                      "FP32, an even Lx, Lz of 64, 128, 288 or 512, tile 4 or 8 "

@@ -105,10 +105,10 @@ constexpr int kZPairThreads = 384;
 // Dynamic shared memory of the column-pair z kernel (with the Ghat tile if gs).
 size_t zpair_smem_bytes(int Lz, int tile, bool gs);
 // The two-step register z kernel (FP32, zpass_reg.cuh) covers z length Lz of a box
-// of nz planes: Lz even, Lz / 2 = R1 R2 in its list of plans (R1, R2 returned
-// unless null) and (R1 - 1) R2 <= nz <= Lz / 2, so that only the last of a thread's
-// R1 rows can lie beyond the box (of the smooth lengths up to 512 this leaves out
-// the boxes of 163 to 167 planes).
+// of nz planes: Lz / 2 = R1 R2 for even Lz, Lz = R1 R2 for odd, in the list of plans
+// (R1, R2 returned unless null), and nz such that only the last of a thread's rows can
+// lie beyond the box (of the even lengths up to 512 that leaves out the boxes of 163
+// to 167 planes).
 bool z_reg_plan(int Lz, int nz, int* R1, int* R2);
 constexpr int kZRegTile = 8;
 // The same for the x passes (xpass_reg.cuh), and their CTAs per right-hand side.

@@ -153,41 +153,38 @@ bool encode_zpair_map(CUtensorMap* map, const float2* scratch, int Lx, int Ly, i
 }
 
 // the two-step register kernel, instantiated in zpass_reg_*.cu
-bool z_reg_plan(int Lz, int nz, int* R1, int* R2) {
-  if (Lz % 2) return false;
-  switch (Lz / 2) {
-#define DDA_ZREG_PLAN(A, B) \
-  case (A) * (B):           \
-    if (R1) *R1 = (A);      \
-    if (R2) *R2 = (B);      \
-    return nz <= (A) * (B) && nz >= ((A) - 1) * (B);
-    DDA_ZREG_ALL(DDA_ZREG_PLAN)
-#undef DDA_ZREG_PLAN
-  }
+// (odd lengths: (NJ - 1) R2 <= nz <= (Lz + 1) / 2)
+#define DDA_REG_PLAN_ODD(A, B)                                                  \
+  case (A) * (B):                                                               \
+    if (R1) *R1 = (A);                                                          \
+    if (R2) *R2 = (B);                                                          \
+    return n <= ((A) * (B) + 1) / 2 && n >= (XRegCfg<A, B, false>::NJ - 1) * (B);
+#define DDA_REG_PLAN(A, B) \
+  case 2 * (A) * (B):      \
+    if (R1) *R1 = (A);     \
+    if (R2) *R2 = (B);     \
+    return n <= (A) * (B) && n >= ((A) - 1) * (B);
+
+bool z_reg_plan(int Lz, int n, int* R1, int* R2) {
+  switch (Lz) { DDA_ZREG_ALL(DDA_REG_PLAN) DDA_XREG_ODD(DDA_REG_PLAN_ODD) }
   return false;
 }
 
 // the register x passes, instantiated in xpass_reg_*.cu
-bool x_reg_plan(int Lx, int nx, int* R1, int* R2) {
-  if (Lx % 2) return false;
-  switch (Lx / 2) {
-#define DDA_XREG_PLAN(A, B) \
-  case (A) * (B):           \
-    if (R1) *R1 = (A);      \
-    if (R2) *R2 = (B);      \
-    return nx <= (A) * (B) && nx >= ((A) - 1) * (B);
-    DDA_XREG_ALL(DDA_XREG_PLAN)
-#undef DDA_XREG_PLAN
-  }
+bool x_reg_plan(int Lx, int n, int* R1, int* R2) {
+  switch (Lx) { DDA_XREG_ALL(DDA_REG_PLAN) DDA_XREG_ODD(DDA_REG_PLAN_ODD) }
   return false;
 }
 
 int x_reg_blocks(int Lx, int rows) {
-  switch (Lx / 2) {
+  switch (Lx) {
 #define DDA_XREG_BLOCKS(A, B) \
-  case (A) * (B): return x_reg_grid(rows, XRegCfg<A, B>::LW);
-    DDA_XREG_ALL(DDA_XREG_BLOCKS)
+  case 2 * (A) * (B): return x_reg_grid(rows, XRegCfg<A, B, true>::LW);
+#define DDA_XREG_BLOCKS_ODD(A, B) \
+  case (A) * (B): return x_reg_grid(rows, XRegCfg<A, B, false>::LW);
+    DDA_XREG_ALL(DDA_XREG_BLOCKS) DDA_XREG_ODD(DDA_XREG_BLOCKS_ODD)
 #undef DDA_XREG_BLOCKS
+#undef DDA_XREG_BLOCKS_ODD
   }
   return 0;
 }
@@ -196,34 +193,35 @@ int x_reg_blocks(int Lx, int rows) {
 cudaError_t configure_reg_kernels(int Lx, int Ly, int Lz) {
   cudaError_t e = cudaSuccess;
   auto ok = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
-  const int hx = Lx % 2 ? 0 : Lx / 2, hy = Ly % 2 ? 0 : Ly / 2, hz = Lz % 2 ? 0 : Lz / 2;
-  ok(configure_z_reg_part0(hz)); ok(configure_z_reg_part1(hz)); ok(configure_z_reg_part2(hz));
-  ok(configure_z_reg_part3(hz)); ok(configure_z_reg_part4(hz)); ok(configure_z_reg_part5(hz));
-  ok(configure_x_reg_part0(hx)); ok(configure_x_reg_part1(hx)); ok(configure_x_reg_part2(hx));
-  ok(configure_x_reg_part3(hx)); ok(configure_x_reg_part4(hx)); ok(configure_x_reg_part5(hx));
-  ok(configure_x_reg_part6(hx)); ok(configure_x_reg_part7(hx));
-  ok(configure_y_reg_part0(hy)); ok(configure_y_reg_part1(hy)); ok(configure_y_reg_part2(hy));
-  ok(configure_y_reg_part3(hy));
+  ok(configure_z_reg_part0(Lz)); ok(configure_z_reg_part1(Lz)); ok(configure_z_reg_part2(Lz));
+  ok(configure_z_reg_part3(Lz)); ok(configure_z_reg_part4(Lz)); ok(configure_z_reg_part5(Lz));
+  ok(configure_x_reg_part0(Lx)); ok(configure_x_reg_part1(Lx)); ok(configure_x_reg_part2(Lx));
+  ok(configure_x_reg_part3(Lx)); ok(configure_x_reg_part4(Lx)); ok(configure_x_reg_part5(Lx));
+  ok(configure_x_reg_part6(Lx)); ok(configure_x_reg_part7(Lx)); ok(configure_x_reg_part8(Lx));
+  ok(configure_y_reg_part0(Ly)); ok(configure_y_reg_part1(Ly)); ok(configure_y_reg_part2(Ly));
+  ok(configure_y_reg_part3(Ly));
   return e;
 }
 
 bool launch_x_fwd_reg_any(int mode, const OpView<float>& op, int R, const float2* x, float2* buf,
                           const int* active, XinArgs<float> xa, cudaStream_t st) {
-  if (!op.twx_reg || op.Lx % 2) return false;
+  if (!op.twx_reg) return false;
 #define DDA_XREG_TRY(P) launch_x_fwd_reg_part##P(mode, op, R, x, buf, active, xa, st)
   return DDA_XREG_TRY(0) || DDA_XREG_TRY(1) || DDA_XREG_TRY(2) || DDA_XREG_TRY(3) ||
-         DDA_XREG_TRY(4) || DDA_XREG_TRY(5) || DDA_XREG_TRY(6) || DDA_XREG_TRY(7);
+         DDA_XREG_TRY(4) || DDA_XREG_TRY(5) || DDA_XREG_TRY(6) || DDA_XREG_TRY(7) ||
+         DDA_XREG_TRY(8);
 #undef DDA_XREG_TRY
 }
 
 bool launch_x_inv_reg_any(int mode, const OpView<float>& op, int R, const float2* buf,
                           const float2* x, float2* y, const int* active, const float2* rhat,
                           double* partials, cudaStream_t st, FoldArgs fold) {
-  if (!op.twx_reg || op.Lx % 2) return false;
+  if (!op.twx_reg) return false;
   const XInvArgs a{buf, x, y, rhat, partials, fold};
 #define DDA_XREG_TRY(P) launch_x_inv_reg_part##P(mode, op, R, a, active, st)
   return DDA_XREG_TRY(0) || DDA_XREG_TRY(1) || DDA_XREG_TRY(2) || DDA_XREG_TRY(3) ||
-         DDA_XREG_TRY(4) || DDA_XREG_TRY(5) || DDA_XREG_TRY(6) || DDA_XREG_TRY(7);
+         DDA_XREG_TRY(4) || DDA_XREG_TRY(5) || DDA_XREG_TRY(6) || DDA_XREG_TRY(7) ||
+         DDA_XREG_TRY(8);
 #undef DDA_XREG_TRY
 }
 
@@ -237,7 +235,7 @@ static bool launch_z_reg_any(const OpView<float>& op, int R, float2* buf, const 
 bool launch_z_fixed(const OpView<float>& op, const MatvecLaunch& L, int R, float2* scratch,
                     const int* active, cudaStream_t st) {
   bool done = false;
-  if (L.z_pair == 3) return op.twz_reg && op.Lz % 2 == 0 && launch_z_reg_any(op, R, scratch, active, st);
+  if (L.z_pair == 3) return op.twz_reg && launch_z_reg_any(op, R, scratch, active, st);
   if (L.z_pair) {
     if (!z_pair_applies(op.Lz, op.Lx, L.z_tile) || !op.twz_pair) return false;
     dispatch_length(op.Lz, PairPlans{}, [&](auto plan) {
@@ -292,7 +290,7 @@ bool launch_y_fixed(bool inv, const OpView<float>& op, const MatvecLaunch& L, in
                     float2* scratch, const int* active, cudaStream_t st) {
   bool done = false;
   // the register y passes, instantiated in ypass_reg_*.cu
-  if (L.y_reg && op.twy_reg && op.Ly % 2 == 0) {
+  if (L.y_reg && op.twy_reg) {
 #define DDA_YREG_TRY(P) launch_y_reg_part##P(inv, op, R, scratch, active, st)
     if (DDA_YREG_TRY(0) || DDA_YREG_TRY(1) || DDA_YREG_TRY(2) || DDA_YREG_TRY(3)) return true;
 #undef DDA_YREG_TRY

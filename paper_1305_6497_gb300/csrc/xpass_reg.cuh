@@ -24,20 +24,24 @@
 // where it was 5.7e-8 (RMS).
 #pragma once
 
-#include "fft_reg.cuh"
-#include "matvec_impl.cuh"
+#include "reg_step.cuh"
 
 namespace dda {
 
 constexpr int kXRegWarps = 4;  // per CTA
 
-template <int R1, int R2> struct XRegCfg {
-  static constexpr int n = R1 * R2, L = 2 * n;
-  static constexpr int ROW = R2 | 1, LS = R1 * ROW;  // float4 per k1 and per line
+// EO: L = 2 R1 R2, even and odd frequencies as halves; otherwise L = R1 R2 is odd and
+// the line is transformed whole, its rows j1 >= NJ zero.
+template <int R1, int R2, bool EO = true> struct XRegCfg {
+  static constexpr int n = R1 * R2, L = EO ? 2 * n : n;
+  static constexpr int NJ = EO ? R1 : ((L + 1) / 2 + R2 - 1) / R2;
+  static constexpr int NQ = EO ? 2 * R1 : R1;        // step 2's threads per row
+  static constexpr int EL = EO ? 2 : 1;              // float2 per element
+  static constexpr int ROW = R2 | 1, LS = R1 * ROW;  // elements per k1 and per line
   // issue slots a row costs with LW rows per warp (a packed R1-point DFT against a
   // scalar R2-point one), the least of LW = 1..4
   static constexpr int cost(int lw) {
-    return ((lw * R2 + 31) / 32 * R1 * 22 + (lw * 2 * R1 + 31) / 32 * R2 * 14) * 12 / lw;
+    return ((lw * R2 + 31) / 32 * R1 * (EO ? 22 : 14) + (lw * NQ + 31) / 32 * R2 * 14) * 12 / lw;
   }
   static constexpr int pick() {
     int b = 1;
@@ -46,8 +50,8 @@ template <int R1, int R2> struct XRegCfg {
     return b;
   }
   static constexpr int LW = pick();
-  static constexpr int U1 = LW * R2, U2 = LW * 2 * R1;
-  static constexpr size_t smem = (size_t)kXRegWarps * LW * LS * 16;
+  static constexpr int U1 = LW * R2, U2 = LW * NQ;
+  static constexpr size_t smem = (size_t)kXRegWarps * LW * LS * 8 * EL;
   static constexpr int regs = (4 * R1 > 2 * R2 ? 4 * R1 : 2 * R2) + 48;
   static constexpr int by_regs = 65536 / (32 * kXRegWarps * ((regs + 7) / 8 * 8));
   static constexpr int MINB = by_regs > 8 ? 8 : by_regs;
@@ -62,17 +66,18 @@ inline int x_reg_grid(int rows, int LW) {
   return (one + loops - 1) / loops;
 }
 
-template <int R1, int R2, int MODE>
-__global__ void __launch_bounds__(32 * kXRegWarps, XRegCfg<R1, R2>::MINB)
+template <int R1, int R2, bool EO, int MODE>
+__global__ void __launch_bounds__(32 * kXRegWarps, XRegCfg<R1, R2, EO>::MINB)
 k_x_fwd_reg(OpView<float> op, const float2* __restrict__ in, float2* __restrict__ buf,
             const int* __restrict__ active, XinArgs<float> xa) {
-  using K = XRegCfg<R1, R2>;
+  using K = XRegCfg<R1, R2, EO>;
   using C = float2;
+  constexpr int NJ = K::NJ, NQ = K::NQ, EL = K::EL;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int r = blockIdx.y;
   if (active && !active[r]) return;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  float4* sm = reinterpret_cast<float4*>(smem_raw) + wid * (K::LW * K::LS);
+  float2* sm = reinterpret_cast<float2*>(smem_raw) + wid * (EL * K::LW * K::LS);
   const int nx = op.nx, Lx = K::L;
   const int rows = 3 * op.nz * op.ny;
   C s1 = make_float2(0.f, 0.f), s2 = s1, s3 = s1;
@@ -99,26 +104,26 @@ k_x_fwd_reg(OpView<float> op, const float2* __restrict__ in, float2* __restrict_
       const int line = u / R2, j2 = u % R2;
       const int row = row0 + line;
       if (row >= rows) break;
-      const bool last = j2 + R2 * (R1 - 1) < nx;   // j < nx holds for the other j1
+      const bool last = j2 + R2 * (NJ - 1) < nx;   // j < nx holds for the other j1
       const int64_t g0 = off + (int64_t)row * nx + j2;
-      C x[R1];
+      C x[NJ];
       if constexpr (MODE == XIN_PLAIN) {
 #pragma unroll
-        for (int j = 0; j < R1; ++j) x[j] = __ldg(in + g0 + (j < R1 - 1 || last ? R2 * j : 0));
+        for (int j = 0; j < NJ; ++j) x[j] = __ldg(in + g0 + (j < NJ - 1 || last ? R2 * j : 0));
       } else {
-        C vb[R1], vc[R1], vd[R1];
+        C vb[NJ], vc[NJ], vd[NJ];
 #pragma unroll
-        for (int j = 0; j < R1; ++j) {
-          const int64_t g = g0 + (j < R1 - 1 || last ? R2 * j : 0);
+        for (int j = 0; j < NJ; ++j) {
+          const int64_t g = g0 + (j < NJ - 1 || last ? R2 * j : 0);
           x[j] = xa.r[g];
           if (MODE != XIN_S) vb[j] = xa.pv[g];
           vc[j] = MODE == XIN_Q ? xa.d[g] : xa.v[g];
           if (MODE == XIN_Q) vd[j] = xa.x[g];
         }
 #pragma unroll
-        for (int j = 0; j < R1; ++j) {
+        for (int j = 0; j < NJ; ++j) {
           const int64_t g = g0 + R2 * j;
-          const bool st = j < R1 - 1 || last;
+          const bool st = j < NJ - 1 || last;
           if (MODE == XIN_P) {
             x[j] = cadd(x[j], cmul(s1, csub(vb[j], cmul(s2, vc[j]))));
           } else if (MODE == XIN_Q) {
@@ -135,63 +140,46 @@ k_x_fwd_reg(OpView<float> op, const float2* __restrict__ in, float2* __restrict_
           if (st) xa.pv[g] = x[j];
         }
       }
-      if (!last) x[R1 - 1] = make_float2(0.f, 0.f);
-      cv<f32p> a[R1];
-      static_for<R1>([&](auto jc) {
-        constexpr int j = decltype(jc)::value;
-        const cv<float> o =
-            cvrot<false>(cv<float>{x[j].x, x[j].y}, cx_cos(j, 2 * R1), cx_sin(j, 2 * R1));
-        a[j] = {pk_make(x[j].x, o.re), pk_make(x[j].y, o.im)};
-      });
-      rdft<R1, false>(a);
-      float4* d = sm + line * K::LS + j2;
-#pragma unroll
-      for (int k = 0; k < R1; ++k) {
-        const float4 w = __ldg(tw + k * R2 + j2);
-        cv<float> e, o;
-        pk_split(a[k].re, e.re, o.re);
-        pk_split(a[k].im, e.im, o.im);
-        e = cvmul(e, cv<float>{w.x, w.y});
-        o = cvmul(o, cv<float>{w.z, w.w});
-        d[k * K::ROW] = make_float4(e.re, e.im, o.re, o.im);
-      }
+      if (!last) x[NJ - 1] = make_float2(0.f, 0.f);
+      reg_step1<R1, R2, EO>(x, tw + j2, sm + EL * (line * K::LS + j2), EL * K::ROW);
     }
     __syncwarp();
     for (int u = lane; u < K::U2; u += 32) {
-      const int line = u / (2 * R1), q = u % (2 * R1);
+      const int line = u / NQ, q = u % NQ;  // q = 2 k1 + parity, or k1
       const int row = row0 + line;
       if (row >= rows) break;
-      const float2* s = reinterpret_cast<const float2*>(sm + line * K::LS + (q >> 1) * K::ROW) + (q & 1);
+      const float2* s = sm + EL * (line * K::LS + (EO ? q >> 1 : q) * K::ROW) + (EO ? q & 1 : 0);
       cv<float> a[R2];
 #pragma unroll
       for (int j = 0; j < R2; ++j) {
-        const float2 e = s[2 * j];
+        const float2 e = s[EL * j];
         a[j] = {e.x, e.y};
       }
       rdft<R2, false>(a);
       const int plane = fast_div(row, op.div_ny), y = row - plane * op.ny;
       C* drow = dst + plane * plane_sz + (int64_t)y * Lx + q;
 #pragma unroll
-      for (int k = 0; k < R2; ++k) drow[2 * R1 * k] = make_float2(a[k].re, a[k].im);
+      for (int k = 0; k < R2; ++k) drow[NQ * k] = make_float2(a[k].re, a[k].im);
     }
     __syncwarp();
   }
 }
 
-template <int R1, int R2, int MODE>
-__global__ void __launch_bounds__(32 * kXRegWarps, XRegCfg<R1, R2>::MINB)
+template <int R1, int R2, bool EO, int MODE>
+__global__ void __launch_bounds__(32 * kXRegWarps, XRegCfg<R1, R2, EO>::MINB)
 k_x_inv_reg(OpView<float> op, const float2* __restrict__ buf, const float2* __restrict__ xin,
             float2* __restrict__ yout, const int* __restrict__ active,
             const float2* __restrict__ rhat, double* __restrict__ partials, FoldArgs fold) {
-  using K = XRegCfg<R1, R2>;
+  using K = XRegCfg<R1, R2, EO>;
   using C = float2;
+  constexpr int NJ = K::NJ, NQ = K::NQ, EL = K::EL;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int kAiSmem = 24;
   __shared__ C sai[kAiSmem];
   const int r = blockIdx.y;
   if (active && !active[r]) return;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  float4* sm = reinterpret_cast<float4*>(smem_raw) + wid * (K::LW * K::LS);
+  float2* sm = reinterpret_cast<float2*>(smem_raw) + wid * (EL * K::LW * K::LS);
   const int nx = op.nx, Lx = K::L;
   const int rows = 3 * op.nz * op.ny;
   const bool ai_smem = op.ncomp1 * 3 <= kAiSmem;
@@ -209,7 +197,7 @@ k_x_inv_reg(OpView<float> op, const float2* __restrict__ buf, const float2* __re
   for (int row0 = (blockIdx.x * kXRegWarps + wid) * K::LW; row0 < rows;
        row0 += gridDim.x * kXRegWarps * K::LW) {
     for (int u = lane; u < K::U2; u += 32) {
-      const int line = u / (2 * R1), q = u % (2 * R1);
+      const int line = u / NQ, q = u % NQ;
       const int row = row0 + line;
       if (row >= rows) break;
       const int plane = fast_div(row, op.div_ny), y = row - plane * op.ny;
@@ -217,53 +205,40 @@ k_x_inv_reg(OpView<float> op, const float2* __restrict__ buf, const float2* __re
       cv<float> a[R2];
 #pragma unroll
       for (int k = 0; k < R2; ++k) {
-        const float2 e = __ldcg(srow + 2 * R1 * k);
+        const float2 e = __ldcg(srow + NQ * k);
         a[k] = {e.x, e.y};
       }
       rdft<R2, true>(a);
-      float2* s = reinterpret_cast<float2*>(sm + line * K::LS + (q >> 1) * K::ROW) + (q & 1);
+      float2* s = sm + EL * (line * K::LS + (EO ? q >> 1 : q) * K::ROW) + (EO ? q & 1 : 0);
 #pragma unroll
-      for (int j = 0; j < R2; ++j) s[2 * j] = make_float2(a[j].re, a[j].im);
+      for (int j = 0; j < R2; ++j) s[EL * j] = make_float2(a[j].re, a[j].im);
     }
     __syncwarp();
     for (int u = lane; u < K::U1; u += 32) {
       const int line = u / R2, j2 = u % R2;
       const int row = row0 + line;
       if (row >= rows) break;
-      const bool last = j2 + R2 * (R1 - 1) < nx;
+      const bool last = j2 + R2 * (NJ - 1) < nx;
       // row = (c nz + z) ny + y  ->  sites (z ny + y) nx + j
       const int c = fast_div(fast_div(row, op.div_ny), op.div_nz);
       const uint8_t* cmp = op.comp + (int64_t)(row - c * op.nz * op.ny) * nx + j2;
       const int64_t g0 = off + (int64_t)row * nx + j2;
-      C xv[R1], hv[R1];
-      int cm[R1];
+      C xv[NJ], hv[NJ];
+      int cm[NJ];
 #pragma unroll
-      for (int j = 0; j < R1; ++j) {
-        const int o = j < R1 - 1 || last ? R2 * j : 0;
+      for (int j = 0; j < NJ; ++j) {
+        const int o = j < NJ - 1 || last ? R2 * j : 0;
         xv[j] = __ldg(xin + g0 + o);
         if (MODE == XOUT_RV) hv[j] = __ldg(rhat + g0 + o);
         cm[j] = __ldg(cmp + o);
       }
-      const float4* d = sm + line * K::LS + j2;
-      cv<f32p> a[R1];
+      C s[NJ];
+      reg_step1_inv<R1, R2, EO>(sm + EL * (line * K::LS + j2), EL * K::ROW, tw + j2, s);
 #pragma unroll
-      for (int k = 0; k < R1; ++k) {
-        const float4 p = d[k * K::ROW], w = __ldg(tw + k * R2 + j2);
-        const cv<float> e = cvmulc(cv<float>{w.x, w.y}, cv<float>{p.x, p.y});
-        const cv<float> o = cvmulc(cv<float>{w.z, w.w}, cv<float>{p.z, p.w});
-        a[k] = {pk_make(e.re, o.re), pk_make(e.im, o.im)};
-      }
-      rdft<R1, true>(a);
-      static_for<R1>([&](auto jc) {
-        constexpr int j = decltype(jc)::value;
-        constexpr float cw = (float)cx_cos(j, 2 * R1), sw = (float)cx_sin(j, 2 * R1);
-        if (j == R1 - 1 && !last) return;
-        float re, im, ro, io;
-        pk_split(a[j].re, re, ro);
-        pk_split(a[j].im, im, io);
-        const C s = make_float2(fmaf(cw, ro, fmaf(-sw, io, re)), fmaf(cw, io, fmaf(sw, ro, im)));
+      for (int j = 0; j < NJ; ++j) {
+        if (j == NJ - 1 && !last) break;
         C out = make_float2(0.f, 0.f);
-        if (cm[j]) out = csub(cmul(ai[3 * cm[j] + c], xv[j]), s);
+        if (cm[j]) out = csub(cmul(ai[3 * cm[j] + c], xv[j]), s[j]);
         yout[g0 + R2 * j] = out;
         if constexpr (MODE == XOUT_RV) {
           acc.add(0, hv[j].x * out.x + hv[j].y * out.y);
@@ -279,7 +254,7 @@ k_x_inv_reg(OpView<float> op, const float2* __restrict__ buf, const float2* __re
           acc.add(1, xv[j].x * out.y + xv[j].y * out.x);
           acc.step();
         }
-      });
+      }
     }
     __syncwarp();
   }
@@ -292,30 +267,30 @@ k_x_inv_reg(OpView<float> op, const float2* __restrict__ buf, const float2* __re
   }
 }
 
-template <int R1, int R2, int MODE>
+template <int R1, int R2, bool EO, int MODE>
 void launch_x_fwd_reg(const OpView<float>& op, int R, const float2* x, float2* buf,
                       const int* active, XinArgs<float> xa, cudaStream_t st) {
-  using K = XRegCfg<R1, R2>;
+  using K = XRegCfg<R1, R2, EO>;
   const dim3 g(x_reg_grid(3 * op.nz * op.ny, K::LW), R);
-  k_x_fwd_reg<R1, R2, MODE><<<g, 32 * kXRegWarps, K::smem, st>>>(op, x, buf, active, xa);
+  k_x_fwd_reg<R1, R2, EO, MODE><<<g, 32 * kXRegWarps, K::smem, st>>>(op, x, buf, active, xa);
 }
-template <int R1, int R2, int MODE>
+template <int R1, int R2, bool EO, int MODE>
 void launch_x_inv_reg(const OpView<float>& op, int R, const float2* buf, const float2* x, float2* y,
                       const int* active, const float2* rhat, double* partials, cudaStream_t st,
                       FoldArgs fold) {
-  using K = XRegCfg<R1, R2>;
+  using K = XRegCfg<R1, R2, EO>;
   const dim3 g(x_reg_grid(3 * op.nz * op.ny, K::LW), R);
-  k_x_inv_reg<R1, R2, MODE><<<g, 32 * kXRegWarps, K::smem, st>>>(op, buf, x, y, active, rhat,
+  k_x_inv_reg<R1, R2, EO, MODE><<<g, 32 * kXRegWarps, K::smem, st>>>(op, buf, x, y, active, rhat,
                                                                 partials, fold);
 }
-template <int R1, int R2> cudaError_t configure_x_reg() {
-  const void* k[] = {(const void*)k_x_fwd_reg<R1, R2, XIN_PLAIN>, (const void*)k_x_fwd_reg<R1, R2, XIN_P>,
-                     (const void*)k_x_fwd_reg<R1, R2, XIN_S>, (const void*)k_x_fwd_reg<R1, R2, XIN_Q>,
-                     (const void*)k_x_inv_reg<R1, R2, XOUT_PLAIN>, (const void*)k_x_inv_reg<R1, R2, XOUT_RV>,
-                     (const void*)k_x_inv_reg<R1, R2, XOUT_TS>, (const void*)k_x_inv_reg<R1, R2, XOUT_QT>};
+template <int R1, int R2, bool EO> cudaError_t configure_x_reg() {
+  const void* k[] = {(const void*)k_x_fwd_reg<R1, R2, EO, XIN_PLAIN>, (const void*)k_x_fwd_reg<R1, R2, EO, XIN_P>,
+                     (const void*)k_x_fwd_reg<R1, R2, EO, XIN_S>, (const void*)k_x_fwd_reg<R1, R2, EO, XIN_Q>,
+                     (const void*)k_x_inv_reg<R1, R2, EO, XOUT_PLAIN>, (const void*)k_x_inv_reg<R1, R2, EO, XOUT_RV>,
+                     (const void*)k_x_inv_reg<R1, R2, EO, XOUT_TS>, (const void*)k_x_inv_reg<R1, R2, EO, XOUT_QT>};
   for (const void* f : k) {
     const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)XRegCfg<R1, R2>::smem);
+                                               (int)XRegCfg<R1, R2, EO>::smem);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -349,48 +324,57 @@ struct XInvArgs {
                                    cudaStream_t st);                                         \
   bool launch_x_inv_reg_part##PART(int mode, const OpView<float>& op, int R,                  \
                                    const XInvArgs& a, const int* active, cudaStream_t st);   \
-  cudaError_t configure_x_reg_part##PART(int half);
+  cudaError_t configure_x_reg_part##PART(int L);
 DDA_XREG_DECLARE(0) DDA_XREG_DECLARE(1) DDA_XREG_DECLARE(2) DDA_XREG_DECLARE(3)
 DDA_XREG_DECLARE(4) DDA_XREG_DECLARE(5) DDA_XREG_DECLARE(6) DDA_XREG_DECLARE(7)
+DDA_XREG_DECLARE(8)
 
-template <int A, int B>
+template <int A, int B, bool EO>
 void x_fwd_reg_mode(int mode, const OpView<float>& op, int R, const float2* x, float2* buf,
                     const int* active, XinArgs<float> xa, cudaStream_t st) {
-  if (mode == XIN_PLAIN) launch_x_fwd_reg<A, B, XIN_PLAIN>(op, R, x, buf, active, xa, st);
-  else if (mode == XIN_P) launch_x_fwd_reg<A, B, XIN_P>(op, R, x, buf, active, xa, st);
-  else if (mode == XIN_S) launch_x_fwd_reg<A, B, XIN_S>(op, R, x, buf, active, xa, st);
-  else launch_x_fwd_reg<A, B, XIN_Q>(op, R, x, buf, active, xa, st);
+  if (mode == XIN_PLAIN) launch_x_fwd_reg<A, B, EO, XIN_PLAIN>(op, R, x, buf, active, xa, st);
+  else if (mode == XIN_P) launch_x_fwd_reg<A, B, EO, XIN_P>(op, R, x, buf, active, xa, st);
+  else if (mode == XIN_S) launch_x_fwd_reg<A, B, EO, XIN_S>(op, R, x, buf, active, xa, st);
+  else launch_x_fwd_reg<A, B, EO, XIN_Q>(op, R, x, buf, active, xa, st);
 }
-template <int A, int B>
+template <int A, int B, bool EO>
 void x_inv_reg_mode(int mode, const OpView<float>& op, int R, const XInvArgs& a, const int* active,
                     cudaStream_t st) {
   if (mode == XOUT_PLAIN)
-    launch_x_inv_reg<A, B, XOUT_PLAIN>(op, R, a.buf, a.x, a.y, active, a.rhat, a.partials, st, a.fold);
+    launch_x_inv_reg<A, B, EO, XOUT_PLAIN>(op, R, a.buf, a.x, a.y, active, a.rhat, a.partials, st, a.fold);
   else if (mode == XOUT_RV)
-    launch_x_inv_reg<A, B, XOUT_RV>(op, R, a.buf, a.x, a.y, active, a.rhat, a.partials, st, a.fold);
+    launch_x_inv_reg<A, B, EO, XOUT_RV>(op, R, a.buf, a.x, a.y, active, a.rhat, a.partials, st, a.fold);
   else if (mode == XOUT_TS)
-    launch_x_inv_reg<A, B, XOUT_TS>(op, R, a.buf, a.x, a.y, active, a.rhat, a.partials, st, a.fold);
+    launch_x_inv_reg<A, B, EO, XOUT_TS>(op, R, a.buf, a.x, a.y, active, a.rhat, a.partials, st, a.fold);
   else
-    launch_x_inv_reg<A, B, XOUT_QT>(op, R, a.buf, a.x, a.y, active, a.rhat, a.partials, st, a.fold);
+    launch_x_inv_reg<A, B, EO, XOUT_QT>(op, R, a.buf, a.x, a.y, active, a.rhat, a.partials, st, a.fold);
 }
-#define DDA_XREG_FWD(A, B) case (A) * (B): x_fwd_reg_mode<A, B>(mode, op, R, x, buf, active, xa, st); return true;
-#define DDA_XREG_INV(A, B) case (A) * (B): x_inv_reg_mode<A, B>(mode, op, R, a, active, st); return true;
-#define DDA_XREG_CONFIG(A, B) case (A) * (B): return configure_x_reg<A, B>();
-#define DDA_XREG_DEFINE(PART)                                                                \
+#define DDA_XREG_FWD(A, B) \
+  case 2 * (A) * (B): x_fwd_reg_mode<A, B, true>(mode, op, R, x, buf, active, xa, st); return true;
+#define DDA_XREG_INV(A, B) \
+  case 2 * (A) * (B): x_inv_reg_mode<A, B, true>(mode, op, R, a, active, st); return true;
+#define DDA_XREG_CONFIG(A, B) case 2 * (A) * (B): return configure_x_reg<A, B, true>();
+#define DDA_XREG_FWD_ODD(A, B) \
+  case (A) * (B): x_fwd_reg_mode<A, B, false>(mode, op, R, x, buf, active, xa, st); return true;
+#define DDA_XREG_INV_ODD(A, B) \
+  case (A) * (B): x_inv_reg_mode<A, B, false>(mode, op, R, a, active, st); return true;
+#define DDA_XREG_CONFIG_ODD(A, B) case (A) * (B): return configure_x_reg<A, B, false>();
+// LIST: the lengths' plans, ODD: empty or _ODD
+#define DDA_XREG_DEFINE(PART, LIST, ODD)                                                     \
   bool launch_x_fwd_reg_part##PART(int mode, const OpView<float>& op, int R, const float2* x, \
                                    float2* buf, const int* active, XinArgs<float> xa,        \
                                    cudaStream_t st) {                                        \
-    switch (op.Lx / 2) { DDA_XREG_PART##PART(DDA_XREG_FWD) }                                 \
+    switch (op.Lx) { LIST(DDA_XREG_FWD##ODD) }                                               \
     return false;                                                                            \
   }                                                                                          \
   bool launch_x_inv_reg_part##PART(int mode, const OpView<float>& op, int R,                  \
                                    const XInvArgs& a, const int* active, cudaStream_t st) {  \
-    switch (op.Lx / 2) { DDA_XREG_PART##PART(DDA_XREG_INV) }                                 \
+    switch (op.Lx) { LIST(DDA_XREG_INV##ODD) }                                               \
     return false;                                                                            \
   }                                                                                          \
-  cudaError_t configure_x_reg_part##PART(int half) {                                           \
-    switch (half) { DDA_XREG_PART##PART(DDA_XREG_CONFIG) }                                     \
-    return cudaSuccess;                                                                        \
+  cudaError_t configure_x_reg_part##PART(int L) {                                            \
+    switch (L) { LIST(DDA_XREG_CONFIG##ODD) }                                                \
+    return cudaSuccess;                                                                      \
   }
 
 }  // namespace dda

@@ -19,13 +19,15 @@
 
 namespace dda {
 
-template <int R1, int R2> struct YRegCfg {
-  static constexpr int n = R1 * R2, L = 2 * n;
+template <int R1, int R2, bool EO = true> struct YRegCfg {
+  static constexpr int n = R1 * R2, L = EO ? 2 * n : n;
+  static constexpr int NJ = XRegCfg<R1, R2, EO>::NJ, NQ = XRegCfg<R1, R2, EO>::NQ;
+  static constexpr int EL = EO ? 2 : 1;  // float2 per element
   static constexpr int TILE = n <= 128 || n >= 192 ? 16 : 8;
-  static constexpr int U1 = TILE * R2, U2 = TILE * 2 * R1;
+  static constexpr int U1 = TILE * R2, U2 = TILE * NQ;
   static constexpr int most = ((U1 > U2 ? U1 : U2) + 31) / 32 * 32;
   static constexpr int NT = most > 320 ? (most / 2 + 31) / 32 * 32 : most;
-  static constexpr size_t smem = (size_t)n * TILE * 16;
+  static constexpr size_t smem = (size_t)n * TILE * 8 * EL;
   static constexpr int regs = (4 * R1 > 2 * R2 ? 4 * R1 : 2 * R2) + 44;
   static constexpr int by_regs = 65536 / (NT * ((regs + 7) / 8 * 8));
   static constexpr int by_smem = (int)(227 * 1024 / (smem + 1024));
@@ -33,13 +35,13 @@ template <int R1, int R2> struct YRegCfg {
   static constexpr int MINB = fit < 1 ? 1 : fit > 2048 / NT ? 2048 / NT : fit;
 };
 
-template <int R1, int R2, bool INV>
-__global__ void __launch_bounds__(YRegCfg<R1, R2>::NT, YRegCfg<R1, R2>::MINB)
+template <int R1, int R2, bool EO, bool INV>
+__global__ void __launch_bounds__(YRegCfg<R1, R2, EO>::NT, YRegCfg<R1, R2, EO>::MINB)
 k_y_reg(OpView<float> op, float2* __restrict__ buf, const int* __restrict__ active) {
-  using K = YRegCfg<R1, R2>;
-  constexpr int TILE = K::TILE, NT = K::NT;
+  using K = YRegCfg<R1, R2, EO>;
+  constexpr int TILE = K::TILE, NT = K::NT, NJ = K::NJ, NQ = K::NQ, EL = K::EL;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  float4* sm = reinterpret_cast<float4*>(smem_raw);
+  float2* sm = reinterpret_cast<float2*>(smem_raw);
   const int r = blockIdx.z;
   if (active && !active[r]) return;
   const int Lx = op.Lx, ny = op.ny;
@@ -48,119 +50,96 @@ k_y_reg(OpView<float> op, float2* __restrict__ buf, const int* __restrict__ acti
   float2* base = buf + ((int64_t)r * 3 * op.nz + blockIdx.y) * (int64_t)K::L * Lx + col0;
   const float4* __restrict__ tw = op.twy_reg;
   // step 1's threads hold rows j2 + R2 j1 of one column, step 2's the frequencies
-  // 2 (k1 + R1 k2) + p; a half-warp of step 2 covers 8 columns x both parities
-  auto place2 = [&](int u, int& t, int& p, int& k1) {
-    t = u % 8;
-    p = (u / 8) & 1;
-    const int h = u / 16;
-    t += 8 * (h % (TILE / 8));
-    k1 = h / (TILE / 8);
+  // q + NQ k2 (q = 2 k1 + parity, or k1); with two parities a half-warp of step 2
+  // covers 8 columns x both
+  auto place2 = [&](int u, int& t, int& q) {
+    if (EO) {
+      const int h = u / 16;
+      t = u % 8 + 8 * (h % (TILE / 8));
+      q = 2 * (h / (TILE / 8)) + ((u / 8) & 1);
+    } else {
+      t = u % TILE;
+      q = u / TILE;
+    }
+  };
+  auto element = [&](int t, int q) {
+    return sm + EL * ((EO ? q >> 1 : q) * R2 * TILE + t) + (EO ? q & 1 : 0);
   };
   if (!INV) {
     for (int u = threadIdx.x; u < K::U1; u += NT) {
       const int t = u % TILE, j2 = u / TILE;
       const float2* src = base + (int64_t)j2 * Lx + min(t, ncol - 1);
-      const bool last = j2 + R2 * (R1 - 1) < ny;  // row < ny holds for the other j1
-      float2 x[R1];
+      const bool last = j2 + R2 * (NJ - 1) < ny;  // row < ny holds for the other j1
+      float2 x[NJ];
 #pragma unroll
-      for (int j = 0; j < R1; ++j) x[j] = __ldcg(src + (j < R1 - 1 || last ? j * R2 * Lx : 0));
-      if (!last) x[R1 - 1] = make_float2(0.f, 0.f);
-      cv<f32p> a[R1];
-      static_for<R1>([&](auto jc) {
-        constexpr int j = decltype(jc)::value;
-        const cv<float> o =
-            cvrot<false>(cv<float>{x[j].x, x[j].y}, cx_cos(j, 2 * R1), cx_sin(j, 2 * R1));
-        a[j] = {pk_make(x[j].x, o.re), pk_make(x[j].y, o.im)};
-      });
-      rdft<R1, false>(a);
-#pragma unroll
-      for (int k = 0; k < R1; ++k) {
-        const float4 w = __ldg(tw + k * R2 + j2);
-        cv<float> e, o;
-        pk_split(a[k].re, e.re, o.re);
-        pk_split(a[k].im, e.im, o.im);
-        e = cvmul(e, cv<float>{w.x, w.y});
-        o = cvmul(o, cv<float>{w.z, w.w});
-        sm[(k * R2 + j2) * TILE + t] = make_float4(e.re, e.im, o.re, o.im);
-      }
+      for (int j = 0; j < NJ; ++j) x[j] = __ldcg(src + (j < NJ - 1 || last ? j * R2 * Lx : 0));
+      if (!last) x[NJ - 1] = make_float2(0.f, 0.f);
+      reg_step1<R1, R2, EO>(x, tw + j2, sm + EL * (j2 * TILE + t), EL * R2 * TILE);
     }
     __syncthreads();
     for (int u = threadIdx.x; u < K::U2; u += NT) {
-      int t, p, k1;
-      place2(u, t, p, k1);
-      const float2* s = reinterpret_cast<const float2*>(sm + k1 * R2 * TILE + t) + p;
+      int t, q;
+      place2(u, t, q);
+      const float2* s = element(t, q);
       cv<float> a[R2];
 #pragma unroll
       for (int j = 0; j < R2; ++j) {
-        const float2 e = s[2 * TILE * j];
+        const float2 e = s[EL * TILE * j];
         a[j] = {e.x, e.y};
       }
       rdft<R2, false>(a);
       if (t < ncol) {
-        float2* dst = base + (int64_t)(2 * k1 + p) * Lx + t;
+        float2* dst = base + (int64_t)q * Lx + t;
 #pragma unroll
-        for (int k = 0; k < R2; ++k) dst[(int64_t)2 * R1 * k * Lx] = make_float2(a[k].re, a[k].im);
+        for (int k = 0; k < R2; ++k) dst[(int64_t)NQ * k * Lx] = make_float2(a[k].re, a[k].im);
       }
     }
   } else {
     for (int u = threadIdx.x; u < K::U2; u += NT) {
-      int t, p, k1;
-      place2(u, t, p, k1);
-      const float2* src = base + (int64_t)(2 * k1 + p) * Lx + min(t, ncol - 1);
+      int t, q;
+      place2(u, t, q);
+      const float2* src = base + (int64_t)q * Lx + min(t, ncol - 1);
       cv<float> a[R2];
 #pragma unroll
       for (int k = 0; k < R2; ++k) {
-        const float2 e = __ldcg(src + (int64_t)2 * R1 * k * Lx);
+        const float2 e = __ldcg(src + (int64_t)NQ * k * Lx);
         a[k] = {e.x, e.y};
       }
       rdft<R2, true>(a);
-      float2* s = reinterpret_cast<float2*>(sm + k1 * R2 * TILE + t) + p;
+      float2* s = element(t, q);
 #pragma unroll
-      for (int j = 0; j < R2; ++j) s[2 * TILE * j] = make_float2(a[j].re, a[j].im);
+      for (int j = 0; j < R2; ++j) s[EL * TILE * j] = make_float2(a[j].re, a[j].im);
     }
     __syncthreads();
     for (int u = threadIdx.x; u < K::U1; u += NT) {
       const int t = u % TILE, j2 = u / TILE;
       if (t >= ncol) continue;
-      const bool last = j2 + R2 * (R1 - 1) < ny;
-      cv<f32p> a[R1];
-#pragma unroll
-      for (int k = 0; k < R1; ++k) {
-        const float4 q = sm[(k * R2 + j2) * TILE + t], w = __ldg(tw + k * R2 + j2);
-        const cv<float> e = cvmulc(cv<float>{w.x, w.y}, cv<float>{q.x, q.y});
-        const cv<float> o = cvmulc(cv<float>{w.z, w.w}, cv<float>{q.z, q.w});
-        a[k] = {pk_make(e.re, o.re), pk_make(e.im, o.im)};
-      }
-      rdft<R1, true>(a);
+      const bool last = j2 + R2 * (NJ - 1) < ny;
+      float2 y[NJ];
+      reg_step1_inv<R1, R2, EO>(sm + EL * (j2 * TILE + t), EL * R2 * TILE, tw + j2, y);
       float2* dst = base + (int64_t)j2 * Lx + t;
-      static_for<R1>([&](auto jc) {
-        constexpr int j = decltype(jc)::value;
-        constexpr float cw = (float)cx_cos(j, 2 * R1), sw = (float)cx_sin(j, 2 * R1);
-        float re, im, ro, io;
-        pk_split(a[j].re, re, ro);
-        pk_split(a[j].im, im, io);
-        if (j < R1 - 1 || last)
-          dst[(int64_t)j * R2 * Lx] = make_float2(fmaf(cw, ro, fmaf(-sw, io, re)),
-                                                  fmaf(cw, io, fmaf(sw, ro, im)));
-      });
+#pragma unroll
+      for (int j = 0; j < NJ; ++j)
+        if (j < NJ - 1 || last) dst[(int64_t)j * R2 * Lx] = y[j];
     }
   }
 }
 
-template <int R1, int R2>
+template <int R1, int R2, bool EO>
 void launch_y_reg(bool inv, const OpView<float>& op, int R, float2* buf, const int* active,
                   cudaStream_t st) {
-  using K = YRegCfg<R1, R2>;
+  using K = YRegCfg<R1, R2, EO>;
   const dim3 g((op.Lx + K::TILE - 1) / K::TILE, 3 * op.nz, R);
-  if (inv) k_y_reg<R1, R2, true><<<g, K::NT, K::smem, st>>>(op, buf, active);
-  else k_y_reg<R1, R2, false><<<g, K::NT, K::smem, st>>>(op, buf, active);
+  if (inv) k_y_reg<R1, R2, EO, true><<<g, K::NT, K::smem, st>>>(op, buf, active);
+  else k_y_reg<R1, R2, EO, false><<<g, K::NT, K::smem, st>>>(op, buf, active);
 }
-template <int R1, int R2> cudaError_t configure_y_reg() {
+template <int R1, int R2, bool EO> cudaError_t configure_y_reg() {
+  const int smem = (int)YRegCfg<R1, R2, EO>::smem;
   const cudaError_t e = cudaFuncSetAttribute(
-      k_y_reg<R1, R2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)YRegCfg<R1, R2>::smem);
+      k_y_reg<R1, R2, EO, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_y_reg<R1, R2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)YRegCfg<R1, R2>::smem);
+  return cudaFuncSetAttribute(k_y_reg<R1, R2, EO, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              smem);
 }
 
 // The plans of the x passes, in parts that compile side by side (ypass_reg_*.cu).
@@ -171,20 +150,24 @@ template <int R1, int R2> cudaError_t configure_y_reg() {
 #define DDA_YREG_DECLARE(PART)                                                                    \
   bool launch_y_reg_part##PART(bool inv, const OpView<float>& op, int R, float2* buf,             \
                                const int* active, cudaStream_t st);                               \
-  cudaError_t configure_y_reg_part##PART(int half);
+  cudaError_t configure_y_reg_part##PART(int L);
 DDA_YREG_DECLARE(0) DDA_YREG_DECLARE(1) DDA_YREG_DECLARE(2) DDA_YREG_DECLARE(3)
 
-#define DDA_YREG_LAUNCH(A, B) case (A) * (B): launch_y_reg<A, B>(inv, op, R, buf, active, st); return true;
-#define DDA_YREG_CONFIG(A, B) case (A) * (B): return configure_y_reg<A, B>();
-#define DDA_YREG_DEFINE(PART)                                                                     \
+#define DDA_YREG_LAUNCH(A, B) \
+  case 2 * (A) * (B): launch_y_reg<A, B, true>(inv, op, R, buf, active, st); return true;
+#define DDA_YREG_CONFIG(A, B) case 2 * (A) * (B): return configure_y_reg<A, B, true>();
+#define DDA_YREG_LAUNCH_ODD(A, B) \
+  case (A) * (B): launch_y_reg<A, B, false>(inv, op, R, buf, active, st); return true;
+#define DDA_YREG_CONFIG_ODD(A, B) case (A) * (B): return configure_y_reg<A, B, false>();
+// ODDS: the list of odd plans, or nothing
+#define DDA_YREG_DEFINE(PART, ODDS)                                                               \
   bool launch_y_reg_part##PART(bool inv, const OpView<float>& op, int R, float2* buf,             \
                                const int* active, cudaStream_t st) {                              \
-    switch (op.Ly / 2) { DDA_YREG_PART##PART(DDA_YREG_LAUNCH) }                                   \
+    switch (op.Ly) { DDA_YREG_PART##PART(DDA_YREG_LAUNCH) ODDS(DDA_YREG_LAUNCH_ODD) }             \
     return false;                                                                                 \
   }                                                                                               \
-  cudaError_t configure_y_reg_part##PART(int half) {                                               \
-    switch (half) { DDA_YREG_PART##PART(DDA_YREG_CONFIG) }                                         \
-    return cudaSuccess;                                                                            \
+  cudaError_t configure_y_reg_part##PART(int L) {                                                 \
+    switch (L) { DDA_YREG_PART##PART(DDA_YREG_CONFIG) ODDS(DDA_YREG_CONFIG_ODD) }                 \
+    return cudaSuccess;                                                                           \
   }
-
 }  // namespace dda

@@ -2,5 +2,5 @@
 #include "ypass_reg.cuh"
 
 namespace dda {
-DDA_YREG_DEFINE(2)
+DDA_YREG_DEFINE(2, DDA_REG_NONE)
 }  // namespace dda

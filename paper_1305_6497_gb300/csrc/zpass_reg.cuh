@@ -39,24 +39,29 @@
 // 589 -> 180 us; 48x96x144 319 -> 128 us; 64^3 76 (tuned 54) -> 47 us.
 #pragma once
 
-#include "fft_reg.cuh"
-#include "matvec_impl.cuh"
+#include "reg_step.cuh"
 
 namespace dda {
 
-template <int R1, int R2> struct ZRegCfg {
-  static constexpr int n = R1 * R2, L = 2 * n, Hz = n + 1;
-  static constexpr int TILE = n <= 96 ? 8 : 4;  // columns per CTA
-  static constexpr int U1 = 3 * TILE * R2;      // threads at work in steps 1 and 3
-  static constexpr int U2 = 2 * TILE * R1;      // in step 2
+// EO: L = 2 R1 R2, even and odd frequencies as halves; otherwise L = R1 R2 is odd, the
+// line is transformed whole in scalar arithmetic (elements of 8 bytes, rows j1 >= NJ
+// zero, no parities in step 2).
+template <int R1, int R2, bool EO> struct ZRegCfg {
+  static constexpr int n = R1 * R2, L = EO ? 2 * n : n, Hz = L / 2 + 1;
+  static constexpr int NJ = EO ? R1 : ((L + 1) / 2 + R2 - 1) / R2;
+  static constexpr int EL = EO ? 2 : 1;              // float2 per element
+  static constexpr int TILE = !EO || n <= 96 ? 8 : 4;  // columns per CTA
+  static constexpr int U1 = 3 * TILE * R2;           // threads at work in steps 1 and 3
+  static constexpr int U2 = (EO ? 2 : 1) * TILE * R1;  // in step 2
   static constexpr int NT = ((U1 > U2 ? U1 : U2) + 31) / 32 * 32;
-  // float4 per (component, k1): with 4 columns a half-warp covers two k1, which
-  // half a bank row more keeps apart
-  static constexpr int ROW = R2 * TILE + (TILE == 4 && R2 % 2 == 0 ? 4 : 0);
+  // elements per (component, k1): with 4 columns a half-warp covers two k1, which
+  // half a bank row more keeps apart (odd L: 8 columns and odd R2 do that already)
+  static constexpr int ROW = R2 * TILE + (EO && TILE == 4 && R2 % 2 == 0 ? 4 : 0);
   // float4 per column of the Ghat tile: 8 columns want an odd stride, 4 columns
   // (x 2 parities) one of 2 mod 4
   static constexpr int GS = TILE == 8 ? (3 * Hz) | 1 : (3 * Hz + 1) / 4 * 4 + 2;
-  static constexpr size_t smem = (size_t)(3 * R1 * ROW + TILE * GS + n) * 16;
+  static constexpr int ex4 = (3 * R1 * ROW * EL + 1) / 2;  // exchange, in float4
+  static constexpr size_t smem = (size_t)(ex4 + TILE * GS + n) * 16;
   static constexpr int regs1 = 4 * R1 + 44, regs2 = 6 * R2 + 44;
   static constexpr int regs = ((regs1 > regs2 ? regs1 : regs2) + 7) / 8 * 8;
   static constexpr int by_regs = 65536 / (NT * regs), by_smem = (int)(227 * 1024 / (smem + 1024));
@@ -68,15 +73,16 @@ __device__ __forceinline__ float flip_if(float a, unsigned m) {
   return __uint_as_float(__float_as_uint(a) ^ m);
 }
 
-template <int R1, int R2, bool ASYNC>
-__global__ void __launch_bounds__(ZRegCfg<R1, R2>::NT, ZRegCfg<R1, R2>::MINB)
+template <int R1, int R2, bool EO, bool ASYNC>
+__global__ void __launch_bounds__(ZRegCfg<R1, R2, EO>::NT, ZRegCfg<R1, R2, EO>::MINB)
 k_fft_z_reg(OpView<float> op, float2* __restrict__ buf, int R, int per,
             const int* __restrict__ active) {
-  using K = ZRegCfg<R1, R2>;
+  using K = ZRegCfg<R1, R2, EO>;
   constexpr int n = K::n, L = K::L, TILE = K::TILE, NT = K::NT, ROW = K::ROW, Hz = K::Hz;
+  constexpr int NJ = K::NJ, EL = K::EL;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  float4* sm = reinterpret_cast<float4*>(smem_raw);
-  float4* gsm = sm + 3 * R1 * ROW;
+  float2* sm = reinterpret_cast<float2*>(smem_raw);
+  float4* gsm = reinterpret_cast<float4*>(smem_raw) + K::ex4;
   float4* tws = gsm + TILE * K::GS;
   const int hy = blockIdx.y;
   const int Lx = op.Lx, Ly = op.Ly, nz = op.nz;
@@ -96,12 +102,12 @@ k_fft_z_reg(OpView<float> op, float2* __restrict__ buf, int R, int per,
   const int t1 = threadIdx.x % TILE, j2 = (threadIdx.x / TILE) % R2;
   const int c1 = threadIdx.x / (TILE * R2);
   const bool on1 = c1 < 3 && t1 < ncol;
-  const bool last = j2 + R2 * (R1 - 1) < nz;  // z < nz holds for the other j1
+  const bool last = j2 + R2 * (NJ - 1) < nz;  // z < nz holds for the other j1
   float2* const first = buf + col0 + min(t1, ncol - 1) + min(c1, 2) * comp + j2 * plane;
   const int64_t row0 = (int64_t)op.ypos_at[hy] * Lx;
   const int64_t row1 = (int64_t)op.ypos_at[self ? hy : Ly - hy] * Lx;
   auto line = [&](int w) { return first + (w >> 1) * 3 * comp + ((w & 1) ? row1 : row0); };
-  float4* own = sm + c1 * (R1 * ROW) + j2 * TILE + t1;
+  float2* own = sm + EL * (c1 * (R1 * ROW) + j2 * TILE + t1);
   // The next pass's input is asked for as soon as step 3 has read the thread's
   // words of shared memory, and lands in them (ASYNC: 16-byte asynchronous copies
   // past L1, each holding the two columns of a pair of threads for one row; the
@@ -109,23 +115,26 @@ k_fft_z_reg(OpView<float> op, float2* __restrict__ buf, int R, int per,
   // L1 for each of their 32-byte rows until they arrive, and the shared memory
   // leaves L1 room for a fifth of a pass's; they remain for odd Lx, where pairs of
   // columns are not 16-byte aligned.  Every load is unconditional as far as it can
-  // be: only the last row (j1 = R1 - 1) may lie beyond nz.
-  float2 x[R1];
+  // be: only the last row (j1 = NJ - 1) may lie beyond nz.  (EO: row j1 lands in word
+  // j1 / 2 of the pair's thread of j1's parity; odd L, words of 8 bytes: in word j1 of
+  // both.)
+  float2 x[NJ];
   auto fetch = [&](int w) {
     if constexpr (ASYNC) {
       if (!on1) return;
       const float2* src = line(w) - (t1 & 1);
 #pragma unroll
-      for (int i = 0; i < (R1 + 1) / 2; ++i) {
+      for (int i = 0; i < (NJ + 1) / 2; ++i) {
         const int j = 2 * i + (t1 & 1);
-        if (j < R1 - 1 || (j == R1 - 1 && last)) cp_async<16>(own + i * ROW, src + (int64_t)j * R2 * plane);
+        float2* dst = EO ? own + EL * i * ROW : own - (t1 & 1) + j * ROW;
+        if (j < NJ - 1 || (j == NJ - 1 && last)) cp_async<16>(dst, src + (int64_t)j * R2 * plane);
       }
       cp_async_commit();
     } else {
       const float2* src = line(w);
 #pragma unroll
-      for (int j = 0; j < R1; ++j)
-        x[j] = __ldcg(src + (j < R1 - 1 || last ? (int64_t)j * R2 * plane : 0));
+      for (int j = 0; j < NJ; ++j)
+        x[j] = __ldcg(src + (j < NJ - 1 || last ? (int64_t)j * R2 * plane : 0));
     }
   };
   fetch(v);
@@ -145,7 +154,8 @@ k_fft_z_reg(OpView<float> op, float2* __restrict__ buf, int R, int per,
   for (int e = threadIdx.x; e < n; e += NT) cp_async<16>(tws + e, op.twz_reg + e);
   cp_async_commit();
   // and in step 2
-  const int t2 = threadIdx.x % TILE, p2 = (threadIdx.x / TILE) & 1, k2 = threadIdx.x / (2 * TILE);
+  const int t2 = threadIdx.x % TILE, p2 = EO ? (threadIdx.x / TILE) & 1 : 0;
+  const int k2 = threadIdx.x / ((EO ? 2 : 1) * TILE);
   const unsigned mx = op.kx_at[col0 + min(t2, ncol - 1)] > (Lx >> 1) ? 0x80000000u : 0u;
   const float4* tw = tws + j2;
 
@@ -161,38 +171,21 @@ k_fft_z_reg(OpView<float> op, float2* __restrict__ buf, int R, int per,
       __syncwarp();
       if (c1 < 3) {
 #pragma unroll
-        for (int j = 0; j < R1; ++j)
-          x[j] = reinterpret_cast<const float2*>(own - (t1 & 1) + (j & 1) + (j >> 1) * ROW)[t1 & 1];
+        for (int j = 0; j < NJ; ++j)
+          x[j] = EO ? own[EL * ((j & 1) - (t1 & 1) + (j >> 1) * ROW) + (t1 & 1)] : own[j * ROW];
       }
       __syncwarp();
     }
     if (c1 < 3) {
-      cv<f32p> a[R1];
-      if (!last) x[R1 - 1] = make_float2(0.f, 0.f);
-      static_for<R1>([&](auto jc) {
-        constexpr int j = decltype(jc)::value;  // w_L^(R2 j) = exp(-i pi j / R1)
-        const cv<float> o =
-            cvrot<false>(cv<float>{x[j].x, x[j].y}, cx_cos(j, 2 * R1), cx_sin(j, 2 * R1));
-        a[j] = {pk_make(x[j].x, o.re), pk_make(x[j].y, o.im)};
-      });
-      rdft<R1, false>(a);
-#pragma unroll
-      for (int k = 0; k < R1; ++k) {
-        const float4 w = tw[k * R2];
-        cv<float> e, o;
-        pk_split(a[k].re, e.re, o.re);
-        pk_split(a[k].im, e.im, o.im);
-        e = cvmul(e, cv<float>{w.x, w.y});
-        o = cvmul(o, cv<float>{w.z, w.w});
-        own[k * ROW] = make_float4(e.re, e.im, o.re, o.im);
-      }
+      if (!last) x[NJ - 1] = make_float2(0.f, 0.f);
+      reg_step1<R1, R2, EO>(x, tw, own, EL * ROW);
     }
     __syncthreads();
     if (!ASYNC && vn < vend) fetch(vn);  // lands while step 2 computes
 
     // ---- 2. R2-point DFTs of the three components, multiply, inverse DFTs
     if (k2 < R1) {
-      float2* q = reinterpret_cast<float2*>(sm + k2 * ROW + t2) + p2;
+      float2* q = sm + EL * (k2 * ROW + t2) + p2;
       const float4* g = gsm + t2 * K::GS;
       const unsigned my = (v & 1) ? 0x80000000u : 0u;
       cv<float> s[3][R2];
@@ -200,21 +193,22 @@ k_fft_z_reg(OpView<float> op, float2* __restrict__ buf, int R, int per,
       for (int c = 0; c < 3; ++c) {
 #pragma unroll
         for (int j = 0; j < R2; ++j) {
-          const float2 e = q[2 * (c * (R1 * ROW) + j * TILE)];
+          const float2 e = q[EL * (c * (R1 * ROW) + j * TILE)];
           s[c][j] = {e.x, e.y};
         }
         rdft<R2, false>(s[c]);
       }
-      // position j holds kz = 2 (k2 + R1 j) + p2: row kz of the octant below n,
-      // row L - kz (z reflected) above; for even R2 every j is on one side (kz = n
-      // sits on both)
-      const float4* glo = g + 2 * k2 + p2;
-      const float4* ghi = g + L - 2 * k2 - p2;
+      // position j holds kz = 2 (k2 + R1 j) + p2 (odd L: k2 + R1 j): row kz of the
+      // octant up to L / 2, row L - kz (z reflected) above; for even R2 every j is on
+      // one side (kz = n sits on both)
+      constexpr int KS = EO ? 2 : 1;
+      const float4* glo = g + KS * k2 + p2;
+      const float4* ghi = g + L - KS * k2 - p2;
       static_for<R2>([&](auto jc) {
         constexpr int j = decltype(jc)::value;
         constexpr bool mid = R2 % 2 == 1 && 2 * j + 1 == R2;
-        const bool fz = mid ? 2 * (k2 + R1 * j) + p2 > n : 2 * j >= R2;
-        const float4* gp = fz ? ghi - 2 * R1 * j : glo + 2 * R1 * j;
+        const bool fz = mid ? KS * (k2 + R1 * j) + p2 > L / 2 : 2 * j >= R2;
+        const float4* gp = fz ? ghi - KS * R1 * j : glo + KS * R1 * j;
         const float4 g0 = gp[0], g1 = gp[Hz], g2 = gp[2 * Hz];
         // odd components change sign under the reflection of an odd axis
         const cv<float> xx{g0.x, g0.y}, yy{g1.z, g1.w}, zz{g2.z, g2.w};
@@ -233,7 +227,7 @@ k_fft_z_reg(OpView<float> op, float2* __restrict__ buf, int R, int per,
         rdft<R2, true>(s[c]);
 #pragma unroll
         for (int j = 0; j < R2; ++j)
-          q[2 * (c * (R1 * ROW) + j * TILE)] = make_float2(s[c][j].re, s[c][j].im);
+          q[EL * (c * (R1 * ROW) + j * TILE)] = make_float2(s[c][j].re, s[c][j].im);
       }
     }
     __syncthreads();
@@ -242,45 +236,31 @@ k_fft_z_reg(OpView<float> op, float2* __restrict__ buf, int R, int per,
     // reads here what it wrote in step 1 and nobody else does, so the next pass's
     // step 1 needs no barrier
     if (c1 < 3) {
-      cv<f32p> a[R1];
-#pragma unroll
-      for (int k = 0; k < R1; ++k) {
-        const float4 q = own[k * ROW], w = tw[k * R2];
-        const cv<float> e = cvmulc(cv<float>{w.x, w.y}, cv<float>{q.x, q.y});
-        const cv<float> o = cvmulc(cv<float>{w.z, w.w}, cv<float>{q.z, q.w});
-        a[k] = {pk_make(e.re, o.re), pk_make(e.im, o.im)};
-      }
-      if (ASYNC && vn < vend) fetch(vn);  // lands while this step computes
-      rdft<R1, true>(a);
+      float2 y[NJ];
+      reg_step1_inv<R1, R2, EO>(own, EL * ROW, tw, y,
+                                [&]() { if (ASYNC && vn < vend) fetch(vn); });
       float2* dst = line(v);
-      static_for<R1>([&](auto jc) {
-        constexpr int j = decltype(jc)::value;
-        constexpr float cw = (float)cx_cos(j, 2 * R1), sw = (float)cx_sin(j, 2 * R1);
-        float re, im, ro, io;
-        pk_split(a[j].re, re, ro);
-        pk_split(a[j].im, im, io);
-        if (on1 && (j < R1 - 1 || last))
-          dst[(int64_t)j * R2 * plane] = make_float2(fmaf(cw, ro, fmaf(-sw, io, re)),
-                                                     fmaf(cw, io, fmaf(sw, ro, im)));
-      });
+#pragma unroll
+      for (int j = 0; j < NJ; ++j)
+        if (on1 && (j < NJ - 1 || last)) dst[(int64_t)j * R2 * plane] = y[j];
     }
     if (vn >= vend) return;
     v = vn;
   }
 }
 
-template <int R1, int R2> cudaError_t configure_z_reg() {
-  cudaError_t e = cudaFuncSetAttribute(k_fft_z_reg<R1, R2, false>,
+template <int R1, int R2, bool EO> cudaError_t configure_z_reg() {
+  cudaError_t e = cudaFuncSetAttribute(k_fft_z_reg<R1, R2, EO, false>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)ZRegCfg<R1, R2>::smem);
+                                       (int)ZRegCfg<R1, R2, EO>::smem);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_fft_z_reg<R1, R2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)ZRegCfg<R1, R2>::smem);
+    e = cudaFuncSetAttribute(k_fft_z_reg<R1, R2, EO, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)ZRegCfg<R1, R2, EO>::smem);
   return e;
 }
-template <int R1, int R2>
+template <int R1, int R2, bool EO>
 void launch_z_reg(const OpView<float>& op, int R, float2* buf, const int* active, cudaStream_t st) {
-  using K = ZRegCfg<R1, R2>;
+  using K = ZRegCfg<R1, R2, EO>;
   const int tiles = (op.Lx + K::TILE - 1) / K::TILE, hy = op.Ly / 2 + 1;
   // passes per CTA: as many as leave four waves of CTAs (more passes save Ghat
   // reads, fewer waves lose to the last one: 100x75x135, 2 RHS, 262 us with four
@@ -289,9 +269,9 @@ void launch_z_reg(const OpView<float>& op, int R, float2* buf, const int* active
   per = per < 1 ? 1 : per > 2 * R ? 2 * R : per;
   const dim3 g(tiles, hy, (unsigned)((2 * R + per - 1) / per));
   if (op.Lx % 2 == 0 && ((uintptr_t)buf & 15) == 0)
-    k_fft_z_reg<R1, R2, true><<<g, K::NT, K::smem, st>>>(op, buf, R, (int)per, active);
+    k_fft_z_reg<R1, R2, EO, true><<<g, K::NT, K::smem, st>>>(op, buf, R, (int)per, active);
   else
-    k_fft_z_reg<R1, R2, false><<<g, K::NT, K::smem, st>>>(op, buf, R, (int)per, active);
+    k_fft_z_reg<R1, R2, EO, false><<<g, K::NT, K::smem, st>>>(op, buf, R, (int)per, active);
 }
 
 // The plans, in parts that compile side by side (zpass_reg_*.cu): X(R1, R2).
@@ -308,20 +288,25 @@ void launch_z_reg(const OpView<float>& op, int R, float2* buf, const int* active
 #define DDA_ZREG_DECLARE(PART)                                                                 \
   bool launch_z_reg_part##PART(const OpView<float>& op, int R, float2* buf, const int* active, \
                                cudaStream_t st);                                               \
-  cudaError_t configure_z_reg_part##PART(int half);
+  cudaError_t configure_z_reg_part##PART(int L);
 DDA_ZREG_DECLARE(0) DDA_ZREG_DECLARE(1) DDA_ZREG_DECLARE(2)
 DDA_ZREG_DECLARE(3) DDA_ZREG_DECLARE(4) DDA_ZREG_DECLARE(5)
 
-#define DDA_ZREG_LAUNCH(A, B) case (A) * (B): launch_z_reg<A, B>(op, R, buf, active, st); return true;
-#define DDA_ZREG_CONFIG(A, B) case (A) * (B): return configure_z_reg<A, B>();
-#define DDA_ZREG_DEFINE(PART)                                                                  \
+#define DDA_ZREG_LAUNCH(A, B) \
+  case 2 * (A) * (B): launch_z_reg<A, B, true>(op, R, buf, active, st); return true;
+#define DDA_ZREG_CONFIG(A, B) case 2 * (A) * (B): return configure_z_reg<A, B, true>();
+#define DDA_ZREG_LAUNCH_ODD(A, B) \
+  case (A) * (B): launch_z_reg<A, B, false>(op, R, buf, active, st); return true;
+#define DDA_ZREG_CONFIG_ODD(A, B) case (A) * (B): return configure_z_reg<A, B, false>();
+// ODDS: the list of odd plans (DDA_XREG_ODD), or nothing
+#define DDA_ZREG_DEFINE(PART, ODDS)                                                            \
   bool launch_z_reg_part##PART(const OpView<float>& op, int R, float2* buf, const int* active, \
                                cudaStream_t st) {                                              \
-    switch (op.Lz / 2) { DDA_ZREG_PART##PART(DDA_ZREG_LAUNCH) }                                \
+    switch (op.Lz) { DDA_ZREG_PART##PART(DDA_ZREG_LAUNCH) ODDS(DDA_ZREG_LAUNCH_ODD) }          \
     return false;                                                                              \
   }                                                                                            \
-  cudaError_t configure_z_reg_part##PART(int half) {                                           \
-    switch (half) { DDA_ZREG_PART##PART(DDA_ZREG_CONFIG) }                                     \
+  cudaError_t configure_z_reg_part##PART(int L) {                                              \
+    switch (L) { DDA_ZREG_PART##PART(DDA_ZREG_CONFIG) ODDS(DDA_ZREG_CONFIG_ODD) }              \
     return cudaSuccess;                                                                        \
   }
 

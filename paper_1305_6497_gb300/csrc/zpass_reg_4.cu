@@ -2,5 +2,5 @@
 #include "zpass_reg.cuh"
 
 namespace dda {
-DDA_ZREG_DEFINE(4)
+DDA_ZREG_DEFINE(4, DDA_REG_NONE)
 }  // namespace dda

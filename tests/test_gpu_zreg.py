@@ -16,7 +16,10 @@ pytestmark = pytest.mark.gpu
 SHAPES = [(2, 3, 9), (3, 5, 11), (13, 8, 12), (8, 13, 16), (14, 9, 26), (9, 11, 32), (10, 7, 33),
           (7, 10, 64), (13, 6, 76), (5, 9, 96), (12, 5, 97), (6, 7, 128), (3, 9, 129),
           (10, 4, 144), (5, 6, 168), (13, 4, 162), (4, 6, 200), (5, 4, 216), (4, 5, 225),
-          (6, 4, 251), (5, 5, 256)]
+          (6, 4, 251), (5, 5, 256),
+          # odd z lengths 15 .. 225, both ends of their boxes, with and without copies
+          (9, 3, 7), (7, 5, 8), (13, 4, 13), (10, 3, 14), (9, 5, 21), (14, 4, 23), (6, 7, 37),
+          (37, 3, 38), (11, 9, 41), (5, 4, 65), (13, 3, 68), (9, 4, 109), (3, 5, 113)]
 
 
 @pytest.mark.parametrize("shape", SHAPES)
@@ -54,13 +57,17 @@ X_SHAPES = [(9, 3, 2), (10, 5, 3), (11, 4, 5), (15, 7, 3), (17, 5, 4), (26, 3, 5
             (33, 6, 3), (42, 3, 4), (51, 4, 3), (64, 7, 5), (73, 3, 2), (82, 5, 3), (91, 2, 5),
             (101, 3, 4), (114, 4, 3), (126, 3, 5), (129, 5, 2), (136, 3, 3), (145, 2, 4),
             (151, 3, 3), (161, 3, 2), (168, 2, 3), (189, 3, 3), (193, 2, 2), (204, 3, 2),
-            (217, 2, 3), (226, 3, 2), (251, 2, 3), (256, 3, 3)]
+            (217, 2, 3), (226, 3, 2), (251, 2, 3), (256, 3, 3),
+            (7, 5, 3), (8, 3, 2), (13, 4, 5), (14, 3, 3), (21, 5, 2), (23, 3, 4), (37, 4, 3),
+            (38, 3, 5), (41, 7, 3), (65, 3, 2), (68, 2, 3), (109, 3, 3), (113, 2, 2)]
 
 
 @pytest.mark.parametrize("nx,ny", [(3, 9), (2, 10), (9, 11), (5, 16), (17, 26), (9, 33),
                                    (4, 64), (5, 73), (9, 82), (3, 101), (17, 128), (3, 129),
                                    (5, 136), (2, 145), (9, 150), (3, 168), (2, 189), (5, 193),
-                                   (9, 204), (2, 225), (3, 240), (9, 251), (2, 256)])
+                                   (9, 204), (2, 225), (3, 240), (9, 251), (2, 256),
+                                   (3, 7), (17, 8), (2, 13), (9, 14), (5, 21), (4, 23), (9, 37),
+                                   (2, 38), (17, 41), (3, 65), (9, 68), (2, 109), (5, 113)])
 def test_register_y_passes_match(nx, ny):
     """Column tiles with one column, a partial tile and several tiles."""
     from paper_1305_6497_gb300 import binding as B
@@ -131,7 +138,7 @@ def test_batches_and_frozen_right_hand_sides():
 
 def test_register_z_kernel_is_refused_where_it_has_no_plan():
     from paper_1305_6497_gb300 import binding as B
-    for nz in (13, 125, 165):      # odd Lz, no two-factor plan, two rows beyond the box
+    for nz in (5, 125, 165):       # no two-factor plan, two rows beyond the box
         occ, comp = tg.rect_prism(4, 3, nz)
         t = B.Target(occ, comp, [1.5 + 0.1j], method="CM")
         x = np.ones((t.num_dipoles, 3), np.complex128)
