@@ -201,13 +201,13 @@ struct Workspace {
   // FP32
   DevBuf x32, r32, rh32, p32, v32, s32, t32, scr32, b32;
   DevBuf partials, ks, active, active_outer, norms, sums;
-  DevBuf pol, ph, ainv64, ainv32, ainvdf, wabs, fph, sitebuf;
+  DevBuf pol, ph, ainv64, ainv32, ainvdf, wabs, fph, fdir, sitebuf;
   DevBuf extra64, extra32;  // extra Krylov vectors of BiCGstab(2), GPBi-CG (on first use)
   DevBuf fold;              // per-RHS block counters of the passes that end a scalar step
   template <class F> void each(F f) {
     for (DevBuf* b : {&b64, &x64, &r64, &rh64, &p64, &v64, &s64, &t64, &scr64, &x32, &r32,
                       &rh32, &p32, &v32, &s32, &t32, &scr32, &b32, &partials, &ks, &active,
-                      &active_outer, &norms, &sums, &pol, &ph, &ainv64, &ainv32, &ainvdf, &wabs, &fph,
+                      &active_outer, &norms, &sums, &pol, &ph, &ainv64, &ainv32, &ainvdf, &wabs, &fph, &fdir,
                       &extra64, &extra32, &fold,
                       &sitebuf})
       f(*b);
@@ -1294,11 +1294,11 @@ static int64_t workspace_bytes(const dda_target* t, int R, dda_precision prec, i
   const int nblk = std::max(reduce_blocks(3 * t->nbox), 3 * t->nz * t->ny);
   // Krylov partials [R][nblk][<= 8]; far field, one incidence at a time:
   // [2][ndir+1][fblk][6]
-  const int fblk = std::min(reduce_blocks(t->nbox), 304);
+  const int fblk = farfield_blocks(t->nx, t->ny, t->nz, ndir + 1);
   b += std::max((int64_t)8 * R * nblk, (int64_t)12 * (ndir + 1) * fblk) * 8;
   b += (int64_t)R * (sizeof(KState) + 64) + (int64_t)R * (t->nx + t->ny + t->nz + 8) * 16;
   b += (int64_t)fold_bytes(R);  // scalar-step counters and group sums
-  b += (int64_t)(ndir + 1) * (t->nx + t->ny + t->nz) * 16 + t->N * (int64_t)R * 48;
+  b += (int64_t)(ndir + 1) * ((t->nx + t->ny + t->nz) * 16 + 24) + t->N * (int64_t)R * 48;
   return b;
 }
 
@@ -1324,7 +1324,7 @@ static void ensure_workspace(dda_target* t, int R, dda_precision prec, int ndir)
   const int nblk = std::max({reduce_blocks(3 * t->nbox), (rows + t->L32.x_lines - 1) / t->L32.x_lines,
                              (rows + t->L64.x_lines - 1) / t->L64.x_lines,
                              t->L32.x_reg ? x_reg_blocks(t->Lx, rows) : 1});
-  const int fblk = std::min(reduce_blocks(t->nbox), 304);
+  const int fblk = farfield_blocks(t->nx, t->ny, t->nz, ndir + 1);
   w.partials.ensure((size_t)std::max((int64_t)8 * R * nblk, (int64_t)12 * (ndir + 1) * fblk) * 8);
   w.ks.ensure(sizeof(KState) * R);
   w.active.ensure(sizeof(int) * R);
@@ -1338,6 +1338,7 @@ static void ensure_workspace(dda_target* t, int R, dda_precision prec, int ndir)
   w.ainvdf.ensure(sizeof(df64c) * (size_t)R * (t->ncomp + 1) * 3);
   w.wabs.ensure(sizeof(double) * (size_t)R * (t->ncomp + 1) * 3);
   w.fph.ensure(sizeof(double2) * (size_t)(ndir + 1) * (t->nx + t->ny + t->nz));
+  w.fdir.ensure(sizeof(double) * 3 * (size_t)(ndir + 1));
   w.sitebuf.ensure(sizeof(double2) * 3 * (size_t)t->N * R);
   w.R = R;
 }
@@ -1792,7 +1793,7 @@ dda_status dda_solve(dda_target* t, const dda_solve_params* p, dda_solve_result*
     // ---- per-RHS tables ----
     const int nc1 = t->ncomp + 1;
     // alpha^{-1} tables [R][ncomp+1][3]: one entry per lattice axis
-    std::vector<double2> pol(3 * R), ph, ai(3 * R * nc1), fph;
+    std::vector<double2> pol(3 * R), ph, ai(3 * R * nc1);
     std::vector<float2> ai32(3 * R * nc1);
     std::vector<double> wabs(3 * R * nc1, 0.0);
     const double k3 = kd * kd * kd;
@@ -1987,10 +1988,9 @@ dda_status dda_solve(dda_target* t, const dda_solve_params* p, dda_solve_result*
     std::vector<double> ff;
     if (res->famp) {
       ff.resize((size_t)p->n_inc * D * p->npol * 6);
-      const int fblk = std::min(reduce_blocks(nbox), 304);
+      const int fblk = farfield_blocks(t->nx, t->ny, t->nz, D);
+      std::vector<double> fdir(3 * (size_t)D);
       for (int i = 0; i < p->n_inc; ++i) {
-        fph.clear();
-        std::vector<double2> fx, fy, fz;
         const double* x = incs[i].khat;
         const double* y = incs[i].yhat;
         const double zz[3] = {x[1] * y[2] - x[2] * y[1], x[2] * y[0] - x[0] * y[2],
@@ -1998,25 +1998,20 @@ dda_status dda_solve(dda_target* t, const dda_solve_params* p, dda_solve_result*
         for (int d = 0; d < D; ++d) {
           const double th = d == 0 ? 0.0 : p->dirs[2 * (d - 1)];
           const double phi = d == 0 ? 0.0 : p->dirs[2 * (d - 1) + 1];
-          double nv[3];
           for (int c = 0; c < 3; ++c)
-            nv[c] = x[c] * std::cos(th) + y[c] * std::sin(th) * std::cos(phi) +
-                    zz[c] * std::sin(th) * std::sin(phi);
-          axis_phase(t->nx, kd, nv[0], -1.0, fx);
-          axis_phase(t->ny, kd, nv[1], -1.0, fy);
-          axis_phase(t->nz, kd, nv[2], -1.0, fz);
+            fdir[3 * (size_t)d + c] = x[c] * std::cos(th) + y[c] * std::sin(th) * std::cos(phi) +
+                                      zz[c] * std::sin(th) * std::sin(phi);
         }
-        fph.insert(fph.end(), fx.begin(), fx.end());
-        fph.insert(fph.end(), fy.begin(), fy.end());
-        fph.insert(fph.end(), fz.begin(), fz.end());
-        CK(cudaMemcpyAsync(w.fph.p, fph.data(), sizeof(double2) * fph.size(),
+        CK(cudaMemcpyAsync(w.fdir.p, fdir.data(), sizeof(double) * fdir.size(),
                            cudaMemcpyHostToDevice, st));
+        CK(launch_direction_phases(t->nx, t->ny, t->nz, D, kd, w.fdir.as<double>(),
+                                   w.fph.as<double2>(), st));
         const double2* dfx = w.fph.as<double2>();
         const double2* dfy = dfx + (size_t)D * t->nx;
         const double2* dfz = dfy + (size_t)D * t->ny;
         const double2* Pi = w.x64.as<double2>() + (size_t)i * p->npol * n;
         CK(launch_farfield(t->nx, t->ny, t->nz, t->comp.as<uint8_t>(), p->npol, D, Pi, dfx,
-                           dfy, dfz, part, fblk, st));
+                           dfy, dfz, part, st));
         CK(launch_finalize_sums(p->npol * D, fblk, 6, part, w.sums.as<double>(), st));
         CK(cudaMemcpyAsync(ff.data() + (size_t)i * D * p->npol * 6, w.sums.p,
                            sizeof(double) * D * p->npol * 6, cudaMemcpyDeviceToHost, st));

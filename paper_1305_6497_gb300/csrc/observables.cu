@@ -56,46 +56,157 @@ cudaError_t launch_cross_sections(int nx, int ny, int nz, const uint8_t* comp, R
   return cudaGetLastError();
 }
 
-// grid: (nblk, R, D); partials [(d*R + r)*nblk + blk][6]
-__global__ void k_farfield(int nx, int ny, int nz, const uint8_t* __restrict__ comp,
-                           const double2* __restrict__ P, const double2* __restrict__ fphx,
-                           const double2* __restrict__ fphy, const double2* __restrict__ fphz,
-                           double* partials, int d0) {
-  const int r = blockIdx.y, d = d0 + (int)blockIdx.z, R = gridDim.y;
-  const int64_t nbox = (int64_t)nx * ny * nz;
-  double acc[6] = {0, 0, 0, 0, 0, 0};
-  GRID_LOOP(i, nbox) {
-    if (comp[i]) {
-      const int ix = (int)(i % nx);
-      const int64_t q = i / nx;
-      const int iy = (int)(q % ny), iz = (int)(q / ny);
-      const double2 ph = cmul(cmul(fphx[(int64_t)d * nx + ix], fphy[(int64_t)d * ny + iy]),
-                              fphz[(int64_t)d * nz + iz]);
+// Phase tables exp(-i kd n_a (i - (n_a^box - 1) / 2)) of D directions n (dirs [D][3]) on the
+// three axes: [D][nx], then [D][ny], then [D][nz].
+__global__ void k_direction_phases(int nx, int ny, int nz, int D, double kd,
+                                   const double* __restrict__ dirs, double2* __restrict__ ph) {
+  const int per = nx + ny + nz;
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < D * per; e += gridDim.x * blockDim.x) {
+    const int d = e / per, q = e - d * per;
+    const int a = q < nx ? 0 : q < nx + ny ? 1 : 2;
+    const int n = a == 0 ? nx : a == 1 ? ny : nz;
+    const int i = a == 0 ? q : a == 1 ? q - nx : q - nx - ny;
+    double sn, cs;
+    sincos(-kd * dirs[3 * d + a] * (i - 0.5 * (n - 1)), &sn, &cs);
+    ph[(a == 0 ? (int64_t)d * nx : a == 1 ? (int64_t)D * nx + (int64_t)d * ny
+                                          : (int64_t)D * (nx + ny) + (int64_t)d * nz) + i] =
+        make_double2(cs, sn);
+  }
+}
+
+cudaError_t launch_direction_phases(int nx, int ny, int nz, int D, double kd, const double* dirs,
+                                    double2* ph, cudaStream_t st) {
+  const int64_t n = (int64_t)D * (nx + ny + nz);
+  const int blocks = (int)std::min<int64_t>((n + 127) / 128, 152 * 8);
+  k_direction_phases<<<blocks, 128, 0, st>>>(nx, ny, nz, D, kd, dirs, ph);
+  note_launch();
+  return cudaGetLastError();
+}
+
+// Far field of R right-hand sides (the polarizations of an incidence) in D directions.
+// A thread holds one lattice column (x, y) and DC directions: over its z it sums
+// ez_d(z) P, 12 FP64 multiply-adds a site, direction and polarization with a phase
+// that is the same for every thread, and only then multiplies by ex_d(x) ey_d(y) and
+// joins the block's sum.  P is read once for DC directions and every polarization;
+// warps skip planes where none of their sites is occupied.
+//
+// What bounds it: FP64 arithmetic.  A phase per site and direction (a thread per site,
+// two complex products a site) took 20 instructions for each polarization, and the
+// tables came from the host: 350 scattering directions of each orientation of the
+// 48x96x144 ellipsoid took 83 ms of a 222 ms orientation average, now 29 of 167.
+//
+// grid: (column blocks x z chunks, direction chunks); partials [(d R + r) nblk + blk][6]
+template <int DC, int R>
+__global__ void __launch_bounds__(kThreads)
+k_farfield(int nx, int ny, int nz, int cols, int zper, int D, const uint8_t* __restrict__ comp,
+           const double2* __restrict__ P, const double2* __restrict__ fphx,
+           const double2* __restrict__ fphy, const double2* __restrict__ fphz,
+           double* __restrict__ partials) {
+  const int cb = blockIdx.x % cols, zc = blockIdx.x / cols, d0 = blockIdx.y * DC;
+  const int64_t nxy = (int64_t)nx * ny, nbox = nxy * nz;
+  const int64_t col = (int64_t)cb * kThreads + threadIdx.x;
+  const bool in = col < nxy;
+  double2 acc[DC][R][3];
+#pragma unroll
+  for (int d = 0; d < DC; ++d)
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) acc[d][r][c] = make_double2(0.0, 0.0);
+  const int z1 = min(nz, (zc + 1) * zper);
+  for (int z = zc * zper; z < z1; ++z) {
+    const bool occ = in && comp[z * nxy + col];
+    if (!__any_sync(0xffffffffu, occ)) continue;
+    double2 p[R][3];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int c = 0; c < 3; ++c)  // vacant sites hold zeros
+        p[r][c] = in ? P[((int64_t)r * 3 + c) * nbox + z * nxy + col] : make_double2(0.0, 0.0);
+#pragma unroll
+    for (int d = 0; d < DC; ++d) {
+      const double2 e = __ldg(fphz + (int64_t)min(d0 + d, D - 1) * nz + z);
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          double2& a = acc[d][r][c];
+          a.x = fma(p[r][c].x, e.x, fma(-p[r][c].y, e.y, a.x));
+          a.y = fma(p[r][c].x, e.y, fma(p[r][c].y, e.x, a.y));
+        }
+    }
+  }
+  const int ix = in ? (int)(col % nx) : 0, iy = in ? (int)(col / nx) : 0;
+#pragma unroll
+  for (int d = 0; d < DC; ++d) {
+    if (d0 + d >= D) break;
+    const double2 xy = cmul(fphx[(int64_t)(d0 + d) * nx + ix], fphy[(int64_t)(d0 + d) * ny + iy]);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      double v[6], tot[6];
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        const double2 t = cmul(P[((int64_t)r * 3 + c) * nbox + i], ph);
-        acc[2 * c] += t.x;
-        acc[2 * c + 1] += t.y;
+        const double2 t = cmul(acc[d][r][c], xy);
+        v[2 * c] = t.x;
+        v[2 * c + 1] = t.y;
+      }
+      block_sum<6>(v, tot);
+      if (threadIdx.x == 0) {
+        double* o = partials + (((int64_t)(d0 + d) * R + r) * gridDim.x + blockIdx.x) * 6;
+#pragma unroll
+        for (int i = 0; i < 6; ++i) o[i] = tot[i];
       }
     }
   }
-  double tot[6];
-  block_sum<6>(acc, tot);
-  if (threadIdx.x == 0) {
-    double* o = partials + (((int64_t)d * R + r) * gridDim.x + blockIdx.x) * 6;
-#pragma unroll
-    for (int i = 0; i < 6; ++i) o[i] = tot[i];
-  }
+}
+
+// Directions per thread: the accumulators of four directions and two polarizations
+// take 96 registers; fewer where that wastes less of the last chunk.  z chunks: only
+// as many as about four blocks per SM need (every chunk closes with a block sum of
+// its own, which costs as much as ten planes), of two planes or more.
+static void farfield_grid(int nx, int ny, int nz, int D, int& dc, int& cols, int& zchunks) {
+  dc = 4;
+  for (int c : {3, 2, 1})
+    if ((D + c - 1) / c * c < (D + dc - 1) / dc * dc) dc = c;
+  cols = (int)(((int64_t)nx * ny + kThreads - 1) / kThreads);
+  const int64_t blocks = (int64_t)cols * ((D + dc - 1) / dc);
+  zchunks = (int)std::max<int64_t>(1, std::min<int64_t>((608 + blocks - 1) / blocks, (nz + 1) / 2));
+  const int per = (nz + zchunks - 1) / zchunks;
+  zchunks = (nz + per - 1) / per;
+}
+
+int farfield_blocks(int nx, int ny, int nz, int D) {
+  int dc, cols, zchunks;
+  farfield_grid(nx, ny, nz, D, dc, cols, zchunks);
+  return cols * zchunks;
 }
 
 cudaError_t launch_farfield(int nx, int ny, int nz, const uint8_t* comp, int R, int D,
                             const double2* P, const double2* fphx, const double2* fphy,
-                            const double2* fphz, double* partials, int nblk,
-                            cudaStream_t st) {
-  // grid.z is limited to 65535 directions per launch
-  for (int d0 = 0; d0 < D; d0 += 65535) {
-    dim3 g(nblk, R, std::min(65535, D - d0));
-    k_farfield<<<g, kThreads, 0, st>>>(nx, ny, nz, comp, P, fphx, fphy, fphz, partials, d0);
+                            const double2* fphz, double* partials, cudaStream_t st) {
+  int dc, cols, zchunks;
+  farfield_grid(nx, ny, nz, D, dc, cols, zchunks);
+  const int zper = (nz + zchunks - 1) / zchunks;
+  for (int c0 = 0; c0 < (D + dc - 1) / dc; c0 += 65535) {  // grid.y limit
+    const int d0 = c0 * dc, n = std::min(D - d0, 65535 * dc);
+    const dim3 g(cols * zchunks, (n + dc - 1) / dc);
+#define DDA_FAR(DC, RR)                                                                      \
+  k_farfield<DC, RR><<<g, kThreads, 0, st>>>(nx, ny, nz, cols, zper, n, comp, P,             \
+                                             fphx + (int64_t)d0 * nx, fphy + (int64_t)d0 * ny, \
+                                             fphz + (int64_t)d0 * nz,                        \
+                                             partials + (int64_t)d0 * R * cols * zchunks * 6)
+    if (R == 1) {
+      if (dc == 4) DDA_FAR(4, 1);
+      else if (dc == 3) DDA_FAR(3, 1);
+      else if (dc == 2) DDA_FAR(2, 1);
+      else DDA_FAR(1, 1);
+    } else {
+      if (dc == 4) DDA_FAR(4, 2);
+      else if (dc == 3) DDA_FAR(3, 2);
+      else if (dc == 2) DDA_FAR(2, 2);
+      else DDA_FAR(1, 2);
+    }
+#undef DDA_FAR
     note_launch();
   }
   return cudaGetLastError();
