@@ -120,18 +120,38 @@ static std::vector<int> factor_radices(int L) {
   return r;
 }
 
+// The roots exp(-2 pi i k / L), k < L, in long double: every twiddle of an axis is one
+// of them, so a new target evaluates L cosines and sines per axis instead of one per
+// table entry (about 5 L, in software on hosts whose long double has 128 bits).
+struct Roots {
+  int L;
+  std::vector<long double> re, im;
+  explicit Roots(int n) : L(n), re(n), im(n) {
+    const long double two_pi = 6.283185307179586476925286766559L;
+    for (int k = 0; k < n; ++k) {
+      // k/n of a turn as q quarters and a remainder of at most an eighth either way
+      const int q = (int)((4LL * k + n / 2) / n);
+      const long double a = two_pi * ((long double)k - (long double)q * n / 4) / n;
+      const long double c = cosl(a), s = sinl(a);
+      const long double cs[4] = {c, -s, -c, s}, sn[4] = {s, c, -s, -c};
+      re[k] = cs[q & 3];
+      im[k] = -sn[q & 3];
+    }
+  }
+};
+
 // In-place plan: stage t has radix rs[t], block B_t = L / (rs[0]...rs[t-1]) and
 // twiddles exp(-2 pi i j m / B_t), j < B_t/rs[t], m = 1..rs[t]-1.  Also returns
 // which frequency ends up at each position after the forward (decimation in
 // frequency) transform: position sum_t m_t S_t holds sum_t m_t N_t with
 // S_t = B_t/rs[t] and N_t = rs[0]...rs[t-1].
-static AxisPlan make_plan_radices(int L, const std::vector<int>& rs,
+static AxisPlan make_plan_radices(const Roots& root, const std::vector<int>& rs,
                                   std::vector<long double>& twr, std::vector<long double>& twi,
                                   std::vector<int>& k_at);
 
-static AxisPlan make_plan(int L, std::vector<long double>& twr, std::vector<long double>& twi,
-                          std::vector<int>& k_at) {
-  return make_plan_radices(L, factor_radices(L), twr, twi, k_at);
+static AxisPlan make_plan(const Roots& root, std::vector<long double>& twr,
+                          std::vector<long double>& twi, std::vector<int>& k_at) {
+  return make_plan_radices(root, factor_radices(root.L), twr, twi, k_at);
 }
 
 // The radix plan the column-pair z kernel compiles for a z length (radices of
@@ -146,15 +166,15 @@ static std::vector<int> pair_plan_radices(int L) {
   }
 }
 
-static AxisPlan make_plan_radices(int L, const std::vector<int>& rs,
+static AxisPlan make_plan_radices(const Roots& root, const std::vector<int>& rs,
                                   std::vector<long double>& twr, std::vector<long double>& twi,
                                   std::vector<int>& k_at) {
   AxisPlan P{};
+  const int L = root.L;
   P.L = L;
   P.nstage = (int)rs.size();
   int B = L, off = 0;
   twr.clear(); twi.clear();
-  const long double two_pi = 6.283185307179586476925286766559L;
   std::vector<int> S(P.nstage), Nt(P.nstage);
   int nprod = 1;
   for (int t = 0; t < P.nstage; ++t) {
@@ -166,10 +186,9 @@ static AxisPlan make_plan_radices(int L, const std::vector<int>& rs,
     P.sdiv[t] = ((1ull << 36) + (unsigned long long)Sp - 1) / (unsigned long long)Sp;
     for (int j = 0; j < Sp; ++j)
       for (int m = 1; m < R; ++m) {
-        const long long num = ((long long)j * m) % (long long)B;
-        const long double ang = -two_pi * (long double)num / (long double)B;
-        twr.push_back(cosl(ang));
-        twi.push_back(sinl(ang));
+        const int k = (int)(((long long)j * m) % B) * (L / B);  // B divides L
+        twr.push_back(root.re[k]);
+        twi.push_back(root.im[k]);
       }
     off += Sp * (R - 1);
     S[t] = Sp;
@@ -605,6 +624,38 @@ static int run_device_loop(dda_target* t, int slot, const std::vector<uintptr_t>
   return blocks;
 }
 
+// The CUDA graph of one block of iterations (enqueue() queues it), for the blocks that
+// the host launches one by one: profiled solves.  Captured on first use, so that a
+// solve in one device-side loop never builds it (a new target's first solve saved
+// about 0.5 ms of capture and instantiation).
+template <class ENQ>
+static IterGraph& iter_graph(dda_target* t, int slot, const std::vector<uintptr_t>& sig,
+                             const ENQ& enqueue) {
+  cudaStream_t st = t->stream;
+  IterGraph& g = t->graphs[slot];
+  if (g.exec && g.sig != sig) g.reset();
+  if (g.exec) return g;
+  const long long before = launch_count();
+  CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
+  try {
+    enqueue();
+  } catch (...) {
+    cudaGraph_t broken = nullptr;
+    cudaStreamEndCapture(st, &broken);  // leave capture mode before reporting
+    if (broken) cudaGraphDestroy(broken);
+    throw;
+  }
+  cudaGraph_t graph = nullptr;
+  CK(cudaStreamEndCapture(st, &graph));
+  const cudaError_t ie = cudaGraphInstantiate(&g.exec, graph, 0);
+  cudaGraphDestroy(graph);
+  CK(ie);
+  g.kernels = launch_count() - before;
+  note_launches(-g.kernels);  // captured, not run
+  g.sig = sig;
+  return g;
+}
+
 // ---------------------------------------------------------------------------
 // BiCGSTAB driver, R RHS in lockstep on the device.  Returns the number of
 // iterations per RHS through `its` and the status per RHS.
@@ -661,8 +712,8 @@ static void bicgstab(dda_target* t, const OpView<T>& op, const MatvecLaunch& L, 
       CK(launch_update_xr<T>(n, R, V.x, V.r, V.p, V.s, V.t, V.rh, part, ks, act, st, fr));
     }
   };
-  // A full block is captured once into a CUDA graph and replayed; the graph is
-  // rebuilt only when a pointer, the batch size or the profiling mode changes.
+  // The graphs are rebuilt only when a pointer, the batch size or the profiling mode
+  // changes.
   std::vector<uintptr_t> sig = {(uintptr_t)sizeof(T), (uintptr_t)R, (uintptr_t)t->prof.on,
                                 (uintptr_t)V.r, (uintptr_t)V.p, (uintptr_t)V.v,
                                 (uintptr_t)V.rh, (uintptr_t)V.s, (uintptr_t)V.t,
@@ -670,28 +721,6 @@ static void bicgstab(dda_target* t, const OpView<T>& op, const MatvecLaunch& L, 
                                 (uintptr_t)part, (uintptr_t)act, (uintptr_t)op.ghat,
                                 (uintptr_t)op.ainv, (uintptr_t)nblk_mv, (uintptr_t)nblk,
                                 (uintptr_t)cnt, (uintptr_t)t->schedule_gen};
-  IterGraph& g = t->graphs[sizeof(T) == 4 ? 0 : 1];
-  if (g.exec && g.sig != sig) g.reset();
-  if (!g.exec) {
-    const long long before = launch_count();
-    CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-    try {
-      enqueue_block(kCheckEvery);
-    } catch (...) {
-      cudaGraph_t broken = nullptr;
-      cudaStreamEndCapture(st, &broken);  // leave capture mode before reporting
-      if (broken) cudaGraphDestroy(broken);
-      throw;
-    }
-    cudaGraph_t graph = nullptr;
-    CK(cudaStreamEndCapture(st, &graph));
-    const cudaError_t ie = cudaGraphInstantiate(&g.exec, graph, 0);
-    cudaGraphDestroy(graph);
-    CK(ie);
-    g.kernels = launch_count() - before;
-    note_launches(-g.kernels);  // captured, not run
-    g.sig = sig;
-  }
   // without per-pass profiling the full blocks run as one device-side loop
   // (a single graph launch); the host loop below then only runs a remainder
   // shorter than a block, or every block when profiling
@@ -710,6 +739,8 @@ static void bicgstab(dda_target* t, const OpView<T>& op, const MatvecLaunch& L, 
     // on the device by its active flag, so the extra iterations cost nothing
     const int nq = std::min(kCheckEvery, max_iter - iter);
     if (nq == kCheckEvery) {
+      IterGraph& g = iter_graph(t, sizeof(T) == 4 ? 0 : 1, sig,
+                                [&]() { enqueue_block(kCheckEvery); });
       CK(cudaGraphLaunch(g.exec, st));
       note_launches(g.kernels);
     } else {
@@ -792,28 +823,6 @@ static void qmr(dda_target* t, const OpView<T>& op, const MatvecLaunch& L, int R
                                 (uintptr_t)part, (uintptr_t)act, (uintptr_t)op.ghat,
                                 (uintptr_t)op.ainv, (uintptr_t)nblk_mv, (uintptr_t)nblk,
                                 (uintptr_t)cnt, (uintptr_t)t->schedule_gen};
-  IterGraph& g = t->graphs[sizeof(T) == 4 ? 0 : 1];
-  if (g.exec && g.sig != sig) g.reset();
-  if (!g.exec) {
-    const long long before = launch_count();
-    CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-    try {
-      enqueue_block(kCheckEvery);
-    } catch (...) {
-      cudaGraph_t broken = nullptr;
-      cudaStreamEndCapture(st, &broken);
-      if (broken) cudaGraphDestroy(broken);
-      throw;
-    }
-    cudaGraph_t graph = nullptr;
-    CK(cudaStreamEndCapture(st, &graph));
-    const cudaError_t ie = cudaGraphInstantiate(&g.exec, graph, 0);
-    cudaGraphDestroy(graph);
-    CK(ie);
-    g.kernels = launch_count() - before;
-    note_launches(-g.kernels);
-    g.sig = sig;
-  }
   // without per-pass profiling the full blocks run as one device-side loop
   // (a single graph launch); the host loop below then only runs a remainder
   // shorter than a block, or every block when profiling
@@ -830,6 +839,8 @@ static void qmr(dda_target* t, const OpView<T>& op, const MatvecLaunch& L, int R
   while (nact > 0 && iter < max_iter) {
     const int nq = std::min(kCheckEvery, max_iter - iter);
     if (nq == kCheckEvery) {
+      IterGraph& g = iter_graph(t, sizeof(T) == 4 ? 0 : 1, sig,
+                                [&]() { enqueue_block(kCheckEvery); });
       CK(cudaGraphLaunch(g.exec, st));
       note_launches(g.kernels);
     } else {
@@ -927,28 +938,6 @@ static void bicgstab2(dda_target* t, const OpView<T>& op, const MatvecLaunch& L,
                                 (uintptr_t)act, (uintptr_t)op.ghat, (uintptr_t)op.ainv,
                                 (uintptr_t)nblk_mv, (uintptr_t)nblk,
                                 (uintptr_t)t->schedule_gen};
-  IterGraph& g = t->graphs[sizeof(T) == 4 ? 0 : 1];
-  if (g.exec && g.sig != sig) g.reset();
-  if (!g.exec) {
-    const long long before = launch_count();
-    CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-    try {
-      enqueue_block(kCycles);
-    } catch (...) {
-      cudaGraph_t broken = nullptr;
-      cudaStreamEndCapture(st, &broken);
-      if (broken) cudaGraphDestroy(broken);
-      throw;
-    }
-    cudaGraph_t graph = nullptr;
-    CK(cudaStreamEndCapture(st, &graph));
-    const cudaError_t ie = cudaGraphInstantiate(&g.exec, graph, 0);
-    cudaGraphDestroy(graph);
-    CK(ie);
-    g.kernels = launch_count() - before;
-    note_launches(-g.kernels);
-    g.sig = sig;
-  }
   int iter = 0;
   if (!t->prof.on && nact > 0) {
     std::vector<uintptr_t> wsig = sig;
@@ -961,6 +950,8 @@ static void bicgstab2(dda_target* t, const OpView<T>& op, const MatvecLaunch& L,
     for (int a : hact) nact += a;
   }
   while (nact > 0 && iter < max_iter) {
+    IterGraph& g = iter_graph(t, sizeof(T) == 4 ? 0 : 1, sig,
+                              [&]() { enqueue_block(kCycles); });
     CK(cudaGraphLaunch(g.exec, st));
     note_launches(g.kernels);
     CK(cudaMemcpyAsync(hact.data(), act, sizeof(int) * R, cudaMemcpyDeviceToHost, st));
@@ -982,9 +973,9 @@ static void bicgstab2(dda_target* t, const OpView<T>& op, const MatvecLaunch& L,
   }
 }
 
-// Runs one block of iterations as a CUDA graph (captured on first use, rebuilt
-// when `sig` changes) until every RHS is frozen on the device.  `per_block`
-// iterations of `nmv` matvecs each are enqueued by `enqueue`.
+// Runs blocks of iterations (see run_device_loop and iter_graph) until every RHS is
+// frozen on the device.  `per_block` iterations of `nmv` matvecs each are enqueued by
+// `enqueue`.
 template <typename T, class ENQ>
 static void run_graph_loop(dda_target* t, const std::vector<uintptr_t>& sig, int per_block,
                            int nmv, int max_iter, int nact, std::vector<int>& hact,
@@ -992,28 +983,6 @@ static void run_graph_loop(dda_target* t, const std::vector<uintptr_t>& sig, int
   cudaStream_t st = t->stream;
   int* act = t->ws.active.as<int>();
   const int R = (int)hact.size();
-  IterGraph& g = t->graphs[sizeof(T) == 4 ? 0 : 1];
-  if (g.exec && g.sig != sig) g.reset();
-  if (!g.exec) {
-    const long long before = launch_count();
-    CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-    try {
-      enqueue();
-    } catch (...) {
-      cudaGraph_t broken = nullptr;
-      cudaStreamEndCapture(st, &broken);
-      if (broken) cudaGraphDestroy(broken);
-      throw;
-    }
-    cudaGraph_t graph = nullptr;
-    CK(cudaStreamEndCapture(st, &graph));
-    const cudaError_t ie = cudaGraphInstantiate(&g.exec, graph, 0);
-    cudaGraphDestroy(graph);
-    CK(ie);
-    g.kernels = launch_count() - before;
-    note_launches(-g.kernels);
-    g.sig = sig;
-  }
   int iter = 0;
   if (!t->prof.on && nact > 0) {
     std::vector<uintptr_t> wsig = sig;
@@ -1025,6 +994,7 @@ static void run_graph_loop(dda_target* t, const std::vector<uintptr_t>& sig, int
     for (int a : hact) nact += a;
   }
   while (nact > 0 && iter < max_iter) {
+    IterGraph& g = iter_graph(t, sizeof(T) == 4 ? 0 : 1, sig, enqueue);
     CK(cudaGraphLaunch(g.exec, st));
     note_launches(g.kernels);
     CK(cudaMemcpyAsync(hact.data(), act, sizeof(int) * R, cudaMemcpyDeviceToHost, st));
@@ -1478,10 +1448,11 @@ dda_status dda_target_create(int nx, int ny, int nz, const uint8_t* occ, const u
     const int Ls[3] = {t->Lx, t->Ly, t->Lz};
     AxisPlan* ps[3] = {&t->px, &t->py, &t->pz};
     std::vector<int> posall;
+    const Roots roots[3] = {Roots(t->Lx), Roots(t->Ly), Roots(t->Lz)};
     for (int a = 0; a < 3; ++a) {
       std::vector<long double> wr, wi;
       std::vector<int> ka;
-      *ps[a] = make_plan(Ls[a], wr, wi, ka);
+      *ps[a] = make_plan(roots[a], wr, wi, ka);
       std::vector<int> pa(Ls[a]);
       for (int q = 0; q < Ls[a]; ++q) pa[ka[q]] = q;
       kat.insert(kat.end(), ka.begin(), ka.end());
@@ -1517,7 +1488,7 @@ dda_status dda_target_create(int nx, int ny, int nz, const uint8_t* occ, const u
     if (!prs.empty()) {
       std::vector<long double> wr, wi;
       std::vector<int> ka;
-      make_plan_radices(t->Lz, prs, wr, wi, ka);
+      make_plan_radices(roots[2], prs, wr, wi, ka);
       std::vector<float2> tp(std::max<size_t>(1, wr.size()), make_float2(1, 0));
       for (size_t i = 0; i < wr.size(); ++i) tp[i] = make_float2((float)wr[i], (float)wi[i]);
       t->twzp.ensure(sizeof(float2) * tp.size());
@@ -1526,21 +1497,22 @@ dda_status dda_target_create(int nx, int ny, int nz, const uint8_t* occ, const u
     // and of the register passes, [k1 < R1][j2 < R2]: w_L^(j2 (2 k1 + parity)), both
     // parities side by side (re, im even; re, im odd), or w_L^(j2 k1) for odd L
     std::vector<float4> tr;
-    auto reg_twiddles = [&](int axis, int L, int r1, int r2) {
-      const long double two_pi = 6.283185307179586476925286766559L;
+    auto reg_twiddles = [&](int axis, int r1, int r2) {
+      const Roots& w = roots[axis];
+      const int L = w.L;
       t->twroff[axis] = (int)tr.size();
       for (int k = 0; k < r1; ++k)
         for (int j = 0; j < r2; ++j) {
           const long long even = L % 2 ? (long long)j * k : 2LL * j * k;
-          const long double a = -two_pi * (long double)(even % L) / L;
-          const long double b = -two_pi * (long double)(((2LL * k + 1) * j) % L) / L;
-          tr.push_back(make_float4((float)cosl(a), (float)sinl(a), (float)cosl(b), (float)sinl(b)));
+          const int a = (int)(even % L), b = (int)(((2LL * k + 1) * j) % L);
+          tr.push_back(make_float4((float)w.re[a], (float)w.im[a], (float)w.re[b],
+                                   (float)w.im[b]));
         }
     };
     int r1 = 0, r2 = 0;
-    if (x_reg_plan(t->Lx, t->nx, &r1, &r2)) reg_twiddles(0, t->Lx, r1, r2);
-    if (x_reg_plan(t->Ly, t->ny, &r1, &r2)) reg_twiddles(1, t->Ly, r1, r2);
-    if (z_reg_plan(t->Lz, t->nz, &r1, &r2)) reg_twiddles(2, t->Lz, r1, r2);
+    if (x_reg_plan(t->Lx, t->nx, &r1, &r2)) reg_twiddles(0, r1, r2);
+    if (x_reg_plan(t->Ly, t->ny, &r1, &r2)) reg_twiddles(1, r1, r2);
+    if (z_reg_plan(t->Lz, t->nz, &r1, &r2)) reg_twiddles(2, r1, r2);
     if (!tr.empty()) {
       t->twr.ensure(sizeof(float4) * tr.size());
       CK(cudaMemcpy(t->twr.p, tr.data(), sizeof(float4) * tr.size(), cudaMemcpyHostToDevice));
@@ -1549,12 +1521,11 @@ dda_status dda_target_create(int nx, int ny, int nz, const uint8_t* occ, const u
     if (z_wide_plan(t->Lz, t->nz, &r1, &r2)) {
       std::vector<float4> td;
       std::vector<double2> tq;
-      const long double two_pi = 6.283185307179586476925286766559L;
       for (int p = 0; p < 2; ++p)
         for (int k = 0; k < r1; ++k)
           for (int j = 0; j < r2; ++j) {
-            const long double a = -two_pi * (long double)(((2LL * k + p) * j) % t->Lz) / t->Lz;
-            const long double re = cosl(a), im = sinl(a);
+            const int a = (int)(((2LL * k + p) * j) % t->Lz);
+            const long double re = roots[2].re[a], im = roots[2].im[a];
             const float rh = (float)re, ih = (float)im;
             td.push_back(make_float4(rh, (float)(re - (long double)rh), ih,
                                      (float)(im - (long double)ih)));
