@@ -166,6 +166,8 @@ template <typename T> struct OpView {
   int Lx, Ly, Lz;                 // FFT grid
   int Hx, Hy, Hz;                 // octant sizes L/2 + 1
   int64_t nbox;                   // nx*ny*nz
+  int src_z0, src_z1;             // planes outside [src_z0, src_z1) of the input hold zeros:
+                                  // the FP64 x and y passes leave them out
   const uint8_t* comp;            // [nbox] 0 = vacant, else composition 1..ncomp
   const C* ghat;                  // octant, already divided by Lx*Ly*Lz: [Hz][Hy][Hx][6],
                                   // FP32 [Hy][Hx][3][Hz][2] (see ghat_f32_offset)

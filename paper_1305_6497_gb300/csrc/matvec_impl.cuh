@@ -74,6 +74,19 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) k_fft_x_fwd(OpVie
   const int row0 = blockIdx.x * nlines;
   const int ps = nlines + 1;
   const int64_t off = (int64_t)r * rows * nx;
+  if constexpr (std::is_same<T, double>::value && MODE == XIN_PLAIN) {
+    // near field: only the target's planes hold dipoles.  A CTA whose rows all lie in
+    // planes without has nothing to do (the y pass writes those planes); rows run
+    // through the planes of a component and on into the next one, so the first and
+    // last row's planes decide unless the rows pass a component's end
+    if (op.src_z1 - op.src_z0 < op.nz) {
+      const int q0 = row0 / op.ny, q1 = (min(row0 + nlines, rows) - 1) / op.ny;
+      const int z0 = q0 % op.nz, z1 = q1 % op.nz;
+      if (q0 / op.nz == q1 / op.nz ? z1 < op.src_z0 || z0 >= op.src_z1
+                                   : q1 - q0 < op.nz && z0 >= op.src_z1 && z1 < op.src_z0)
+        return;
+    }
+  }
   C c1 = mk<C>(0, 0), c2 = mk<C>(0, 0), c3 = mk<C>(0, 0);
   if constexpr (MODE == XIN_P) {
     C sc[2];
@@ -199,6 +212,16 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) k_fft_y(OpView<T>
   C* base = buf + ((int64_t)r * 3 * op.nz + blockIdx.y) * (int64_t)Ly * Lx + col0;
   ColIO<C> in{base, Lx, ncol, INV ? Ly : op.ny};
   ColIO<C> out{base, Lx, ncol, INV ? op.ny : Ly};
+  if constexpr (std::is_same<T, double>::value && !INV) {
+    const int z = blockIdx.y % op.nz;
+    if (z < op.src_z0 || z >= op.src_z1) {  // a plane of zeros (see k_fft_x_fwd)
+      for (int e = threadIdx.x; e < Ly * tile; e += blockDim.x) {
+        const int p = e / tile;
+        out(e - p * tile, p, mk<C>(0, 0));
+      }
+      return;
+    }
+  }
   if (op.py.nstage >= 2) {
     // ny of the Ly rows carry data (forward input, inverse output)
     const bool half = 2 * op.ny <= Ly;
