@@ -375,6 +375,7 @@ static OpView<T> make_view(const dda_target* t, const void* ghat, const void* ai
   v.Lx = t->Lx; v.Ly = t->Ly; v.Lz = t->Lz;
   v.Hx = t->Lx / 2 + 1; v.Hy = t->Ly / 2 + 1; v.Hz = t->Lz / 2 + 1;
   v.nbox = t->nbox;
+  v.chain = !t->prof.on;
   v.src_z0 = 0;
   v.src_z1 = t->nz;
   v.comp = t->comp.as<uint8_t>();
@@ -719,7 +720,8 @@ static void bicgstab(dda_target* t, const OpView<T>& op, const MatvecLaunch& L, 
       CK(launch_matvec_s<T>(op, L, R, V.r, V.v, V.s, V.t, V.scr, ks, part, act, st,
                             t->prof.iter_set(q, 1), fo));
       // x += alpha p + omega s; r = s - omega t; <rhat, r>, <r, r>
-      CK(launch_update_xr<T>(n, R, V.x, V.r, V.p, V.s, V.t, V.rh, part, ks, act, st, fr));
+      CK(launch_update_xr<T>(n, R, V.x, V.r, V.p, V.s, V.t, V.rh, part, ks, act, st, fr,
+                             op.chain != 0));
     }
   };
   // The graphs are rebuilt only when a pointer, the batch size or the profiling mode
@@ -824,7 +826,7 @@ static void qmr(dda_target* t, const OpView<T>& op, const MatvecLaunch& L, int R
       CK(launch_matvec_q<T>(op, L, R, V.r, q, d, V.x, V.t, V.scr, ks, part, act, st,
                             t->prof.iter_set(k, 0), fs));
       // r -= alpha t; ||r||^2, r^T r; rotation and the next pending update
-      CK(launch_qmr_update_r<T>(n, R, V.r, V.t, part, ks, act, st, fq));
+      CK(launch_qmr_update_r<T>(n, R, V.r, V.t, part, ks, act, st, fq, op.chain != 0));
     }
   };
   std::vector<uintptr_t> sig = {(uintptr_t)1000 + sizeof(T), (uintptr_t)R, (uintptr_t)t->prof.on,
@@ -907,6 +909,13 @@ static void bicgstab2(dda_target* t, const OpView<T>& op, const MatvecLaunch& L,
   }
   CK(launch_state_init(R, nblk, part, ks, act, tol, max_iter, st));
   CK(launch_bs2_scalar(6, R, nblk, part, ks, act, st));
+  // alpha is a step of the product before it (as in bicgstab)
+  w.fold.ensure(fold_bytes(R));
+  unsigned* cnt = w.fold.as<unsigned>();
+  double* gsum = reinterpret_cast<double*>(w.fold.as<char>() + fold_gsum_offset(R));
+  CK(cudaMemsetAsync(cnt, 0, fold_gsum_offset(R), st));
+  const FoldArgs fa{ks, act, cnt, FOLD_ALPHA, gsum};
+  const bool chain = op.chain != 0;
   std::vector<int> hact(R);
   CK(cudaMemcpyAsync(hact.data(), act, sizeof(int) * R, cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
@@ -915,30 +924,28 @@ static void bicgstab2(dda_target* t, const OpView<T>& op, const MatvecLaunch& L,
   const int nblk_mv = matvec_partial_blocks<T>(op, L);
   constexpr int kCycles = kCheckEvery / 2;  // two iterations per cycle
   auto vec = [&](int which) {
-    CK(launch_bs2_vec<T>(which, n, R, V.x, r0, r1, r2, u0, u1, u2, rt, part, ks, act, st));
+    CK(launch_bs2_vec<T>(which, n, R, V.x, r0, r1, r2, u0, u1, u2, rt, part, ks, act, st, chain));
   };
   auto enqueue_block = [&](int ncyc) {
     for (int c = 0; c < ncyc; ++c) {
-      CK(launch_bs2_scalar(0, R, nblk, part, ks, act, st));          // beta, rho0
+      CK(launch_bs2_scalar(0, R, nblk, part, ks, act, st, chain));   // beta, rho0
       vec(0);                                                        // u0 = r0 - beta u0
       CK(launch_matvec_rv<T>(op, L, R, u0, u1, rt, V.scr, part, act, st,
-                             t->prof.iter_set(2 * c, 0)));           // u1 = A u0
-      CK(launch_scalar_alpha(R, nblk_mv, part, ks, act, st));        // alpha
+                             t->prof.iter_set(2 * c, 0), fa));       // u1 = A u0; alpha
       vec(1);                                                        // r0 -= alpha u1
       CK(launch_matvec_rv<T>(op, L, R, r0, r1, rt, V.scr, part, act, st,
                              t->prof.iter_set(2 * c, 1)));           // r1 = A r0
-      CK(launch_bs2_scalar(2, R, nblk_mv, part, ks, act, st));      // beta, rho0
+      CK(launch_bs2_scalar(2, R, nblk_mv, part, ks, act, st, chain));  // beta, rho0
       vec(2);                                                        // x, u0, u1
       CK(launch_matvec_rv<T>(op, L, R, u1, u2, rt, V.scr, part, act, st,
-                             t->prof.iter_set(2 * c + 1, 0)));       // u2 = A u1
-      CK(launch_scalar_alpha(R, nblk_mv, part, ks, act, st));        // alpha
+                             t->prof.iter_set(2 * c + 1, 0), fa));   // u2 = A u1; alpha
       vec(3);                                                        // r0, r1, x
-      CK(launch_matvec<T>(op, L, R, r1, r2, V.scr, act, st,
+      CK(launch_matvec<T>(follows_kernel(op), L, R, r1, r2, V.scr, act, st,
                           t->prof.iter_set(2 * c + 1, 1)));          // r2 = A r1
       vec(4);                                                        // Gram partials
-      CK(launch_bs2_scalar(4, R, nblk, part, ks, act, st));          // g1, g2, omega
+      CK(launch_bs2_scalar(4, R, nblk, part, ks, act, st, chain));   // g1, g2, omega
       vec(5);                                                        // MR update
-      CK(launch_bs2_scalar(5, R, nblk, part, ks, act, st));          // convergence
+      CK(launch_bs2_scalar(5, R, nblk, part, ks, act, st, chain));   // convergence
     }
   };
   std::vector<uintptr_t> sig = {(uintptr_t)2000 + sizeof(T), (uintptr_t)R, (uintptr_t)t->prof.on,
@@ -946,7 +953,7 @@ static void bicgstab2(dda_target* t, const OpView<T>& op, const MatvecLaunch& L,
                                 (uintptr_t)u2, (uintptr_t)r1, (uintptr_t)r2, (uintptr_t)V.x,
                                 (uintptr_t)V.scr, (uintptr_t)ks, (uintptr_t)part,
                                 (uintptr_t)act, (uintptr_t)op.ghat, (uintptr_t)op.ainv,
-                                (uintptr_t)nblk_mv, (uintptr_t)nblk,
+                                (uintptr_t)nblk_mv, (uintptr_t)nblk, (uintptr_t)cnt,
                                 (uintptr_t)t->schedule_gen};
   int iter = 0;
   if (!t->prof.on && nact > 0) {

@@ -36,10 +36,13 @@ template <typename C> __device__ __forceinline__ C d2c(double2 a) { return mk<C>
 
 // u0 = r0 - beta u0
 template <typename T>
-__global__ void k_bs2_a(int64_t n, const cplx_t<T>* __restrict__ r0, cplx_t<T>* __restrict__ u0,
-                        const KState* __restrict__ ks, const int* __restrict__ active) {
+__global__ void k_bs2_a(int64_t n, const cplx_t<T>* r0, cplx_t<T>* u0,
+                        const KState* ks, const int* active) {
   using C = cplx_t<T>;
   const int rr = blockIdx.y;
+  chain_next();
+  chain_wait();
+  r0 = chained(r0); u0 = chained(u0); ks = chained(ks); active = chained(active);
   if (!active[rr]) return;
   C sc[1];
   block_scalars<C, 1>({ks[rr].beta}, sc);
@@ -50,10 +53,13 @@ __global__ void k_bs2_a(int64_t n, const cplx_t<T>* __restrict__ r0, cplx_t<T>* 
 
 // r0 = r0 - alpha u1
 template <typename T>
-__global__ void k_bs2_b(int64_t n, cplx_t<T>* __restrict__ r0, const cplx_t<T>* __restrict__ u1,
-                        const KState* __restrict__ ks, const int* __restrict__ active) {
+__global__ void k_bs2_b(int64_t n, cplx_t<T>* r0, const cplx_t<T>* u1,
+                        const KState* ks, const int* active) {
   using C = cplx_t<T>;
   const int rr = blockIdx.y;
+  chain_next();
+  chain_wait();
+  r0 = chained(r0); u1 = chained(u1); ks = chained(ks); active = chained(active);
   if (!active[rr]) return;
   C sc[1];
   block_scalars<C, 1>({ks[rr].alpha}, sc);
@@ -64,12 +70,16 @@ __global__ void k_bs2_b(int64_t n, cplx_t<T>* __restrict__ r0, const cplx_t<T>* 
 
 // x += alpha u0 (alpha of j = 0); u0 = r0 - beta u0; u1 = r1 - beta u1
 template <typename T>
-__global__ void k_bs2_c(int64_t n, cplx_t<T>* __restrict__ x, const cplx_t<T>* __restrict__ r0,
-                        const cplx_t<T>* __restrict__ r1, cplx_t<T>* __restrict__ u0,
-                        cplx_t<T>* __restrict__ u1, const KState* __restrict__ ks,
-                        const int* __restrict__ active) {
+__global__ void k_bs2_c(int64_t n, cplx_t<T>* x, const cplx_t<T>* r0,
+                        const cplx_t<T>* r1, cplx_t<T>* u0,
+                        cplx_t<T>* u1, const KState* ks,
+                        const int* active) {
   using C = cplx_t<T>;
   const int rr = blockIdx.y;
+  chain_next();
+  chain_wait();
+  x = chained(x); r0 = chained(r0); r1 = chained(r1); u0 = chained(u0); u1 = chained(u1);
+  ks = chained(ks); active = chained(active);
   if (!active[rr]) return;
   C sc[2];
   block_scalars<C, 2>({ks[rr].alpha, ks[rr].beta}, sc);
@@ -77,21 +87,25 @@ __global__ void k_bs2_c(int64_t n, cplx_t<T>* __restrict__ x, const cplx_t<T>* _
   const int64_t off = (int64_t)rr * n;
   GRID_LOOP(i, n) {
     const int64_t g = off + i;
-    const C a0 = u0[g];
-    x[g] = cadd(x[g], cmul(alpha, a0));
-    u0[g] = csub(r0[g], cmul(beta, a0));
-    u1[g] = csub(r1[g], cmul(beta, u1[g]));
+    const C a0 = u0[g], a1 = u1[g], b0 = r0[g], b1 = r1[g], xv = x[g];
+    x[g] = cadd(xv, cmul(alpha, a0));
+    u0[g] = csub(b0, cmul(beta, a0));
+    u1[g] = csub(b1, cmul(beta, a1));
   }
 }
 
 // r0 -= alpha u1; r1 -= alpha u2; x += alpha u0
 template <typename T>
-__global__ void k_bs2_d(int64_t n, cplx_t<T>* __restrict__ x, cplx_t<T>* __restrict__ r0,
-                        cplx_t<T>* __restrict__ r1, const cplx_t<T>* __restrict__ u0,
-                        const cplx_t<T>* __restrict__ u1, const cplx_t<T>* __restrict__ u2,
-                        const KState* __restrict__ ks, const int* __restrict__ active) {
+__global__ void k_bs2_d(int64_t n, cplx_t<T>* x, cplx_t<T>* r0,
+                        cplx_t<T>* r1, const cplx_t<T>* u0,
+                        const cplx_t<T>* u1, const cplx_t<T>* u2,
+                        const KState* ks, const int* active) {
   using C = cplx_t<T>;
   const int rr = blockIdx.y;
+  chain_next();
+  chain_wait();
+  x = chained(x); r0 = chained(r0); r1 = chained(r1); u0 = chained(u0); u1 = chained(u1);
+  u2 = chained(u2); ks = chained(ks); active = chained(active);
   if (!active[rr]) return;
   C sc[1];
   block_scalars<C, 1>({ks[rr].alpha}, sc);
@@ -99,19 +113,24 @@ __global__ void k_bs2_d(int64_t n, cplx_t<T>* __restrict__ x, cplx_t<T>* __restr
   const int64_t off = (int64_t)rr * n;
   GRID_LOOP(i, n) {
     const int64_t g = off + i;
-    r0[g] = csub(r0[g], cmul(alpha, u1[g]));
-    r1[g] = csub(r1[g], cmul(alpha, u2[g]));
-    x[g] = cadd(x[g], cmul(alpha, u0[g]));
+    const C a0 = u0[g], a1 = u1[g], a2 = u2[g], b0 = r0[g], b1 = r1[g], xv = x[g];
+    r0[g] = csub(b0, cmul(alpha, a1));
+    r1[g] = csub(b1, cmul(alpha, a2));
+    x[g] = cadd(xv, cmul(alpha, a0));
   }
 }
 
 // Gram entries: ||r1||^2, ||r2||^2, <r1, r2>, <r1, r0>, <r2, r0>  ([R][nblk][8])
 template <typename T>
-__global__ void k_bs2_gram(int64_t n, const cplx_t<T>* __restrict__ r0,
-                           const cplx_t<T>* __restrict__ r1, const cplx_t<T>* __restrict__ r2,
-                           double* partials, const int* __restrict__ active) {
+__global__ void k_bs2_gram(int64_t n, const cplx_t<T>* r0,
+                           const cplx_t<T>* r1, const cplx_t<T>* r2,
+                           double* partials, const int* active) {
   using C = cplx_t<T>;
   const int rr = blockIdx.y;
+  chain_next();
+  chain_wait();
+  r0 = chained(r0); r1 = chained(r1); r2 = chained(r2); partials = chained(partials);
+  active = chained(active);
   if (!active[rr]) return;
   const int64_t off = (int64_t)rr * n;
   ChunkAcc<T, 8> acc;
@@ -133,14 +152,19 @@ __global__ void k_bs2_gram(int64_t n, const cplx_t<T>* __restrict__ r0,
 // minimal-residual update: u0 -= g1 u1 + g2 u2; x += g1 r0 + g2 r1;
 // r0 -= g1 r1 + g2 r2; partials <rt, r0>, ||r0||^2  ([R][nblk][4])
 template <typename T>
-__global__ void k_bs2_e(int64_t n, cplx_t<T>* __restrict__ x, cplx_t<T>* __restrict__ r0,
-                        const cplx_t<T>* __restrict__ r1, const cplx_t<T>* __restrict__ r2,
-                        cplx_t<T>* __restrict__ u0, const cplx_t<T>* __restrict__ u1,
-                        const cplx_t<T>* __restrict__ u2, const cplx_t<T>* __restrict__ rt,
-                        double* partials, const KState* __restrict__ ks,
-                        const int* __restrict__ active) {
+__global__ void k_bs2_e(int64_t n, cplx_t<T>* x, cplx_t<T>* r0,
+                        const cplx_t<T>* r1, const cplx_t<T>* r2,
+                        cplx_t<T>* u0, const cplx_t<T>* u1,
+                        const cplx_t<T>* u2, const cplx_t<T>* rt,
+                        double* partials, const KState* ks,
+                        const int* active) {
   using C = cplx_t<T>;
   const int rr = blockIdx.y;
+  chain_next();
+  chain_wait();
+  x = chained(x); r0 = chained(r0); r1 = chained(r1); r2 = chained(r2); u0 = chained(u0);
+  u1 = chained(u1); u2 = chained(u2); rt = chained(rt); partials = chained(partials);
+  ks = chained(ks); active = chained(active);
   if (!active[rr]) return;
   C sc[2];
   block_scalars<C, 2>({ks[rr].qa1, ks[rr].qa2}, sc);
@@ -149,13 +173,12 @@ __global__ void k_bs2_e(int64_t n, cplx_t<T>* __restrict__ x, cplx_t<T>* __restr
   ChunkAcc<T, 4> acc;
   GRID_LOOP(i, n) {
     const int64_t g = off + i;
-    const C a1 = r1[g];
-    u0[g] = csub(u0[g], cadd(cmul(g1, u1[g]), cmul(g2, u2[g])));
-    const C a0 = r0[g];
-    x[g] = cadd(x[g], cadd(cmul(g1, a0), cmul(g2, a1)));
-    const C rn = csub(a0, cadd(cmul(g1, a1), cmul(g2, r2[g])));
+    const C a0 = r0[g], a1 = r1[g], a2 = r2[g], b0 = u0[g], b1 = u1[g], b2 = u2[g];
+    const C xv = x[g], h = rt[g];
+    u0[g] = csub(b0, cadd(cmul(g1, b1), cmul(g2, b2)));
+    x[g] = cadd(xv, cadd(cmul(g1, a0), cmul(g2, a1)));
+    const C rn = csub(a0, cadd(cmul(g1, a1), cmul(g2, a2)));
     r0[g] = rn;
-    const C h = rt[g];
     acc.add(0, h.x * rn.x + h.y * rn.y);
     acc.add(1, h.x * rn.y - h.y * rn.x);
     acc.add(2, rn.x * rn.x + rn.y * rn.y);
@@ -175,6 +198,9 @@ __global__ void k_bs2_e(int64_t n, cplx_t<T>* __restrict__ x, cplx_t<T>* __restr
 __global__ void k_bs2_scalar(int phase, int nblk, const double* partials, KState* ks,
                              int* active) {
   const int r = blockIdx.x;
+  chain_next();
+  chain_wait();
+  partials = chained(partials); ks = chained(ks); active = chained(active);
   if (!active[r]) return;
   double tot[8];
   if (phase == 2) {
@@ -244,35 +270,37 @@ template <typename T>
 cudaError_t launch_bs2_vec(int which, int64_t n, int R, cplx_t<T>* x, cplx_t<T>* r0,
                            cplx_t<T>* r1, cplx_t<T>* r2, cplx_t<T>* u0, cplx_t<T>* u1,
                            cplx_t<T>* u2, const cplx_t<T>* rt, double* partials,
-                           const KState* ks, const int* active, cudaStream_t st) {
+                           const KState* ks, const int* active, cudaStream_t st, bool chain) {
   dim3 g(reduce_blocks(n), R);
+  auto run = [&](auto kernel, auto... a) {
+    launch_chained(chain, kernel, g, kThreads, 0, st, n, a...);
+  };
   switch (which) {
-    case 0: k_bs2_a<T><<<g, kThreads, 0, st>>>(n, r0, u0, ks, active); break;
-    case 1: k_bs2_b<T><<<g, kThreads, 0, st>>>(n, r0, u1, ks, active); break;
-    case 2: k_bs2_c<T><<<g, kThreads, 0, st>>>(n, x, r0, r1, u0, u1, ks, active); break;
-    case 3: k_bs2_d<T><<<g, kThreads, 0, st>>>(n, x, r0, r1, u0, u1, u2, ks, active); break;
-    case 4: k_bs2_gram<T><<<g, kThreads, 0, st>>>(n, r0, r1, r2, partials, active); break;
+    case 0: run(k_bs2_a<T>, r0, u0, ks, active); break;
+    case 1: run(k_bs2_b<T>, r0, u1, ks, active); break;
+    case 2: run(k_bs2_c<T>, x, r0, r1, u0, u1, ks, active); break;
+    case 3: run(k_bs2_d<T>, x, r0, r1, u0, u1, u2, ks, active); break;
+    case 4: run(k_bs2_gram<T>, r0, r1, r2, partials, active); break;
     default:
-      k_bs2_e<T><<<g, kThreads, 0, st>>>(n, x, r0, r1, r2, u0, u1, u2, rt, partials, ks,
-                                          active);
+      run(k_bs2_e<T>, x, r0, r1, r2, u0, u1, u2, rt, partials, ks, active);
   }
   note_launch();
   return cudaGetLastError();
 }
 
 cudaError_t launch_bs2_scalar(int phase, int R, int nblk, const double* partials, KState* ks,
-                              int* active, cudaStream_t st) {
-  k_bs2_scalar<<<R, kThreads, 0, st>>>(phase, nblk, partials, ks, active);
+                              int* active, cudaStream_t st, bool chain) {
+  launch_chained(chain, k_bs2_scalar, dim3(R), kThreads, 0, st, phase, nblk, partials, ks, active);
   note_launch();
   return cudaGetLastError();
 }
 
 template cudaError_t launch_bs2_vec<float>(int, int64_t, int, float2*, float2*, float2*, float2*,
                                            float2*, float2*, float2*, const float2*, double*,
-                                           const KState*, const int*, cudaStream_t);
+                                           const KState*, const int*, cudaStream_t, bool);
 template cudaError_t launch_bs2_vec<double>(int, int64_t, int, double2*, double2*, double2*,
                                             double2*, double2*, double2*, double2*,
                                             const double2*, double*, const KState*, const int*,
-                                            cudaStream_t);
+                                            cudaStream_t, bool);
 
 }  // namespace dda

@@ -166,6 +166,9 @@ template <typename T> struct OpView {
   int Lx, Ly, Lz;                 // FFT grid
   int Hx, Hy, Hz;                 // octant sizes L/2 + 1
   int64_t nbox;                   // nx*ny*nz
+  int chain;                      // host, see launch_chained: 0 -- ordinary launches; 1 --
+                                  // the passes of a product are chained; 2 -- and so is
+                                  // its first pass, which a kernel precedes
   int src_z0, src_z1;             // planes outside [src_z0, src_z1) of the input hold zeros:
                                   // the FP64 x and y passes leave them out
   const uint8_t* comp;            // [nbox] 0 = vacant, else composition 1..ncomp
@@ -187,6 +190,52 @@ template <typename T> struct OpView {
   unsigned long long div_nx, div_ny, div_nz, div_Lx;     // fast_div magics
   AxisPlan px, py, pz;
 };
+
+// ---- launches that overlap their predecessor's end ---------------------------
+// The passes of a product and the vector updates between them form one chain of short
+// kernels (8 to 50 us on boxes of up to 50^3 sites), each of which reads what the one
+// before it wrote.  launch_chained lets a kernel's CTAs become resident as soon as the
+// last CTAs of its predecessor have started: launch latency, index arithmetic and loads
+// of constant tables pass beside the predecessor's end.  The kernel calls
+//   chain_next()  first: its own successor may be set up;
+//   chain_wait()  in every CTA, before it touches anything a kernel of the chain
+//                 writes (and before it returns: a kernel that ends without waiting
+//                 would end before its predecessor has);
+//   chained(p)    on each pointer to such memory: the compiler knows nothing of p from
+//                 before the wait, so no load through it is moved above the wait or
+//                 takes the read-only path.
+// Ordinary and chained, one GB300: an FP32 product of 16^3 sites 38.5 and 32 us, of
+// 75x60x50 77 and 70; in the graph of a solve, whose launches are closer together, 64^3
+// 18.05 and 17.5 ms, 36x41x36 6.09 and 5.88.  The FP64 and double-float passes are not
+// chained: the 16^3 FP64 solve took 1.56 ms ordinary and 1.73 chained (their CTAs are
+// few and large, and those that wait hold the registers of those that work).
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <class P> __device__ __forceinline__ P* chained(P* p) {
+  asm volatile("" : "+l"(p)::"memory");
+  return p;
+}
+// A view for the products inside an iteration, which a kernel precedes.
+template <typename V> V follows_kernel(V op) {
+  if (op.chain) op.chain = 2;
+  return op;
+}
+// on: false -- an ordinary launch (profiled solves record an event between the passes)
+template <class... K, class... A>
+inline void launch_chained(bool on, void (*kernel)(K...), dim3 grid, int threads, size_t smem,
+                           cudaStream_t st, A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = dim3(threads);
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  c.attrs = &at;
+  c.numAttrs = on ? 1 : 0;
+  cudaLaunchKernelEx(&c, kernel, K(args)...);
+}
 
 // ---- asynchronous global -> shared copies (cp.async) ------------------------
 __device__ __forceinline__ unsigned smem_addr(const void* p) {

@@ -210,7 +210,8 @@ template <typename T>
 cudaError_t launch_update_xr(int64_t n, int R, cplx_t<T>* x, cplx_t<T>* r,
                              const cplx_t<T>* p, const cplx_t<T>* s, const cplx_t<T>* t,
                              const cplx_t<T>* rhat, double* partials, const KState* ks,
-                             const int* active, cudaStream_t st, FoldArgs fold = FoldArgs());
+                             const int* active, cudaStream_t st, FoldArgs fold = FoldArgs(),
+                             bool chain = false);
 cudaError_t launch_scalar_rho(int R, int nblk, const double* partials, KState* ks,
                               int* active, cudaStream_t st);
 
@@ -235,7 +236,7 @@ cudaError_t launch_qmr_state(int R, int nblk, const double* partials, KState* ks
 template <typename T>
 cudaError_t launch_qmr_update_r(int64_t n, int R, cplx_t<T>* r, const cplx_t<T>* t,
                                 double* partials, const KState* ks, const int* active,
-                                cudaStream_t st, FoldArgs fold = FoldArgs());
+                                cudaStream_t st, FoldArgs fold = FoldArgs(), bool chain = false);
 template <typename T>
 cudaError_t launch_qmr_flush(int64_t n, int R, cplx_t<T>* x, cplx_t<T>* d,
                              const cplx_t<T>* q, const KState* ks, cudaStream_t st);
@@ -251,9 +252,10 @@ template <typename T>
 cudaError_t launch_bs2_vec(int which, int64_t n, int R, cplx_t<T>* x, cplx_t<T>* r0,
                            cplx_t<T>* r1, cplx_t<T>* r2, cplx_t<T>* u0, cplx_t<T>* u1,
                            cplx_t<T>* u2, const cplx_t<T>* rt, double* partials,
-                           const KState* ks, const int* active, cudaStream_t st);
+                           const KState* ks, const int* active, cudaStream_t st,
+                           bool chain = false);
 cudaError_t launch_bs2_scalar(int phase, int R, int nblk, const double* partials, KState* ks,
-                              int* active, cudaStream_t st);
+                              int* active, cudaStream_t st, bool chain = false);
 
 // GPBi-CG building blocks (gpbicg.cu), vectors of R RHS ([R][n] each).
 // launch_gp_vec `which`:
@@ -285,12 +287,14 @@ cudaError_t launch_cg_vec(int which, int64_t n, int R, cplx_t<T>* x, cplx_t<T>* 
 cudaError_t launch_cg_scalar(int phase, int R, int nblk, const double* partials, KState* ks,
                              int* active, cudaStream_t st);
 // y = A x with the epilogue partials <rhat, y> ([R][nblk][2], nblk =
-// matvec_partial_blocks): a plain input with the XOUT_RV epilogue.
+// matvec_partial_blocks) and, where given, the scalar step on them: a plain input with
+// the XOUT_RV epilogue, inside an iteration (a kernel precedes it).
 template <typename T>
 cudaError_t launch_matvec_rv(const OpView<T>& op, const MatvecLaunch& L, int R,
                              const cplx_t<T>* x, cplx_t<T>* y, const cplx_t<T>* rhat,
                              cplx_t<T>* scratch, double* partials, const int* active,
-                             cudaStream_t st, const cudaEvent_t* ev = nullptr);
+                             cudaStream_t st, const cudaEvent_t* ev = nullptr,
+                             FoldArgs fold = FoldArgs());
 
 // ---- refinement helpers -----------------------------------------------------
 // partials of ||v||^2 per RHS (FP64 vector)

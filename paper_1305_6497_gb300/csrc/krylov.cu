@@ -176,13 +176,17 @@ cudaError_t launch_scalar_alpha(int R, int nblk, const double* partials, KState*
 
 
 template <typename T>
-__global__ void k_update_xr(int64_t n, cplx_t<T>* __restrict__ x, cplx_t<T>* __restrict__ r,
-                            const cplx_t<T>* __restrict__ p, const cplx_t<T>* __restrict__ s,
-                            const cplx_t<T>* __restrict__ t, const cplx_t<T>* __restrict__ rhat,
-                            double* partials, const KState* __restrict__ ks,
-                            const int* __restrict__ active, FoldArgs fold) {
+__global__ void k_update_xr(int64_t n, cplx_t<T>* x, cplx_t<T>* r, const cplx_t<T>* p,
+                            const cplx_t<T>* s, const cplx_t<T>* t, const cplx_t<T>* rhat,
+                            double* partials, const KState* ks, const int* active,
+                            FoldArgs fold) {
   using C = cplx_t<T>;
   const int rr = blockIdx.y;
+  chain_next();
+  chain_wait();
+  x = chained(x); r = chained(r); p = chained(p); s = chained(s); t = chained(t);
+  rhat = chained(rhat); partials = chained(partials); ks = chained(ks); active = chained(active);
+  fold = chained(fold);
   if (!active[rr]) return;
   C sc[2];
   block_scalars<C, 2>({ks[rr].alpha, ks[rr].omega}, sc);
@@ -225,9 +229,10 @@ template <typename T>
 cudaError_t launch_update_xr(int64_t n, int R, cplx_t<T>* x, cplx_t<T>* r,
                              const cplx_t<T>* p, const cplx_t<T>* s, const cplx_t<T>* t,
                              const cplx_t<T>* rhat, double* partials, const KState* ks,
-                             const int* active, cudaStream_t st, FoldArgs fold) {
+                             const int* active, cudaStream_t st, FoldArgs fold, bool chain) {
   dim3 g(reduce_blocks(n), R);
-  k_update_xr<T><<<g, kThreads, 0, st>>>(n, x, r, p, s, t, rhat, partials, ks, active, fold);
+  launch_chained(chain, k_update_xr<T>, g, kThreads, 0, st, n, x, r, p, s, t, rhat, partials, ks,
+                 active, fold);
   note_launch();
   return cudaGetLastError();
 }
@@ -339,12 +344,15 @@ cudaError_t launch_qmr_state(int R, int nblk, const double* partials, KState* ks
 
 
 template <typename T>
-__global__ void k_qmr_update_r(int64_t n, cplx_t<T>* __restrict__ r,
-                               const cplx_t<T>* __restrict__ t, double* partials,
-                               const KState* __restrict__ ks, const int* __restrict__ active,
-                               FoldArgs fold) {
+__global__ void k_qmr_update_r(int64_t n, cplx_t<T>* r, const cplx_t<T>* t, double* partials,
+                               const KState* ks, const int* active, FoldArgs fold) {
   using C = cplx_t<T>;
   const int rr = blockIdx.y;
+  chain_next();
+  chain_wait();
+  r = chained(r); t = chained(t); partials = chained(partials);
+  ks = chained(ks); active = chained(active);
+  fold = chained(fold);
   if (!active[rr]) return;
   C sc[1];
   block_scalars<C, 1>({ks[rr].alpha}, sc);
@@ -380,9 +388,9 @@ __global__ void k_qmr_update_r(int64_t n, cplx_t<T>* __restrict__ r,
 template <typename T>
 cudaError_t launch_qmr_update_r(int64_t n, int R, cplx_t<T>* r, const cplx_t<T>* t,
                                 double* partials, const KState* ks, const int* active,
-                                cudaStream_t st, FoldArgs fold) {
+                                cudaStream_t st, FoldArgs fold, bool chain) {
   dim3 g(reduce_blocks(n), R);
-  k_qmr_update_r<T><<<g, kThreads, 0, st>>>(n, r, t, partials, ks, active, fold);
+  launch_chained(chain, k_qmr_update_r<T>, g, kThreads, 0, st, n, r, t, partials, ks, active, fold);
   note_launch();
   return cudaGetLastError();
 }
@@ -583,14 +591,14 @@ cudaError_t launch_box_to_sites(int64_t N, int64_t nbox, int R, const int64_t* s
   template cudaError_t launch_update_xr<T>(int64_t, int, cplx_t<T>*, cplx_t<T>*,             \
                                            const cplx_t<T>*, const cplx_t<T>*,               \
                                            const cplx_t<T>*, const cplx_t<T>*, double*,      \
-                                           const KState*, const int*, cudaStream_t,    \
-                                           FoldArgs);                                  \
+                                           const KState*, const int*, cudaStream_t,          \
+                                           FoldArgs, bool);                                  \
   template cudaError_t launch_qmr_init<T>(int64_t, int, const cplx_t<T>*, const cplx_t<T>*,  \
                                           cplx_t<T>*, cplx_t<T>*, cplx_t<T>*, double*,       \
                                           cudaStream_t);                                     \
   template cudaError_t launch_qmr_update_r<T>(int64_t, int, cplx_t<T>*, const cplx_t<T>*,    \
                                               double*, const KState*, const int*,            \
-                                              cudaStream_t, FoldArgs);                                 \
+                                              cudaStream_t, FoldArgs, bool);                 \
   template cudaError_t launch_qmr_flush<T>(int64_t, int, cplx_t<T>*, cplx_t<T>*,             \
                                            const cplx_t<T>*, const KState*, cudaStream_t);
 INST(float)

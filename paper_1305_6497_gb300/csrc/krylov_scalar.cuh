@@ -114,6 +114,14 @@ __device__ inline void step_qmr(const double* tot, KState& k, int* active_r) {
   k.rho = rho_new;
 }
 
+__device__ __forceinline__ FoldArgs chained(FoldArgs f) {
+  f.ks = chained(f.ks);
+  f.active = chained(f.active);
+  f.counter = chained(f.counter);
+  f.gsum = chained(f.gsum);
+  return f;
+}
+
 // Called by every thread of every block of a row after the block's NV partials
 // are written (by thread 0).  Two levels of tickets (see FoldArgs): the last
 // block of each group sums the group's partials in block order, the last group

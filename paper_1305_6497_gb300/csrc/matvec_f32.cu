@@ -28,6 +28,6 @@ template cudaError_t launch_matvec<float>(const OpView<float>&, const MatvecLaun
 
 template cudaError_t launch_matvec_rv<float>(const OpView<float>&, const MatvecLaunch&, int,
                                             const float2*, float2*, const float2*, float2*, double*,
-                                            const int*, cudaStream_t, const cudaEvent_t*);
+                                            const int*, cudaStream_t, const cudaEvent_t*, FoldArgs);
 
 }  // namespace dda

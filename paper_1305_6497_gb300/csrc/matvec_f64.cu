@@ -31,6 +31,6 @@ template cudaError_t launch_field<double>(const OpView<double>&, const MatvecLau
                                           bool);
 template cudaError_t launch_matvec_rv<double>(const OpView<double>&, const MatvecLaunch&, int,
                                             const double2*, double2*, const double2*, double2*, double*,
-                                            const int*, cudaStream_t, const cudaEvent_t*);
+                                            const int*, cudaStream_t, const cudaEvent_t*, FoldArgs);
 
 }  // namespace dda

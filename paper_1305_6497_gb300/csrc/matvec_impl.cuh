@@ -52,6 +52,10 @@ template <typename T> struct XinArgs {
   cplx_t<T>* x;
 };
 
+template <typename T> __device__ __forceinline__ XinArgs<T> chained(XinArgs<T> a) {
+  return {chained(a.r), chained(a.pv), chained(a.v), chained(a.ks), chained(a.d), chained(a.x)};
+}
+
 // P: void -- the radix plan is read at run time; a FixedPlan -- Lx and the
 // stages are compile-time constants (FP32, see fft_plan.cuh).
 template <class P> constexpr int plan_len() {
@@ -1199,7 +1203,7 @@ cudaError_t launch_matvec_p(const OpView<T>& op, const MatvecLaunch& L, int R,
                             double* partials, const int* active, cudaStream_t st,
                             const cudaEvent_t* ev, FoldArgs fold) {
   XinArgs<T> xa{r, p, v, ks};
-  return matvec_passes<T, XIN_P, XOUT_RV>(op, L, R, p, v, scratch, active, st, ev, xa, rhat,
+  return matvec_passes<T, XIN_P, XOUT_RV>(follows_kernel(op), L, R, p, v, scratch, active, st, ev, xa, rhat,
                                           partials, fold);
 }
 
@@ -1210,7 +1214,7 @@ cudaError_t launch_matvec_s(const OpView<T>& op, const MatvecLaunch& L, int R,
                             double* partials, const int* active, cudaStream_t st,
                             const cudaEvent_t* ev, FoldArgs fold) {
   XinArgs<T> xa{r, s_vec, v, ks};
-  return matvec_passes<T, XIN_S, XOUT_TS>(op, L, R, s_vec, t_vec, scratch, active, st, ev, xa,
+  return matvec_passes<T, XIN_S, XOUT_TS>(follows_kernel(op), L, R, s_vec, t_vec, scratch, active, st, ev, xa,
                                           nullptr, partials, fold);
 }
 
@@ -1218,9 +1222,9 @@ template <typename T>
 cudaError_t launch_matvec_rv(const OpView<T>& op, const MatvecLaunch& L, int R,
                              const cplx_t<T>* x, cplx_t<T>* y, const cplx_t<T>* rhat,
                              cplx_t<T>* scratch, double* partials, const int* active,
-                             cudaStream_t st, const cudaEvent_t* ev) {
-  return matvec_passes<T, XIN_PLAIN, XOUT_RV>(op, L, R, x, y, scratch, active, st, ev,
-                                              XinArgs<T>{}, rhat, partials);
+                             cudaStream_t st, const cudaEvent_t* ev, FoldArgs fold) {
+  return matvec_passes<T, XIN_PLAIN, XOUT_RV>(follows_kernel(op), L, R, x, y, scratch, active,
+                                              st, ev, XinArgs<T>{}, rhat, partials, fold);
 }
 
 template <typename T>
@@ -1230,7 +1234,7 @@ cudaError_t launch_matvec_q(const OpView<T>& op, const MatvecLaunch& L, int R,
                             double* partials, const int* active, cudaStream_t st,
                             const cudaEvent_t* ev, FoldArgs fold) {
   XinArgs<T> xa{r, q, nullptr, ks, d, x};
-  return matvec_passes<T, XIN_Q, XOUT_QT>(op, L, R, q, t_vec, scratch, active, st, ev, xa,
+  return matvec_passes<T, XIN_Q, XOUT_QT>(follows_kernel(op), L, R, q, t_vec, scratch, active, st, ev, xa,
                                           nullptr, partials, fold);
 }
 

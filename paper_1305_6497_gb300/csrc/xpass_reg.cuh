@@ -68,18 +68,24 @@ inline int x_reg_grid(int rows, int LW) {
 
 template <int R1, int R2, bool EO, int MODE>
 __global__ void __launch_bounds__(32 * kXRegWarps, XRegCfg<R1, R2, EO>::MINB)
-k_x_fwd_reg(OpView<float> op, const float2* __restrict__ in, float2* __restrict__ buf,
-            const int* __restrict__ active, XinArgs<float> xa) {
+k_x_fwd_reg(OpView<float> op, const float2* in, float2* buf, const int* active,
+            XinArgs<float> xa) {
   using K = XRegCfg<R1, R2, EO>;
   using C = float2;
   constexpr int NJ = K::NJ, NQ = K::NQ, EL = K::EL;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int r = blockIdx.y;
-  if (active && !active[r]) return;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   float2* sm = reinterpret_cast<float2*>(smem_raw) + wid * (EL * K::LW * K::LS);
   const int nx = op.nx, Lx = K::L;
   const int rows = 3 * op.nz * op.ny;
+  chain_next();
+  chain_wait();
+  active = chained(active);
+  in = chained(in);
+  buf = chained(buf);
+  xa = chained(xa);
+  if (active && !active[r]) return;
   C s1 = make_float2(0.f, 0.f), s2 = s1, s3 = s1;
   if constexpr (MODE == XIN_P) {
     C sc[2];
@@ -109,7 +115,7 @@ k_x_fwd_reg(OpView<float> op, const float2* __restrict__ in, float2* __restrict_
       C x[NJ];
       if constexpr (MODE == XIN_PLAIN) {
 #pragma unroll
-        for (int j = 0; j < NJ; ++j) x[j] = __ldg(in + g0 + (j < NJ - 1 || last ? R2 * j : 0));
+        for (int j = 0; j < NJ; ++j) x[j] = in[g0 + (j < NJ - 1 || last ? R2 * j : 0)];
       } else {
         C vb[NJ], vc[NJ], vd[NJ];
 #pragma unroll
@@ -167,9 +173,8 @@ k_x_fwd_reg(OpView<float> op, const float2* __restrict__ in, float2* __restrict_
 
 template <int R1, int R2, bool EO, int MODE>
 __global__ void __launch_bounds__(32 * kXRegWarps, XRegCfg<R1, R2, EO>::MINB)
-k_x_inv_reg(OpView<float> op, const float2* __restrict__ buf, const float2* __restrict__ xin,
-            float2* __restrict__ yout, const int* __restrict__ active,
-            const float2* __restrict__ rhat, double* __restrict__ partials, FoldArgs fold) {
+k_x_inv_reg(OpView<float> op, const float2* buf, const float2* xin, float2* yout,
+            const int* active, const float2* rhat, double* partials, FoldArgs fold) {
   using K = XRegCfg<R1, R2, EO>;
   using C = float2;
   constexpr int NJ = K::NJ, NQ = K::NQ, EL = K::EL;
@@ -177,11 +182,11 @@ k_x_inv_reg(OpView<float> op, const float2* __restrict__ buf, const float2* __re
   constexpr int kAiSmem = 24;
   __shared__ C sai[kAiSmem];
   const int r = blockIdx.y;
-  if (active && !active[r]) return;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   float2* sm = reinterpret_cast<float2*>(smem_raw) + wid * (EL * K::LW * K::LS);
   const int nx = op.nx, Lx = K::L;
   const int rows = 3 * op.nz * op.ny;
+  chain_next();
   const bool ai_smem = op.ncomp1 * 3 <= kAiSmem;
   const C* ai = op.ainv + (int64_t)r * op.ncomp1 * 3;
   if (ai_smem) {
@@ -189,6 +194,15 @@ k_x_inv_reg(OpView<float> op, const float2* __restrict__ buf, const float2* __re
     __syncthreads();
     ai = sai;
   }
+  chain_wait();
+  active = chained(active);
+  buf = chained(buf);
+  xin = chained(xin);
+  yout = chained(yout);
+  rhat = chained(rhat);
+  partials = chained(partials);
+  fold = chained(fold);
+  if (active && !active[r]) return;
   const int64_t off = (int64_t)r * rows * nx;
   const int64_t plane_sz = (int64_t)op.Ly * Lx;
   const C* src = buf + (int64_t)r * 3 * op.nz * plane_sz;
@@ -228,8 +242,8 @@ k_x_inv_reg(OpView<float> op, const float2* __restrict__ buf, const float2* __re
 #pragma unroll
       for (int j = 0; j < NJ; ++j) {
         const int o = j < NJ - 1 || last ? R2 * j : 0;
-        xv[j] = __ldg(xin + g0 + o);
-        if (MODE == XOUT_RV) hv[j] = __ldg(rhat + g0 + o);
+        xv[j] = xin[g0 + o];
+        if (MODE == XOUT_RV) hv[j] = rhat[g0 + o];
         cm[j] = __ldg(cmp + o);
       }
       C s[NJ];
@@ -272,7 +286,8 @@ void launch_x_fwd_reg(const OpView<float>& op, int R, const float2* x, float2* b
                       const int* active, XinArgs<float> xa, cudaStream_t st) {
   using K = XRegCfg<R1, R2, EO>;
   const dim3 g(x_reg_grid(3 * op.nz * op.ny, K::LW), R);
-  k_x_fwd_reg<R1, R2, EO, MODE><<<g, 32 * kXRegWarps, K::smem, st>>>(op, x, buf, active, xa);
+  launch_chained(op.chain == 2, k_x_fwd_reg<R1, R2, EO, MODE>, g, 32 * kXRegWarps, K::smem, st, op, x,
+                 buf, active, xa);
 }
 template <int R1, int R2, bool EO, int MODE>
 void launch_x_inv_reg(const OpView<float>& op, int R, const float2* buf, const float2* x, float2* y,
@@ -280,8 +295,8 @@ void launch_x_inv_reg(const OpView<float>& op, int R, const float2* buf, const f
                       FoldArgs fold) {
   using K = XRegCfg<R1, R2, EO>;
   const dim3 g(x_reg_grid(3 * op.nz * op.ny, K::LW), R);
-  k_x_inv_reg<R1, R2, EO, MODE><<<g, 32 * kXRegWarps, K::smem, st>>>(op, buf, x, y, active, rhat,
-                                                                partials, fold);
+  launch_chained(op.chain, k_x_inv_reg<R1, R2, EO, MODE>, g, 32 * kXRegWarps, K::smem, st, op, buf, x,
+                 y, active, rhat, partials, fold);
 }
 template <int R1, int R2, bool EO> cudaError_t configure_x_reg() {
   const void* k[] = {(const void*)k_x_fwd_reg<R1, R2, EO, XIN_PLAIN>, (const void*)k_x_fwd_reg<R1, R2, EO, XIN_P>,

@@ -37,12 +37,16 @@ template <int R1, int R2, bool EO = true> struct YRegCfg {
 
 template <int R1, int R2, bool EO, bool INV>
 __global__ void __launch_bounds__(YRegCfg<R1, R2, EO>::NT, YRegCfg<R1, R2, EO>::MINB)
-k_y_reg(OpView<float> op, float2* __restrict__ buf, const int* __restrict__ active) {
+k_y_reg(OpView<float> op, float2* buf, const int* active) {
   using K = YRegCfg<R1, R2, EO>;
   constexpr int TILE = K::TILE, NT = K::NT, NJ = K::NJ, NQ = K::NQ, EL = K::EL;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* sm = reinterpret_cast<float2*>(smem_raw);
   const int r = blockIdx.z;
+  chain_next();
+  chain_wait();
+  active = chained(active);
+  buf = chained(buf);
   if (active && !active[r]) return;
   const int Lx = op.Lx, ny = op.ny;
   const int col0 = blockIdx.x * TILE;
@@ -130,8 +134,8 @@ void launch_y_reg(bool inv, const OpView<float>& op, int R, float2* buf, const i
                   cudaStream_t st) {
   using K = YRegCfg<R1, R2, EO>;
   const dim3 g((op.Lx + K::TILE - 1) / K::TILE, 3 * op.nz, R);
-  if (inv) k_y_reg<R1, R2, EO, true><<<g, K::NT, K::smem, st>>>(op, buf, active);
-  else k_y_reg<R1, R2, EO, false><<<g, K::NT, K::smem, st>>>(op, buf, active);
+  launch_chained(op.chain, inv ? k_y_reg<R1, R2, EO, true> : k_y_reg<R1, R2, EO, false>, g, K::NT,
+                 K::smem, st, op, buf, active);
 }
 template <int R1, int R2, bool EO> cudaError_t configure_y_reg() {
   const int smem = (int)YRegCfg<R1, R2, EO>::smem;

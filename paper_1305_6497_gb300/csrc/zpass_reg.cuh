@@ -75,8 +75,7 @@ __device__ __forceinline__ float flip_if(float a, unsigned m) {
 
 template <int R1, int R2, bool EO, bool ASYNC>
 __global__ void __launch_bounds__(ZRegCfg<R1, R2, EO>::NT, ZRegCfg<R1, R2, EO>::MINB)
-k_fft_z_reg(OpView<float> op, float2* __restrict__ buf, int R, int per,
-            const int* __restrict__ active) {
+k_fft_z_reg(OpView<float> op, float2* buf, int R, int per, const int* active) {
   using K = ZRegCfg<R1, R2, EO>;
   constexpr int n = K::n, L = K::L, TILE = K::TILE, NT = K::NT, ROW = K::ROW, Hz = K::Hz;
   constexpr int NJ = K::NJ, EL = K::EL;
@@ -93,8 +92,16 @@ k_fft_z_reg(OpView<float> op, float2* __restrict__ buf, int R, int per,
     while (v < vend && ((self && (v & 1)) || (active && !active[v >> 1]))) ++v;
     return v;
   };
-  int v = next(blockIdx.z * per);
-  if (v >= vend) return;
+  // a right-hand side frozen before the predecessor has ended stays so
+  chain_next();
+  if (active) {
+    int v = blockIdx.z * per;
+    while (v < vend && !static_cast<const volatile int*>(active)[v >> 1]) ++v;
+    if (v >= vend) {
+      chain_wait();
+      return;
+    }
+  }
   const int col0 = blockIdx.x * TILE;
   const int ncol = min(TILE, Lx - col0);
   const int64_t plane = (int64_t)Ly * Lx, comp = nz * plane;
@@ -103,6 +110,29 @@ k_fft_z_reg(OpView<float> op, float2* __restrict__ buf, int R, int per,
   const int c1 = threadIdx.x / (TILE * R2);
   const bool on1 = c1 < 3 && t1 < ncol;
   const bool last = j2 + R2 * (NJ - 1) < nz;  // z < nz holds for the other j1
+  // the Ghat tile: columns of 3 x Hz 16-byte pieces, contiguous
+  int hx[TILE];
+#pragma unroll
+  for (int t = 0; t < TILE; ++t) {
+    const int kx = op.kx_at[col0 + min(t, ncol - 1)];
+    hx[t] = kx > (Lx >> 1) ? Lx - kx : kx;
+  }
+#pragma unroll
+  for (int t = 0; t < TILE; ++t) {
+    const float4* src =
+        reinterpret_cast<const float4*>(op.ghat) + ((int64_t)hy * op.Hx + hx[t]) * 3 * Hz;
+    for (int q = threadIdx.x; q < 3 * Hz; q += NT) cp_async<16>(gsm + t * K::GS + q, src + q);
+  }
+  for (int e = threadIdx.x; e < n; e += NT) cp_async<16>(tws + e, op.twz_reg + e);
+  cp_async_commit();
+  chain_wait();
+  active = chained(active);
+  buf = chained(buf);
+  int v = next(blockIdx.z * per);
+  if (v >= vend) {
+    cp_async_wait_all();
+    return;
+  }
   float2* const first = buf + col0 + min(t1, ncol - 1) + min(c1, 2) * comp + j2 * plane;
   const int64_t row0 = (int64_t)op.ypos_at[hy] * Lx;
   const int64_t row1 = (int64_t)op.ypos_at[self ? hy : Ly - hy] * Lx;
@@ -138,21 +168,6 @@ k_fft_z_reg(OpView<float> op, float2* __restrict__ buf, int R, int per,
     }
   };
   fetch(v);
-  // the Ghat tile: columns of 3 x Hz 16-byte pieces, contiguous
-  int hx[TILE];
-#pragma unroll
-  for (int t = 0; t < TILE; ++t) {
-    const int kx = op.kx_at[col0 + min(t, ncol - 1)];
-    hx[t] = kx > (Lx >> 1) ? Lx - kx : kx;
-  }
-#pragma unroll
-  for (int t = 0; t < TILE; ++t) {
-    const float4* src =
-        reinterpret_cast<const float4*>(op.ghat) + ((int64_t)hy * op.Hx + hx[t]) * 3 * Hz;
-    for (int q = threadIdx.x; q < 3 * Hz; q += NT) cp_async<16>(gsm + t * K::GS + q, src + q);
-  }
-  for (int e = threadIdx.x; e < n; e += NT) cp_async<16>(tws + e, op.twz_reg + e);
-  cp_async_commit();
   // and in step 2
   const int t2 = threadIdx.x % TILE, p2 = EO ? (threadIdx.x / TILE) & 1 : 0;
   const int k2 = threadIdx.x / ((EO ? 2 : 1) * TILE);
@@ -269,9 +284,11 @@ void launch_z_reg(const OpView<float>& op, int R, float2* buf, const int* active
   per = per < 1 ? 1 : per > 2 * R ? 2 * R : per;
   const dim3 g(tiles, hy, (unsigned)((2 * R + per - 1) / per));
   if (op.Lx % 2 == 0 && ((uintptr_t)buf & 15) == 0)
-    k_fft_z_reg<R1, R2, EO, true><<<g, K::NT, K::smem, st>>>(op, buf, R, (int)per, active);
+    launch_chained(op.chain, k_fft_z_reg<R1, R2, EO, true>, g, K::NT, K::smem, st, op, buf, R, (int)per,
+                   active);
   else
-    k_fft_z_reg<R1, R2, EO, false><<<g, K::NT, K::smem, st>>>(op, buf, R, (int)per, active);
+    launch_chained(op.chain, k_fft_z_reg<R1, R2, EO, false>, g, K::NT, K::smem, st, op, buf, R,
+                   (int)per, active);
 }
 
 // The plans, in parts that compile side by side (zpass_reg_*.cu): X(R1, R2).
