@@ -131,7 +131,7 @@ def pass_bytes(box, grid, s):
 def _source_hash():
     h = hashlib.sha256()
     for f in ("matvec_impl.cuh", "fft_core.cuh", "fft_plan.cuh", "matvec_fixed.cu",
-              "zpass_pair.cuh", "dda_common.cuh"):
+              "zpass_pair.cuh", "dda_common.cuh", "fft_reg.cuh", "reg_step.cuh", "zpass_reg.cuh"):
         with open(os.path.join(ROOT, "paper_1305_6497_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -437,10 +437,15 @@ def run_gpu(args, rank, world, local_rank):
     achieved = alg / (tms / 1e3) / 1e9
     peak, peak_kind = _peaks()
     traffic_launch = _ncu_traffic(dom, wl)
-    # the z pass runs the column-pair kernel for z kinds 2..7, else the
-    # one-column-tile kernels
-    zk = schedule["fp32"]["z_stage_ghat"]
-    kname = {"z_mul": "k_fft_z_pairs" if zk >= 2 else "k_fft_z_mul"}.get(dom, f"k_fft_{dom}")
+    # z kind 8: the register kernel, 2..7: the column-pair kernel, 0 and 1: the
+    # one-column-tile kernels; + 16 and + 32: the register x and y passes
+    kind = schedule["fp32"]["z_stage_ghat"]
+    zk = kind % 16
+    xreg, yreg = kind // 16 % 2, kind // 32 % 2
+    kname = {"z_mul": "k_fft_z_reg" if zk == 8 else "k_fft_z_pairs" if zk >= 2 else "k_fft_z_mul",
+             "x_fwd": "k_x_fwd_reg" if xreg else "k_fft_x_fwd",
+             "x_inv": "k_x_inv_reg" if xreg else "k_fft_x_inv",
+             }.get(dom, "k_y_reg" if yreg else f"k_fft_{dom}")
     share = {f"{p}": round(kern_ms[("fp32", p)] / sum(step_ms), 4) for p in B.PASSES}
     share.update({f"{p}_fp64": round(kern_ms[("fp64", p)] / sum(step_ms), 4)
                   for p in B.PASSES})

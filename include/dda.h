@@ -293,8 +293,9 @@ dda_status dda_autotune(dda_target* t, double kd, int n_rhs);
  * kernel (two columns per thread, both rows of an octant row and every
  * right-hand side per CTA, its own radix-8 plan; Ghat through L2 / staged);
  * 6 / 7 -- the same with each pass's column tile moved by TMA tensor copies;
- * 8 -- the FP32 register kernel (the default where the z length has a plan; its
- * tile is reported as 8, its pitch and threads are fixed by the plan).
+ * 8 -- the register kernel (FP32: the default where the z length has a plan, tile
+ * reported as 8; FP64: the default for z lengths up to 80 with a plan, tile reported
+ * as 4; pitch and threads are fixed by the plan).
  * + 16 -- the FP32 register x passes, + 32 -- the register y passes (defaults
  * where the axis length has a plan; x lines / y tile and their threads are then
  * not used). */
@@ -307,8 +308,8 @@ dda_status dda_target_schedule(const dda_target* t, int precision, int* out8);
  * 32; up to 384 for the FP32 z pass when the target's z length has a compiled
  * radix plan for that tile; exactly 384 for kinds 2..7, which need FP32, an
  * even Lx, Lz of 64, 128, 288 or 512 and tile 4 or 8, and for 6/7 nz <= 256;
- * kind 8 needs FP32, tile 8 and an even Lz with a two-factor plan; + 16 and + 32
- * FP32 and such an Lx, Ly),
+ * kind 8 needs an Lz with a two-factor plan and tile 8 (FP32) or 4 (FP64, even
+ * Lz up to 512); + 16 and + 32 need FP32 and such an Lx, Ly),
  * or needing more than 200 KB of shared memory: DDA_ERR_INVALID_ARG.  Kinds
  * 0/1, 2/3 and 8 factor the z transform differently (the same transform, results
  * equal to FP32 rounding); otherwise the schedule changes tiling and launch

@@ -30,8 +30,8 @@
 // without a conflict, and so do the reads of the Ghat tile (see ROW and GS).
 //
 // What bounds it: instruction issue and the shared-memory pipe (of the 64x64x256
-// brick: 52% and 55% busy, 17% of the DRAM bandwidth, 155 thread instructions per
-// stored point against 216 of the column-pair kernel).  8 columns per CTA (64-byte
+// brick: 49% and 55% busy, 29% of the DRAM bandwidth, 153 thread instructions per
+// stored point against 214 of the column-pair kernel).  8 columns per CTA (64-byte
 // rows in global memory) up to n = 96 and 4 above leave room for two to four CTAs.
 // Per launch with two right-hand sides, before (the default one-tile or, where
 // named, the tuned kernel) and now: 256^3 box 8600 (tuned pair kernel 4460) ->

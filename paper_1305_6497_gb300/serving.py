@@ -6,8 +6,8 @@ GPU at once, each on its own ``dda_target`` and therefore its own CUDA stream,
 so their kernels overlap on the device.  A request is admitted as soon as a
 slot is free AND the device bytes it needs fit in the HBM budget.  Its bytes
 are the library's host-only estimate for a new target of its shape
-(``dda_estimate_solve_bytes``: creation arrays, Green-tensor transform with its
-transient build grids, solve workspace); nothing is allocated before
+(``dda_estimate_solve_bytes``: creation arrays, Green-tensor transform,
+solve workspace); nothing is allocated before
 admission.  Finished solves return their reservation at once, so requests that
 arrive while others run start as room appears -- not a queue drained one at a
 time.
