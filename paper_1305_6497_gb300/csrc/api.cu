@@ -315,8 +315,15 @@ struct LoopGraph {
 
 // Writes a byte of every page of an output array (all of which a copy overwrites), so
 // that a caller's freshly allocated pages are mapped while the device computes and not
-// one by one under the copy.
+// one by one under the copy.  Pageable memory only: pinned pages are mapped, and a
+// device pointer is the copy's to refuse.
 static void touch_pages(void* p, size_t bytes) {
+  cudaPointerAttributes at{};
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
+  if (at.type != cudaMemoryTypeUnregistered) return;
   volatile char* c = static_cast<volatile char*>(p);
   for (size_t i = 0; i < bytes; i += 4096) c[i] = 0;
 }
