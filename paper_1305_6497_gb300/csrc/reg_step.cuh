@@ -3,6 +3,8 @@
 // and the plans of odd lengths.
 #pragma once
 
+#include <type_traits>
+
 #include "fft_reg.cuh"
 #include "matvec_impl.cuh"
 
@@ -45,23 +47,32 @@ __device__ __forceinline__ void reg_step1(const float2 (&x)[NJ], const float4* t
     }
   }
 }
-// Its inverse: the elements src[k pitch] to the outputs y[0..NJ).
-// `loaded` is called
-// once the elements have been read (and may be overwritten).
-template <int R1, int R2, bool EO, int NJ, class F>
-__device__ __forceinline__ void reg_step1_inv(const float2* src, int pitch, const float4* tw,
-                                              float2 (&y)[NJ], const F& loaded) {
-  if constexpr (EO) {
-    cv<f32p> a[R1];
+// Its inverse in two parts, of which only the first reads shared memory: the elements
+// src[k pitch], times the conjugate twiddles, and from them the outputs y[0..NJ).
+template <bool EO> using reg_cv = cv<std::conditional_t<EO, f32p, float>>;
+
+template <int R1, int R2, bool EO>
+__device__ __forceinline__ void reg_step1_inv_read(const float2* src, int pitch, const float4* tw,
+                                                   reg_cv<EO> (&a)[R1]) {
 #pragma unroll
-    for (int k = 0; k < R1; ++k) {
-      const float4 q = *reinterpret_cast<const float4*>(src + k * pitch), w = tw[k * R2];
+  for (int k = 0; k < R1; ++k) {
+    const float4 w = tw[k * R2];
+    if constexpr (EO) {
+      const float4 q = *reinterpret_cast<const float4*>(src + k * pitch);
       const cv<float> e = cvmulc(cv<float>{w.x, w.y}, cv<float>{q.x, q.y});
       const cv<float> o = cvmulc(cv<float>{w.z, w.w}, cv<float>{q.z, q.w});
       a[k] = {pk_make(e.re, o.re), pk_make(e.im, o.im)};
+    } else {
+      const float2 q = src[k * pitch];
+      a[k] = cvmulc(cv<float>{w.x, w.y}, cv<float>{q.x, q.y});
     }
-    loaded();
-    rdft<R1, true>(a);
+  }
+}
+
+template <int R1, bool EO, int NJ>
+__device__ __forceinline__ void reg_step1_inv_out(reg_cv<EO> (&a)[R1], float2 (&y)[NJ]) {
+  rdft<R1, true>(a);
+  if constexpr (EO) {
     static_for<R1>([&](auto jc) {
       constexpr int j = decltype(jc)::value;
       constexpr float cw = (float)cx_cos(j, 2 * R1), sw = (float)cx_sin(j, 2 * R1);
@@ -71,15 +82,6 @@ __device__ __forceinline__ void reg_step1_inv(const float2* src, int pitch, cons
       y[j] = make_float2(fmaf(cw, ro, fmaf(-sw, io, re)), fmaf(cw, io, fmaf(sw, ro, im)));
     });
   } else {
-    cv<float> a[R1];
-#pragma unroll
-    for (int k = 0; k < R1; ++k) {
-      const float2 q = src[k * pitch];
-      const float4 w = tw[k * R2];
-      a[k] = cvmulc(cv<float>{w.x, w.y}, cv<float>{q.x, q.y});
-    }
-    loaded();
-    rdft<R1, true>(a);
 #pragma unroll
     for (int j = 0; j < NJ; ++j) y[j] = make_float2(a[j].re, a[j].im);
   }
@@ -88,7 +90,9 @@ __device__ __forceinline__ void reg_step1_inv(const float2* src, int pitch, cons
 template <int R1, int R2, bool EO, int NJ>
 __device__ __forceinline__ void reg_step1_inv(const float2* src, int pitch, const float4* tw,
                                               float2 (&y)[NJ]) {
-  reg_step1_inv<R1, R2, EO>(src, pitch, tw, y, []() {});
+  reg_cv<EO> a[R1];
+  reg_step1_inv_read<R1, R2, EO>(src, pitch, tw, a);
+  reg_step1_inv_out<R1, EO>(a, y);
 }
 // odd lengths R1 R2
 #define DDA_XREG_ODD(X) X(5, 3) X(5, 5) X(9, 3) X(9, 5) X(15, 5) X(9, 9) X(15, 9) X(15, 15)

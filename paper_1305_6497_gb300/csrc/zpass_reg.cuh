@@ -139,7 +139,7 @@ k_fft_z_reg(OpView<float> op, float2* buf, int R, int per, const int* active) {
   auto line = [&](int w) { return first + (w >> 1) * 3 * comp + ((w & 1) ? row1 : row0); };
   float2* own = sm + EL * (c1 * (R1 * ROW) + j2 * TILE + t1);
   // The next pass's input is asked for as soon as step 3 has read the thread's
-  // words of shared memory, and lands in them (ASYNC: 16-byte asynchronous copies
+  // words of shared memory (odd L: both threads' of a pair), and lands in them (ASYNC: 16-byte asynchronous copies
   // past L1, each holding the two columns of a pair of threads for one row; the
   // threads of a pair take the even and the odd rows).  Plain loads need a line of
   // L1 for each of their 32-byte rows until they arrive, and the shared memory
@@ -249,11 +249,21 @@ k_fft_z_reg(OpView<float> op, float2* buf, int R, int per, const int* active) {
 
     // ---- 3. inverse R1-point DFTs, the halves joined, to global memory.  A thread
     // reads here what it wrote in step 1 and nobody else does, so the next pass's
-    // step 1 needs no barrier
+    // step 1 needs no barrier.  The next pass's copies land in these words: in the
+    // thread's own for EO, but in both threads' of a pair for odd L, where neither
+    // may ask for them before the other has read its words (a warp barrier that
+    // every thread of the CTA passes: the last warp may hold threads with c1 = 3)
+    reg_cv<EO> a[R1];
+    constexpr bool pair = ASYNC && !EO;
+    if constexpr (pair) {
+      if (c1 < 3) reg_step1_inv_read<R1, R2, EO>(own, EL * ROW, tw, a);
+      __syncwarp();
+    }
     if (c1 < 3) {
+      if constexpr (!pair) reg_step1_inv_read<R1, R2, EO>(own, EL * ROW, tw, a);
+      if (ASYNC && vn < vend) fetch(vn);
       float2 y[NJ];
-      reg_step1_inv<R1, R2, EO>(own, EL * ROW, tw, y,
-                                [&]() { if (ASYNC && vn < vend) fetch(vn); });
+      reg_step1_inv_out<R1, EO>(a, y);
       float2* dst = line(v);
 #pragma unroll
       for (int j = 0; j < NJ; ++j)
