@@ -61,13 +61,15 @@ cudaError_t launch_cross_sections(int nx, int ny, int nz, const uint8_t* comp, R
 __global__ void k_direction_phases(int nx, int ny, int nz, int D, double kd,
                                    const double* __restrict__ dirs, double2* __restrict__ ph) {
   const int per = nx + ny + nz;
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < D * per; e += gridDim.x * blockDim.x) {
-    const int d = e / per, q = e - d * per;
+  const int64_t entries = (int64_t)D * per;  // 2^31 of them are 34 GB, which the part holds
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < entries;
+       e += (int64_t)gridDim.x * blockDim.x) {
+    const int d = (int)(e / per), q = (int)(e - (int64_t)d * per);
     const int a = q < nx ? 0 : q < nx + ny ? 1 : 2;
     const int n = a == 0 ? nx : a == 1 ? ny : nz;
     const int i = a == 0 ? q : a == 1 ? q - nx : q - nx - ny;
     double sn, cs;
-    sincos(-kd * dirs[3 * d + a] * (i - 0.5 * (n - 1)), &sn, &cs);
+    sincos(-kd * dirs[3 * (int64_t)d + a] * (i - 0.5 * (n - 1)), &sn, &cs);
     ph[(a == 0 ? (int64_t)d * nx : a == 1 ? (int64_t)D * nx + (int64_t)d * ny
                                           : (int64_t)D * (nx + ny) + (int64_t)d * nz) + i] =
         make_double2(cs, sn);

@@ -40,3 +40,27 @@ def test_amplitudes_match_the_sum_over_dipoles(shape, ndir, npol):
                 assert abs(o["famp"][i, d, 0, l] - kd ** 3 * eth @ F) <= 1e-13 * big
                 assert abs(o["famp"][i, d, 1, l] - kd ** 3 * eph @ F) <= 1e-13 * big
     t.close()
+
+
+@pytest.mark.parametrize("ndir", [2093055, 2100001])
+def test_phase_tables_of_more_than_int_max_entries(ndir):
+    """A line of 1024 sites, whose phase tables have 1026 entries a direction: just
+    below 2^31 entries (where a 32-bit index passes 2^31 in its last stride) and
+    above.  The directions repeat, so every amplitude is one of the first 4096."""
+    from paper_1305_6497_gb300 import binding as B
+    occ, comp = tg.rect_prism(1024, 1, 1)
+    kh, yh, e1 = W._lab_incidence([(0.4, 0.9, 1.3)])
+    rng = np.random.default_rng(8)
+    some = np.stack([rng.uniform(0, np.pi, 4096), rng.uniform(0, 2 * np.pi, 4096)], 1)
+    dirs = np.resize(some, (ndir, 2))
+    t = B.Target(occ, comp, [1.3 + 0.05j], method="CM")
+    kw = dict(yhat=yh, npol=1, tol=1e-8)
+    o = t.solve(0.3, kh, e1, dirs=dirs, **kw)
+    f = o["famp"][0, 1:, :, 0]
+    first = t.solve(0.3, kh, e1, dirs=some[:64], **kw)
+    t.close()
+    big = 0.3 ** 3 * np.abs(o["P"]).sum()
+    assert np.abs(f[:64] - first["famp"][0, 1:, :, 0]).max() <= 1e-13 * big
+    for k in range(0, ndir, 4096):
+        part = f[k:k + 4096]
+        np.testing.assert_array_equal(part, f[:len(part)])
