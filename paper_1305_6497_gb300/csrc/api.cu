@@ -1286,13 +1286,16 @@ static int64_t workspace_bytes(const dda_target* t, int R, dda_precision prec, i
   b += ns * 16;  // FP64 scratch (final/true residual matvec)
   if (f32) b += 8 * nv * 8 + ns * 8;
   const int nblk = std::max(reduce_blocks(3 * t->nbox), 3 * t->nz * t->ny);
-  // Krylov partials [R][nblk][<= 8]; far field, one incidence at a time:
-  // [2][ndir+1][fblk][6]
-  const int fblk = farfield_blocks(t->nx, t->ny, t->nz, ndir + 1);
-  b += std::max((int64_t)8 * R * nblk, (int64_t)12 * (ndir + 1) * fblk) * 8;
+  // Krylov partials [R][nblk][<= 8]; far field, one incidence and chunk of directions
+  // at a time: [2][fdir][fblk][6]
+  const int fdir = farfield_chunk(t->nx, t->ny, t->nz, ndir + 1);
+  const int fblk = farfield_blocks(t->nx, t->ny, t->nz, fdir);
+  b += std::max((int64_t)8 * R * nblk, (int64_t)12 * fdir * fblk) * 8;
   b += (int64_t)R * (sizeof(KState) + 64) + (int64_t)R * (t->nx + t->ny + t->nz + 8) * 16;
   b += (int64_t)fold_bytes(R);  // scalar-step counters and group sums
-  b += (int64_t)(ndir + 1) * ((t->nx + t->ny + t->nz) * 16 + 24) + t->N * (int64_t)R * 48;
+  // far field: phase tables of a chunk, unit vectors and sums of every direction
+  b += (int64_t)fdir * (t->nx + t->ny + t->nz) * 16 + (int64_t)(ndir + 1) * (24 + 96);
+  b += t->N * (int64_t)R * 48;
   return b;
 }
 
@@ -1318,8 +1321,9 @@ static void ensure_workspace(dda_target* t, int R, dda_precision prec, int ndir)
   const int nblk = std::max({reduce_blocks(3 * t->nbox), (rows + t->L32.x_lines - 1) / t->L32.x_lines,
                              (rows + t->L64.x_lines - 1) / t->L64.x_lines,
                              t->L32.x_reg ? x_reg_blocks(t->Lx, rows) : 1});
-  const int fblk = farfield_blocks(t->nx, t->ny, t->nz, ndir + 1);
-  w.partials.ensure((size_t)std::max((int64_t)8 * R * nblk, (int64_t)12 * (ndir + 1) * fblk) * 8);
+  const int fdir = farfield_chunk(t->nx, t->ny, t->nz, ndir + 1);
+  const int fblk = farfield_blocks(t->nx, t->ny, t->nz, fdir);
+  w.partials.ensure((size_t)std::max((int64_t)8 * R * nblk, (int64_t)12 * fdir * fblk) * 8);
   w.ks.ensure(sizeof(KState) * R);
   w.active.ensure(sizeof(int) * R);
   w.active_outer.ensure(sizeof(int) * R);
@@ -1331,7 +1335,7 @@ static void ensure_workspace(dda_target* t, int R, dda_precision prec, int ndir)
   w.ainv32.ensure(sizeof(float2) * (size_t)R * (t->ncomp + 1) * 3);
   w.ainvdf.ensure(sizeof(df64c) * (size_t)R * (t->ncomp + 1) * 3);
   w.wabs.ensure(sizeof(double) * (size_t)R * (t->ncomp + 1) * 3);
-  w.fph.ensure(sizeof(double2) * (size_t)(ndir + 1) * (t->nx + t->ny + t->nz));
+  w.fph.ensure(sizeof(double2) * (size_t)fdir * (t->nx + t->ny + t->nz));
   w.fdir.ensure(sizeof(double) * 3 * (size_t)(ndir + 1));
   w.sitebuf.ensure(sizeof(double2) * 3 * (size_t)t->N * R);
   w.R = R;
@@ -1983,7 +1987,8 @@ dda_status dda_solve(dda_target* t, const dda_solve_params* p, dda_solve_result*
     std::vector<double> ff;
     if (res->famp) {
       ff.resize((size_t)p->n_inc * D * p->npol * 6);
-      const int fblk = farfield_blocks(t->nx, t->ny, t->nz, D);
+      const int chunk = farfield_chunk(t->nx, t->ny, t->nz, D);
+      const int fblk = farfield_blocks(t->nx, t->ny, t->nz, chunk);
       std::vector<double> fdir(3 * (size_t)D);
       for (int i = 0; i < p->n_inc; ++i) {
         const double* x = incs[i].khat;
@@ -1999,15 +2004,19 @@ dda_status dda_solve(dda_target* t, const dda_solve_params* p, dda_solve_result*
         }
         CK(cudaMemcpyAsync(w.fdir.p, fdir.data(), sizeof(double) * fdir.size(),
                            cudaMemcpyHostToDevice, st));
-        CK(launch_direction_phases(t->nx, t->ny, t->nz, D, kd, w.fdir.as<double>(),
-                                   w.fph.as<double2>(), st));
-        const double2* dfx = w.fph.as<double2>();
-        const double2* dfy = dfx + (size_t)D * t->nx;
-        const double2* dfz = dfy + (size_t)D * t->ny;
         const double2* Pi = w.x64.as<double2>() + (size_t)i * p->npol * n;
-        CK(launch_farfield(t->nx, t->ny, t->nz, t->comp.as<uint8_t>(), p->npol, D, Pi, dfx,
-                           dfy, dfz, part, st));
-        CK(launch_finalize_sums(p->npol * D, fblk, 6, part, w.sums.as<double>(), st));
+        for (int d0 = 0; d0 < D; d0 += chunk) {
+          const int nd = std::min(chunk, D - d0);
+          CK(launch_direction_phases(t->nx, t->ny, t->nz, nd, kd, w.fdir.as<double>() + 3 * (size_t)d0,
+                                     w.fph.as<double2>(), st));
+          const double2* dfx = w.fph.as<double2>();
+          const double2* dfy = dfx + (size_t)nd * t->nx;
+          const double2* dfz = dfy + (size_t)nd * t->ny;
+          CK(launch_farfield(t->nx, t->ny, t->nz, t->comp.as<uint8_t>(), p->npol, chunk, nd, Pi,
+                             dfx, dfy, dfz, part, st));
+          CK(launch_finalize_sums(p->npol * nd, fblk, 6, part,
+                                  w.sums.as<double>() + (size_t)d0 * p->npol * 6, st));
+        }
         CK(cudaMemcpyAsync(ff.data() + (size_t)i * D * p->npol * 6, w.sums.p,
                            sizeof(double) * D * p->npol * 6, cudaMemcpyDeviceToHost, st));
         CK(cudaStreamSynchronize(st));

@@ -336,11 +336,13 @@ cudaError_t launch_nearfield_post(int nx, int ny, int nz, const uint8_t* comp, R
                                   int R, const double2* esca, const double2* fac,
                                   const double* khat, double2* einc, double2* emacro,
                                   double2* binc, cudaStream_t st);
-// far-field sums F[d][r][3] = sum_j P_j exp(-i k n_d . r_j), partials per block
-// (farfield_blocks partials of 6 sums per direction and right-hand side; R = 1 or 2)
-cudaError_t launch_farfield(int nx, int ny, int nz, const uint8_t* comp, int R, int D,
+// far-field sums F[d][r][3] = sum_j P_j exp(-i k n_d . r_j) of n <= D directions, partials
+// per block (farfield_blocks(D) partials of 6 sums per direction and right-hand side;
+// R = 1 or 2).  A launch takes up to D = farfield_chunk directions of a call's.
+cudaError_t launch_farfield(int nx, int ny, int nz, const uint8_t* comp, int R, int D, int n,
                             const double2* P, const double2* fphx, const double2* fphy,
                             const double2* fphz, double* partials, cudaStream_t st);
+int farfield_chunk(int nx, int ny, int nz, int D);
 int farfield_blocks(int nx, int ny, int nz, int D);
 // Its phase tables, [D][nx], [D][ny], [D][nz], from D unit vectors (device).
 cudaError_t launch_direction_phases(int nx, int ny, int nz, int D, double kd, const double* dirs,

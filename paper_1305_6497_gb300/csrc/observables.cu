@@ -177,23 +177,35 @@ static void farfield_grid(int nx, int ny, int nz, int D, int& dc, int& cols, int
   zchunks = (nz + per - 1) / per;
 }
 
+// Directions of one launch.  Every column block leaves six sums per direction and
+// right-hand side: 4096 blocks of a 1024 x 1024 box 393 KB per direction.  A chunk's
+// partial sums stay within 8 MiB (340 directions of a 256^3 box, still 21,000 blocks)
+// and its phase tables within 64 MiB.  Chunks are of equal size and, but for the last,
+// hold a multiple of the four directions of a thread.
+int farfield_chunk(int nx, int ny, int nz, int D) {
+  const int64_t cols = ((int64_t)nx * ny + kThreads - 1) / kThreads;
+  const int64_t c = std::min((8ll << 20) / (96 * cols), (64ll << 20) / (16 * (nx + ny + nz)));
+  const int64_t most = std::max<int64_t>(4, c / 4 * 4), k = (D + most - 1) / most;
+  return (int)std::min<int64_t>(D, ((D + k - 1) / k + 3) / 4 * 4);
+}
+
 int farfield_blocks(int nx, int ny, int nz, int D) {
   int dc, cols, zchunks;
   farfield_grid(nx, ny, nz, D, dc, cols, zchunks);
   return cols * zchunks;
 }
 
-cudaError_t launch_farfield(int nx, int ny, int nz, const uint8_t* comp, int R, int D,
+cudaError_t launch_farfield(int nx, int ny, int nz, const uint8_t* comp, int R, int D, int n,
                             const double2* P, const double2* fphx, const double2* fphy,
                             const double2* fphz, double* partials, cudaStream_t st) {
   int dc, cols, zchunks;
   farfield_grid(nx, ny, nz, D, dc, cols, zchunks);
   const int zper = (nz + zchunks - 1) / zchunks;
-  for (int c0 = 0; c0 < (D + dc - 1) / dc; c0 += 65535) {  // grid.y limit
-    const int d0 = c0 * dc, n = std::min(D - d0, 65535 * dc);
-    const dim3 g(cols * zchunks, (n + dc - 1) / dc);
+  for (int c0 = 0; c0 < (n + dc - 1) / dc; c0 += 65535) {  // grid.y limit
+    const int d0 = c0 * dc, m = std::min(n - d0, 65535 * dc);
+    const dim3 g(cols * zchunks, (m + dc - 1) / dc);
 #define DDA_FAR(DC, RR)                                                                      \
-  k_farfield<DC, RR><<<g, kThreads, 0, st>>>(nx, ny, nz, cols, zper, n, comp, P,             \
+  k_farfield<DC, RR><<<g, kThreads, 0, st>>>(nx, ny, nz, cols, zper, m, comp, P,             \
                                              fphx + (int64_t)d0 * nx, fphy + (int64_t)d0 * ny, \
                                              fphz + (int64_t)d0 * nz,                        \
                                              partials + (int64_t)d0 * R * cols * zchunks * 6)

@@ -45,8 +45,9 @@ def test_amplitudes_match_the_sum_over_dipoles(shape, ndir, npol):
 @pytest.mark.parametrize("ndir", [2093055, 2100001])
 def test_phase_tables_of_more_than_int_max_entries(ndir):
     """A line of 1024 sites, whose phase tables have 1026 entries a direction: just
-    below 2^31 entries (where a 32-bit index passes 2^31 in its last stride) and
-    above.  The directions repeat, so every amplitude is one of the first 4096."""
+    below 2^31 entries in all (where a 32-bit index passes 2^31 in its last stride) and
+    above, in hundreds of chunks.  The directions repeat, so every amplitude is one of
+    the first 4096."""
     from paper_1305_6497_gb300 import binding as B
     occ, comp = tg.rect_prism(1024, 1, 1)
     kh, yh, e1 = W._lab_incidence([(0.4, 0.9, 1.3)])
