@@ -2164,6 +2164,53 @@ void tune_store_locked(const std::string& key, const std::vector<int>& v) {
   out << '\n';
 }
 
+// Why the target cannot run a schedule (the layout of dda_target_schedule), or null.
+const char* schedule_fault(const dda_target* t, bool f64, const int* in8) {
+  const int xl = in8[0], yt = in8[1], zt = in8[2], zp = in8[3];
+  const int zg = in8[4] < 0 || in8[4] > 63 ? -1 : in8[4] & 15;  // z kind; +16, +32: register x, y passes
+  const size_t cs = f64 ? sizeof(double2) : sizeof(float2);
+  if (xl < 1 || xl > 64 || yt < 1 || yt > 64 || (zt != 2 && zt != 4 && zt != 8 && zt != 16) ||
+      zp < 3 * zt || zp > 3 * zt + 8 || zg < 0 || zg > 8 || zg == 4 || zg == 5)
+    return "schedule: x lines 1..64, y tile 1..64, z tile 2/4/8/16, "
+           "z pitch 3*tile..3*tile+8, z staging 0, 1, 2, 3, 6, 7 or 8";
+  if ((in8[4] & 16) && (f64 || !x_reg_plan(t->Lx, t->nx, nullptr, nullptr)))
+    return "schedule: the register x passes (z staging + 16) need FP32 "
+           "and an Lx with a two-factor plan";
+  if ((in8[4] & 32) && (f64 || !x_reg_plan(t->Ly, t->ny, nullptr, nullptr)))
+    return "schedule: the register y passes (z staging + 32) need FP32 "
+           "and an Ly with a two-factor plan";
+  if (zg == 8 && (f64 ? zt != 4 || !z_wide_plan(t->Lz, t->nz, nullptr, nullptr)
+                      : zt != kZRegTile || !z_reg_plan(t->Lz, t->nz, nullptr, nullptr)))
+    return "schedule: z staging 8 (register z kernel) needs z tile 8 "
+           "(FP64: 4) and an Lz with a two-factor plan";
+  if (zg >= 2 && zg != 8 && (f64 || !z_pair_applies(t->Lz, t->Lx, zt) || in8[7] != kZPairThreads))
+    return "schedule: z staging 2/3/6/7 (column-pair z kernel) needs "
+           "FP32, an even Lx, Lz of 64, 128, 288 or 512, tile 4 or 8 "
+           "and 384 threads";
+  if ((zg == 6 || zg == 7) && !z_pair_tma_applies(t->Lz, t->Lx, t->nz, zt))
+    return "schedule: z staging 6/7 (TMA tiles) needs nz <= 256";
+  for (int i = 5; i < 8; ++i) {
+    // the FP32 z pass of a compiled radix plan (and the column-pair one) takes
+    // up to 384 threads
+    const int tmax =
+        (i == 7 && !f64 && (z_fixed_applies(t->pz, zt) || (zg >= 2 && zg != 8))) ? 384 : 256;
+    if (in8[i] < 32 || in8[i] > tmax || in8[i] % 32)
+      return "schedule: threads per CTA must be a multiple of 32 in "
+             "32..256 (FP32 z pass of a compiled plan: ..384)";
+  }
+  const size_t xinv = (size_t)t->Lx * (xl + 1) * cs + (size_t)2 * xl * t->nx * cs;
+  const size_t ysm = (size_t)t->Ly * yt * cs;
+  // a compiled-plan z kernel uses its own pitch, 3 tile (+1 below 128 B rows)
+  const int zpc = (!f64 && z_fixed_applies(t->pz, zt))
+                      ? std::max(zp, 3 * zt + (zt * (int)cs < 128 ? 1 : 0)) : zp;
+  const size_t zsm = zg == 8 ? 0 : zg >= 2 ? zpair_smem_bytes(t->Lz, zt, zg == 3 || zg == 7)
+                             : (((size_t)t->Lz * zpc * cs + 15) & ~(size_t)15) +
+                                   (zg ? (size_t)6 * (t->Lz / 2 + 1) * zt * cs : 0);
+  if (xinv > 200 * 1024 || ysm > 200 * 1024 || zsm > 200 * 1024)
+    return "schedule: a pass would need more than 200 KB of shared memory";
+  return nullptr;
+}
+
 template <typename T>
 void apply_schedule(const dda_target* t, MatvecLaunch& L, const std::vector<int>& v) {
   using C = cplx_t<T>;
@@ -2327,6 +2374,9 @@ dda_status dda_autotune(dda_target* t, double kd, int n_rhs) {
         auto it = g_tune.find(key);
         if (it != g_tune.end()) v = it->second;
       }
+      // an entry that the target cannot run (the file's, which nothing has checked) is
+      // timed anew
+      if (!v.empty() && schedule_fault(t, prec != 0, v.data())) v.clear();
       if (v.empty()) {
         if (prec == 0) {
           OpView<float> op = make_view<float>(t, t->g32.p, w.ainv32.p, t->tw32.p);
@@ -2359,49 +2409,8 @@ dda_status dda_autotune(dda_target* t, double kd, int n_rhs) {
 dda_status dda_set_schedule(dda_target* t, int precision, const int* in8) {
   g_last_error.clear();
   if (!t || !in8) return fail(DDA_ERR_INVALID_ARG, "null argument");
-  const int xl = in8[0], yt = in8[1], zt = in8[2], zp = in8[3];
-  const int zg = in8[4] < 0 || in8[4] > 63 ? -1 : in8[4] & 15;  // z kind; +16, +32: register x, y passes
   const bool f64 = precision == DDA_PREC_FP64;
-  const size_t cs = f64 ? sizeof(double2) : sizeof(float2);
-  if (xl < 1 || xl > 64 || yt < 1 || yt > 64 || (zt != 2 && zt != 4 && zt != 8 && zt != 16) ||
-      zp < 3 * zt || zp > 3 * zt + 8 || zg < 0 || zg > 8 || zg == 4 || zg == 5)
-    return fail(DDA_ERR_INVALID_ARG, "schedule: x lines 1..64, y tile 1..64, z tile 2/4/8/16, "
-                                     "z pitch 3*tile..3*tile+8, z staging 0, 1, 2, 3, 6, 7 or 8");
-  if ((in8[4] & 16) && (f64 || !x_reg_plan(t->Lx, t->nx, nullptr, nullptr)))
-    return fail(DDA_ERR_INVALID_ARG, "schedule: the register x passes (z staging + 16) need FP32 "
-                                     "and an Lx with a two-factor plan");
-  if ((in8[4] & 32) && (f64 || !x_reg_plan(t->Ly, t->ny, nullptr, nullptr)))
-    return fail(DDA_ERR_INVALID_ARG, "schedule: the register y passes (z staging + 32) need FP32 "
-                                     "and an Ly with a two-factor plan");
-  if (zg == 8 && (f64 ? zt != 4 || !z_wide_plan(t->Lz, t->nz, nullptr, nullptr)
-                      : zt != kZRegTile || !z_reg_plan(t->Lz, t->nz, nullptr, nullptr)))
-    return fail(DDA_ERR_INVALID_ARG, "schedule: z staging 8 (register z kernel) needs z tile 8 "
-                                     "(FP64: 4) and an Lz with a two-factor plan");
-  if (zg >= 2 && zg != 8 && (f64 || !z_pair_applies(t->Lz, t->Lx, zt) || in8[7] != kZPairThreads))
-    return fail(DDA_ERR_INVALID_ARG, "schedule: z staging 2/3/6/7 (column-pair z kernel) needs "
-                                     "FP32, an even Lx, Lz of 64, 128, 288 or 512, tile 4 or 8 "
-                                     "and 384 threads");
-  if ((zg == 6 || zg == 7) && !z_pair_tma_applies(t->Lz, t->Lx, t->nz, zt))
-    return fail(DDA_ERR_INVALID_ARG, "schedule: z staging 6/7 (TMA tiles) needs nz <= 256");
-  for (int i = 5; i < 8; ++i) {
-    // the FP32 z pass of a compiled radix plan (and the column-pair one) takes
-    // up to 384 threads
-    const int tmax =
-        (i == 7 && !f64 && (z_fixed_applies(t->pz, zt) || (zg >= 2 && zg != 8))) ? 384 : 256;
-    if (in8[i] < 32 || in8[i] > tmax || in8[i] % 32)
-      return fail(DDA_ERR_INVALID_ARG, "schedule: threads per CTA must be a multiple of 32 in "
-                                       "32..256 (FP32 z pass of a compiled plan: ..384)");
-  }
-  const size_t xinv = (size_t)t->Lx * (xl + 1) * cs + (size_t)2 * xl * t->nx * cs;
-  const size_t ysm = (size_t)t->Ly * yt * cs;
-  // a compiled-plan z kernel uses its own pitch, 3 tile (+1 below 128 B rows)
-  const int zpc = (!f64 && z_fixed_applies(t->pz, zt))
-                      ? std::max(zp, 3 * zt + (zt * (int)cs < 128 ? 1 : 0)) : zp;
-  const size_t zsm = zg == 8 ? 0 : zg >= 2 ? zpair_smem_bytes(t->Lz, zt, zg == 3 || zg == 7)
-                             : (((size_t)t->Lz * zpc * cs + 15) & ~(size_t)15) +
-                                   (zg ? (size_t)6 * (t->Lz / 2 + 1) * zt * cs : 0);
-  if (xinv > 200 * 1024 || ysm > 200 * 1024 || zsm > 200 * 1024)
-    return fail(DDA_ERR_INVALID_ARG, "schedule: a pass would need more than 200 KB of shared memory");
+  if (const char* why = schedule_fault(t, f64, in8)) return fail(DDA_ERR_INVALID_ARG, why);
   try {
     CK(cudaSetDevice(t->device));
     configure(t);
