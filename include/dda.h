@@ -282,7 +282,9 @@ const char* dda_last_error(void);
  * memory), for batches of n_rhs right-hand sides, in FP32 and FP64.  Results
  * are cached per (precision, box, grid, n_rhs) for the process, and appended to
  * the file named by the environment variable DDA_TUNE_FILE when it is set (and
- * read from it first).  Builds the Green-tensor transform for kd if needed.
+ * read from it first; entries that an earlier version of the kernels timed, or that
+ * the target cannot run, are timed anew).  Builds the Green-tensor transform for kd if
+ * needed.
  * Without this call the library uses a fixed rule. */
 dda_status dda_autotune(dda_target* t, double kd, int n_rhs);
 

@@ -2114,9 +2114,11 @@ dda_status dda_solve(dda_target* t, const dda_solve_params* p, dda_solve_result*
 // ---------------------------------------------------------------------------
 // Schedule autotuning with a process-wide cache (optionally persisted in the
 // file named by DDA_TUNE_FILE: one line per key, "key : x_lines y_tile z_tile
-// z_pitch z_stage x_threads y_threads z_threads").
+// z_pitch z_stage x_threads y_threads z_threads").  A key begins with the version of
+// the kernels that were timed: entries of another (or none) stay in the file unused.
 // ---------------------------------------------------------------------------
 constexpr int kScheduleLen = 8;
+constexpr int kScheduleVersion = 2;  // 2: with the register passes (z kind 8, + 16, + 32)
 #include <fstream>
 #include <map>
 #include <mutex>
@@ -2129,8 +2131,8 @@ bool g_tune_loaded = false;
 
 std::string tune_key(const dda_target* t, int prec, int R) {
   std::ostringstream k;
-  k << (prec ? "f64" : "f32") << ' ' << t->nx << ' ' << t->ny << ' ' << t->nz << ' ' << t->Lx
-    << ' ' << t->Ly << ' ' << t->Lz << ' ' << R;
+  k << 'v' << kScheduleVersion << (prec ? " f64 " : " f32 ") << t->nx << ' ' << t->ny << ' '
+    << t->nz << ' ' << t->Lx << ' ' << t->Ly << ' ' << t->Lz << ' ' << R;
   return k.str();
 }
 

@@ -72,3 +72,16 @@ def test_an_entry_the_target_can_run_is_used(tmp_path):
     assert again["fp32"]["x_lines"] == 3 and not again["fp32"]["z_stage_ghat"] & 16
     assert max(err.values()) <= 4e-6
     assert len(path.read_text().splitlines()) == 2
+
+
+def test_an_entry_of_earlier_kernels_is_timed_anew(tmp_path):
+    """Lines without a version were timed before there were register passes."""
+    path = tmp_path / "tune.txt"
+    old = "f32 13 16 16 25 32 32 1 : 3 16 4 13 0 128 128 128\n"
+    path.write_text(old)
+    sched, err = _step(path, (13, 16, 16))
+    assert sched["fp32"]["x_lines"] != 3
+    assert max(err.values()) <= 4e-6
+    assert path.read_text().startswith(old) and len(path.read_text().splitlines()) == 3
+    again, _ = _step(path, (13, 16, 16))
+    assert again == sched and len(path.read_text().splitlines()) == 3
