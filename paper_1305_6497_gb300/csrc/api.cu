@@ -1522,8 +1522,9 @@ dda_status dda_target_create(int nx, int ny, int nz, const uint8_t* occ, const u
       t->twzp.ensure(sizeof(float2) * tp.size());
       CK(cudaMemcpy(t->twzp.p, tp.data(), sizeof(float2) * tp.size(), cudaMemcpyHostToDevice));
     }
-    // and of the register passes, [k1 < R1][j2 < R2]: w_L^(j2 (2 k1 + parity)), both
-    // parities side by side (re, im even; re, im odd), or w_L^(j2 k1) for odd L
+    // and of the register passes, [k1 < R1][j2 < R2]: w_L^(j2 k) for the two frequencies
+    // k of row k1 (reg_odd_shift) side by side (re, im even; re, im odd), or for the one,
+    // k1, of odd L
     std::vector<float4> tr;
     auto reg_twiddles = [&](int axis, int r1, int r2) {
       const Roots& w = roots[axis];
@@ -1532,7 +1533,8 @@ dda_status dda_target_create(int nx, int ny, int nz, const uint8_t* occ, const u
       for (int k = 0; k < r1; ++k)
         for (int j = 0; j < r2; ++j) {
           const long long even = L % 2 ? (long long)j * k : 2LL * j * k;
-          const int a = (int)(even % L), b = (int)(((2LL * k + 1) * j) % L);
+          const long long odd = 2 * ((k + reg_odd_shift(r1)) % r1) + 1;
+          const int a = (int)(even % L), b = (int)(odd * j % L);
           tr.push_back(make_float4((float)w.re[a], (float)w.im[a], (float)w.re[b],
                                    (float)w.im[b]));
         }

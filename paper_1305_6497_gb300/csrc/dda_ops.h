@@ -111,6 +111,9 @@ size_t zpair_smem_bytes(int Lz, int tile, bool gs);
 // to 167 planes).
 bool z_reg_plan(int Lz, int nz, int* R1, int* R2);
 constexpr int kZRegTile = 8;
+// The register passes of even lengths hold, in row k1 of their exchange, the frequencies
+// 2 k1 and 2 ((k1 + reg_odd_shift) mod R1) + 1 (modulo 2 R1; see EoMap).
+constexpr int reg_odd_shift(int R1) { return R1 % 2 ? (R1 - 1) / 2 : reg_odd_shift(R1 / 2); }
 // The same for the x passes (xpass_reg.cuh), and their CTAs per right-hand side.
 bool x_reg_plan(int Lx, int nx, int* R1, int* R2);
 int x_reg_blocks(int Lx, int rows);

@@ -12,7 +12,10 @@
 // stores for one k2 are 2 R1 consecutive values, its loads of box vectors R2.
 //
 // Shared memory: [row][k1][j2] 16-byte (even, odd) pairs, k1 rows an odd number of
-// pairs apart, so that step 2's half-warps (k1, parity) hit distinct banks.
+// pairs apart, so that step 2's half-warps (k1, parity) hit distinct banks.  A row's odd
+// half belongs to another k1 (reg_place); the other way round, with natural rows here
+// and the odd frequencies permuted in the spectra, a warp's stores fell into more
+// 32-byte sectors (216 points: 63.4 us where this takes 60.6).
 //
 // What bounds it: HBM on grids larger than L2 (256^3 box: the update of p and its
 // transform move 4.8 GB in 651 us, all of the measured copy rate), load latency on
@@ -20,8 +23,7 @@
 // warps, each CTA waiting for its slowest stage.  Forward / inverse pass, two
 // right-hand sides, before and now: 256^3 box 1135 / 1319 -> 651 / 1079 us, 128^3
 // 164 / 202 -> 88 / 123, 64^3 29 / 43 -> 18 / 26, 100x75x135 98 / 121 -> 48 / 85,
-// 16^3 17 / 26 -> 6.5 / 12 us.  The error of a product against 64 bits is 5.9e-8
-// where it was 5.7e-8 (RMS).
+// 16^3 17 / 26 -> 6.5 / 12 us.
 #pragma once
 
 #include "reg_step.cuh"
@@ -154,7 +156,8 @@ k_x_fwd_reg(OpView<float> op, const float2* in, float2* buf, const int* active,
       const int line = u / NQ, q = u % NQ;  // q = 2 k1 + parity, or k1
       const int row = row0 + line;
       if (row >= rows) break;
-      const float2* s = sm + EL * (line * K::LS + (EO ? q >> 1 : q) * K::ROW) + (EO ? q & 1 : 0);
+      const int at = reg_place<R1, EO>(q);
+      const float2* s = sm + EL * (line * K::LS + (EO ? at >> 1 : at) * K::ROW) + (EO ? at & 1 : 0);
       cv<float> a[R2];
 #pragma unroll
       for (int j = 0; j < R2; ++j) {
@@ -169,6 +172,12 @@ k_x_fwd_reg(OpView<float> op, const float2* in, float2* buf, const int* active,
     }
     __syncwarp();
   }
+}
+
+// a x - s with two roundings a part: the diagonal term is the largest of a product, and
+// rounding it before s is taken off it was the largest single error left in one
+__device__ __forceinline__ float2 diag_minus(float2 a, float2 x, float2 s) {
+  return make_float2(fmaf(a.x, x.x, fmaf(-a.y, x.y, -s.x)), fmaf(a.x, x.y, fmaf(a.y, x.x, -s.y)));
 }
 
 template <int R1, int R2, bool EO, int MODE>
@@ -223,7 +232,8 @@ k_x_inv_reg(OpView<float> op, const float2* buf, const float2* xin, float2* yout
         a[k] = {e.x, e.y};
       }
       rdft<R2, true>(a);
-      float2* s = sm + EL * (line * K::LS + (EO ? q >> 1 : q) * K::ROW) + (EO ? q & 1 : 0);
+      const int at = reg_place<R1, EO>(q);
+      float2* s = sm + EL * (line * K::LS + (EO ? at >> 1 : at) * K::ROW) + (EO ? at & 1 : 0);
 #pragma unroll
       for (int j = 0; j < R2; ++j) s[EL * j] = make_float2(a[j].re, a[j].im);
     }
@@ -252,7 +262,7 @@ k_x_inv_reg(OpView<float> op, const float2* buf, const float2* xin, float2* yout
       for (int j = 0; j < NJ; ++j) {
         if (j == NJ - 1 && !last) break;
         C out = make_float2(0.f, 0.f);
-        if (cm[j]) out = csub(cmul(ai[3 * cm[j] + c], xv[j]), s[j]);
+        if (cm[j]) out = diag_minus(ai[3 * cm[j] + c], xv[j], s[j]);
         yout[g0 + R2 * j] = out;
         if constexpr (MODE == XOUT_RV) {
           acc.add(0, hv[j].x * out.x + hv[j].y * out.y);

@@ -67,7 +67,8 @@ k_y_reg(OpView<float> op, float2* buf, const int* active) {
     }
   };
   auto element = [&](int t, int q) {
-    return sm + EL * ((EO ? q >> 1 : q) * R2 * TILE + t) + (EO ? q & 1 : 0);
+    const int at = reg_place<R1, EO>(q);
+    return sm + EL * ((EO ? at >> 1 : at) * R2 * TILE + t) + (EO ? at & 1 : 0);
   };
   if (!INV) {
     for (int u = threadIdx.x; u < K::U1; u += NT) {

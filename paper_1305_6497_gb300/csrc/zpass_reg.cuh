@@ -10,12 +10,14 @@
 // is R1-point DFTs, twiddles, R2-point DFTs, each in the registers of one
 // thread, with one exchange through shared memory between them:
 //   1. thread (column t, j2, component): x at z = j2 + R2 j1, both halves'
-//      R1-point DFTs over j1, twiddles w_L^(j2 (2 k1 + parity)), to shared memory;
+//      R1-point DFTs over j1 (eo_step), twiddles w_L^(j2 (2 k1 + parity)), to shared
+//      memory;
 //   2. thread (t, k1, parity): the R2-point DFTs over j2 of all three components,
-//      which gives them at the frequencies 2 (k1 + R1 k2) + parity; the multiply,
-//      and the inverse R2-point DFTs, back in place;
-//   3. thread (t, j2, component): conjugate twiddles, inverse R1-point DFTs, even
-//      half + odd half conj(w_L^j), stored for z < nz.
+//      which gives them at the frequencies 2 (k1 + R1 k2) + parity (the odd ones' k1
+//      counted as reg_freq does); the multiply, and the inverse R2-point DFTs, back in
+//      place;
+//   3. thread (t, j2, component): conjugate twiddles, inverse R1-point DFTs, the halves
+//      joined (eo_step_inv), stored for z < nz.
 // Every value crosses shared memory twice (once each way) and a pass meets two
 // barriers; the kernels that keep lines in shared memory and transform them stage
 // by stage cross it 2 x 3 times for L = 512 and meet ten.
@@ -213,16 +215,17 @@ k_fft_z_reg(OpView<float> op, float2* buf, int R, int per, const int* active) {
         }
         rdft<R2, false>(s[c]);
       }
-      // position j holds kz = 2 (k2 + R1 j) + p2 (odd L: k2 + R1 j): row kz of the
-      // octant up to L / 2, row L - kz (z reflected) above; for even R2 every j is on
-      // one side (kz = n sits on both)
+      // position j holds kz = kf + 2 R1 j (odd L: + R1 j): row kz of the octant up to
+      // L / 2, row L - kz (z reflected) above; for even R2 every j is on one side (kz = n
+      // sits on both)
       constexpr int KS = EO ? 2 : 1;
-      const float4* glo = g + KS * k2 + p2;
-      const float4* ghi = g + L - KS * k2 - p2;
+      const int kf = reg_freq<R1, EO>(EO ? 2 * k2 + p2 : k2);
+      const float4* glo = g + kf;
+      const float4* ghi = g + L - kf;
       static_for<R2>([&](auto jc) {
         constexpr int j = decltype(jc)::value;
         constexpr bool mid = R2 % 2 == 1 && 2 * j + 1 == R2;
-        const bool fz = mid ? KS * (k2 + R1 * j) + p2 > L / 2 : 2 * j >= R2;
+        const bool fz = mid ? kf + KS * R1 * j > L / 2 : 2 * j >= R2;
         const float4* gp = fz ? ghi - KS * R1 * j : glo + KS * R1 * j;
         const float4 g0 = gp[0], g1 = gp[Hz], g2 = gp[2 * Hz];
         // odd components change sign under the reflection of an odd axis
