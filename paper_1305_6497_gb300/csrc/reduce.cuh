@@ -170,6 +170,41 @@ template <int NV> struct ChunkAcc<float, NV> {
   }
 };
 
+// The same for a kernel whose threads hold many elements (the register x passes: up to
+// eight groups of rows, some 200 elements): the totals of chunks of up to 8 elements,
+// closed by flush(), are added up with the additions' errors kept, so that the bound
+// stays at 16 x 2^-24 whatever their number.
+template <int NV> struct LongAcc {
+  float tot[NV], low[NV], part[NV];
+  __host__ __device__ __forceinline__ LongAcc() {
+#pragma unroll
+    for (int i = 0; i < NV; ++i) tot[i] = low[i] = part[i] = 0.0f;
+  }
+  __host__ __device__ __forceinline__ void add(int k, float v) { part[k] += v; }
+  __host__ __device__ __forceinline__ void flush() {
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      const float s = tot[i] + part[i], b = s - tot[i];
+      low[i] += (tot[i] - (s - b)) + (part[i] - b);
+      tot[i] = s;
+      part[i] = 0.0f;
+    }
+  }
+  __host__ __device__ __forceinline__ float total(int i) const { return tot[i] + low[i]; }
+  template <int NOUT> __device__ __forceinline__ void write(double* partials) {
+    static_assert(NOUT <= NV, "more outputs than sums");
+    float v[NOUT], out[NOUT];
+#pragma unroll
+    for (int i = 0; i < NOUT; ++i) v[i] = total(i);
+    block_sum_f<NOUT>(v, out);
+    if (threadIdx.x == 0) {
+      double* o = partials + ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * NOUT;
+#pragma unroll
+      for (int i = 0; i < NOUT; ++i) o[i] = (double)out[i];
+    }
+  }
+};
+
 #define GRID_LOOP(i, n) \
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (n); \
        i += (int64_t)gridDim.x * blockDim.x)

@@ -216,7 +216,7 @@ k_x_inv_reg(OpView<float> op, const float2* buf, const float2* xin, float2* yout
   const int64_t plane_sz = (int64_t)op.Ly * Lx;
   const C* src = buf + (int64_t)r * 3 * op.nz * plane_sz;
   const float4* __restrict__ tw = op.twx_reg;
-  ChunkAcc<float, 4> acc;
+  LongAcc<4> acc;
   for (int row0 = (blockIdx.x * kXRegWarps + wid) * K::LW; row0 < rows;
        row0 += gridDim.x * kXRegWarps * K::LW) {
     for (int u = lane; u < K::U2; u += 32) {
@@ -267,18 +267,17 @@ k_x_inv_reg(OpView<float> op, const float2* buf, const float2* xin, float2* yout
         if constexpr (MODE == XOUT_RV) {
           acc.add(0, hv[j].x * out.x + hv[j].y * out.y);
           acc.add(1, hv[j].x * out.y - hv[j].y * out.x);
-          acc.step();
         } else if constexpr (MODE == XOUT_TS) {
           acc.add(0, out.x * xv[j].x + out.y * xv[j].y);
           acc.add(1, out.x * xv[j].y - out.y * xv[j].x);
           acc.add(2, out.x * out.x + out.y * out.y);
-          acc.step();
         } else if constexpr (MODE == XOUT_QT) {
           acc.add(0, xv[j].x * out.x - xv[j].y * out.y);
           acc.add(1, xv[j].x * out.y + xv[j].y * out.x);
-          acc.step();
         }
+        if (j == 7 && NJ > 8) acc.flush();
       }
+      acc.flush();
     }
     __syncwarp();
   }
