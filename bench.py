@@ -25,6 +25,7 @@ import hashlib
 import json
 import math
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -128,11 +129,25 @@ def pass_bytes(box, grid, s):
     return per_rhs, per_launch
 
 
+def _pass_sources():
+    """The files the passes are compiled from: their units and all they include."""
+    csrc = os.path.join(ROOT, "paper_1305_6497_gb300", "csrc")
+    todo = [f for f in os.listdir(csrc) if re.fullmatch(r"(matvec|[xyz]pass)_\w+\.cu", f)]
+    seen = set()
+    while todo:
+        f = todo.pop()
+        if f in seen or not os.path.exists(os.path.join(csrc, f)):
+            continue
+        seen.add(f)
+        with open(os.path.join(csrc, f)) as fh:
+            todo += re.findall(r'(?m)^#include "([^"]+)"', fh.read())
+    return [os.path.join(csrc, f) for f in sorted(seen)]
+
+
 def _source_hash():
     h = hashlib.sha256()
-    for f in ("matvec_impl.cuh", "fft_core.cuh", "fft_plan.cuh", "matvec_fixed.cu",
-              "zpass_pair.cuh", "dda_common.cuh", "fft_reg.cuh", "reg_step.cuh", "zpass_reg.cuh"):
-        with open(os.path.join(ROOT, "paper_1305_6497_gb300", "csrc", f), "rb") as fh:
+    for f in _pass_sources():
+        with open(f, "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
 
