@@ -382,6 +382,7 @@ static OpView<T> make_view(const dda_target* t, const void* ghat, const void* ai
   v.Lx = t->Lx; v.Ly = t->Ly; v.Lz = t->Lz;
   v.Hx = t->Lx / 2 + 1; v.Hy = t->Ly / 2 + 1; v.Hz = t->Lz / 2 + 1;
   v.nbox = t->nbox;
+  v.gl = ghat_f32_layout(t->twroff[2] >= 0, v.Hx, v.Hy, v.Hz);
   v.chain = !t->prof.on;
   v.src_z0 = 0;
   v.src_z1 = t->nz;
@@ -431,8 +432,8 @@ static void build_transform(dda_target* t, double kd, int kind, DevBuf& g64, Dev
   const int* pos = t->perm.as<int>() + (t->Lx + t->Ly + t->Lz);
   CK(launch_green_transform(op, pos, pos + t->Lx, pos + t->Lx + t->Ly, kd, kind,
                             t->ws.scr64.as<double2>(), g64.as<double2>(),
-                            g32 ? g32->as<float2>() : nullptr, gdf ? gdf->as<df64c>() : nullptr,
-                            t->stream));
+                            g32 ? g32->as<float2>() : nullptr, op.gl,
+                            gdf ? gdf->as<df64c>() : nullptr, t->stream));
   CK(cudaStreamSynchronize(t->stream));
 }
 

@@ -8,7 +8,7 @@
 //    z pass transforms along z, multiplies by the Green tensor transform and
 //    transforms back in place, and the inverse y and x passes shrink back;
 //  - Green tensor transform: one octant [Lz/2+1][Ly/2+1][Lx/2+1][6] complex
-//    (components xx, xy, xz, yy, yz, zz side by side; FP32:
+//    (components xx, xy, xz, yy, yz, zz side by side; FP32 with a register z pass:
 //    [Ly/2+1][Lx/2+1][3][Lz/2+1][2], pairs of components with hz fastest), the
 //    rest follows from the parity of each component in each axis.
 #pragma once
@@ -152,11 +152,18 @@ __host__ __device__ __forceinline__ int fast_div(int q, unsigned long long m) {
   return (int)(((unsigned long long)q * m) >> 36);
 }
 
-// Element (complex) of component c (xx, xy, xz, yy, yz, zz) at octant point
-// (hz, hy, hx) of the FP32 Green transform.
-__host__ __device__ __forceinline__ int64_t ghat_f32_offset(int Hx, int Hz, int hz, int hy, int hx,
-                                                            int c) {
-  return ((((int64_t)hy * Hx + hx) * 3 + (c >> 1)) * Hz + hz) * 2 + (c & 1);
+// Layout of the FP32 Green transform: elements (complex) from one octant point to the
+// next in z and, x fastest, in (y, x), and 16-byte pieces from one pair of components (xx
+// xy | xz yy | yz zz) to the next.  The register z kernel copies columns whole and wants hz
+// fastest; the shared-memory kernels read neighbouring columns at one hz, the components
+// side by side (hz fastest cost them up to 10%: z pass of a 50x50x185 box 284 -> 315 us).
+struct GhatLayout {
+  int64_t sz, sxy;
+  int piece;
+};
+inline GhatLayout ghat_f32_layout(bool z_fastest, int Hx, int Hy, int Hz) {
+  if (z_fastest) return {2, 6 * (int64_t)Hz, Hz};
+  return {6 * (int64_t)Hx * Hy, 6, 1};
 }
 
 // Everything a matvec kernel needs about one target's operator.
@@ -173,7 +180,7 @@ template <typename T> struct OpView {
                                   // the FP64 x and y passes leave them out
   const uint8_t* comp;            // [nbox] 0 = vacant, else composition 1..ncomp
   const C* ghat;                  // octant, already divided by Lx*Ly*Lz: [Hz][Hy][Hx][6],
-                                  // FP32 [Hy][Hx][3][Hz][2] (see ghat_f32_offset)
+                                  // FP32 as gl says
   const C* ainv;                  // [R][ncomp+1][3] alpha^{-1} per RHS and lattice axis
                                   // (the polarizability tensor's diagonal), entry 0 unused
   int ncomp1;                     // ncomp + 1
@@ -189,6 +196,7 @@ template <typename T> struct OpView {
   int* zerr;                      // set to 1 by a kernel whose bounded wait on a copy ran out
   unsigned long long div_nx, div_ny, div_nz, div_Lx;     // fast_div magics
   AxisPlan px, py, pz;
+  GhatLayout gl;
 };
 
 // ---- launches that overlap their predecessor's end ---------------------------

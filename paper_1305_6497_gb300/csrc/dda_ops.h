@@ -73,11 +73,12 @@ bool z_wide_plan(int Lz, int nz, int* R1, int* R2);
 // FP32 and double-float where given (null: not written).  kind: bit 0 = filtered
 // (FCD) scalar Green function; bit 1 = the magnetic vector h (B = h x P) in
 // components 0..2 (3..5 zero) instead of G.  posx .. posz: position holding each
-// frequency; scratch: green_scratch_bytes.
+// frequency; scratch: green_scratch_bytes; gl: layout of g32.
 size_t green_scratch_bytes(int nz, int Lx, int Ly);
 cudaError_t launch_green_transform(const OpView<double>& op, const int* posx, const int* posy,
                                    const int* posz, double kd, int kind, double2* scratch,
-                                   double2* g64, float2* g32, df64c* gdf, cudaStream_t st);
+                                   double2* g64, float2* g32, GhatLayout gl, df64c* gdf,
+                                   cudaStream_t st);
 
 // ---- Krylov / vector kernels -----------------------------------------------
 struct KState {

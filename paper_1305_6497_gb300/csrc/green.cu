@@ -261,7 +261,8 @@ k_green_y(int ny, int nz, AxisPlan P, const double2* __restrict__ tw, const int*
 __global__ void __launch_bounds__(512)
 k_green_z(int nz, AxisPlan P, const double2* __restrict__ tw, const int* __restrict__ pos, int Hx,
           int Hy, int kind, int tile, int64_t first, double scale, const double2* __restrict__ buf,
-          double2* __restrict__ g64, float2* __restrict__ g32, df64c* __restrict__ gdf) {
+          double2* __restrict__ g64, float2* __restrict__ g32, GhatLayout gl,
+          df64c* __restrict__ gdf) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double2* s = reinterpret_cast<double2*>(smem_raw);
   const int L = P.L, Hz = L / 2 + 1, c = blockIdx.x;
@@ -286,7 +287,7 @@ k_green_z(int nz, AxisPlan P, const double2* __restrict__ tw, const int* __restr
     g64[o] = w;
     if (gdf) gdf[o] = from_io<df64c>(w);
     if (g32)
-      g32[ghat_f32_offset(Hx, Hz, hz, (int)(col / Hx), (int)(col % Hx), c)] =
+      g32[hz * gl.sz + col * gl.sxy + (c >> 1) * 2 * gl.piece + (c & 1)] =
           make_float2((float)w.x, (float)w.y);
   }
 }
@@ -297,7 +298,8 @@ size_t green_scratch_bytes(int nz, int Lx, int Ly) {
 
 cudaError_t launch_green_transform(const OpView<double>& op, const int* posx, const int* posy,
                                    const int* posz, double kd, int kind, double2* scratch,
-                                   double2* g64, float2* g32, df64c* gdf, cudaStream_t st) {
+                                   double2* g64, float2* g32, GhatLayout gl, df64c* gdf,
+                                   cudaStream_t st) {
   const int Hx = op.Lx / 2 + 1, Hy = op.Ly / 2 + 1;
   const size_t kLimit = 200 * 1024;
   const void* ks[] = {(const void*)k_green_x, (const void*)k_green_y, (const void*)k_green_z};
@@ -330,7 +332,7 @@ cudaError_t launch_green_transform(const OpView<double>& op, const int* posx, co
     const int nt = (int)(tiles - t0 < 65535 ? tiles - t0 : 65535);
     k_green_z<<<dim3(6, nt), th, (size_t)tile * op.Lz * sizeof(double2), st>>>(
         op.nz, op.pz, op.twz, posz, Hx, Hy, kind, tile, t0 * tile,
-        1.0 / ((double)op.Lx * op.Ly * op.Lz), scratch, g64, g32, gdf);
+        1.0 / ((double)op.Lx * op.Ly * op.Lz), scratch, g64, g32, gl, gdf);
     note_launch();
   }
   return cudaGetLastError();

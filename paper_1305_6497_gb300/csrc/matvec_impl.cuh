@@ -372,13 +372,11 @@ template <typename C> struct ZIO {
 
 // The six components of Ghat at an octant point, xx, xy, xz, yy, yz, zz: side by
 // side in FP64 and double-float ([hz][hy][hx][6]); in FP32 three 16-byte pieces
-// (xx xy | xz yy | yz zz) ghat_piece_f32(op) elements apart, each piece a plane
-// with hz fastest ([hy][hx][3][hz][2]), so that threads at neighbouring z
-// frequencies of one column read neighbouring 16-byte words.
+// (xx xy | xz yy | yz zz), gl.piece of them from one to the next (see GhatLayout).
 template <typename T>
 __device__ __forceinline__ const cplx_t<T>* ghat_at(const OpView<T>& op, int hz, int hy, int hx) {
   if constexpr (std::is_same<T, float>::value)
-    return op.ghat + ghat_f32_offset(op.Hx, op.Hz, hz, hy, hx, 0);
+    return op.ghat + hz * op.gl.sz + ((int64_t)hy * op.Hx + hx) * op.gl.sxy;
   else
     return op.ghat + 6 * (((int64_t)hz * op.Hy + hy) * op.Hx + hx);
 }
@@ -391,9 +389,9 @@ template <> struct G6<float> {
     v[2] = make_float2(b.x, b.y); v[3] = make_float2(b.z, b.w);
     v[4] = make_float2(c.x, c.y); v[5] = make_float2(c.z, c.w);
   }
-  static __device__ __forceinline__ void load(const float2* g, int Hz, float2 (&v)[6]) {
+  static __device__ __forceinline__ void load(const float2* g, int piece, float2 (&v)[6]) {
     const float4* q = reinterpret_cast<const float4*>(g);
-    const float4 a = __ldg(q), b = __ldg(q + Hz), c = __ldg(q + 2 * Hz);
+    const float4 a = __ldg(q), b = __ldg(q + piece), c = __ldg(q + 2 * piece);
     v[0] = make_float2(a.x, a.y); v[1] = make_float2(a.z, a.w);
     v[2] = make_float2(b.x, b.y); v[3] = make_float2(b.z, b.w);
     v[4] = make_float2(c.x, c.y); v[5] = make_float2(c.z, c.w);
@@ -486,7 +484,7 @@ __device__ __forceinline__ void z_mid(cplx_t<T>* s, int ps, int ncol, int col0, 
           G6<T>::load_smem(gs + 6 * (hz * TILE + t), g);
         } else {
           const int hx = fx ? op.Lx - kx : kx;
-          G6<T>::load(ghat_at<T>(op, hz, hy, hx), op.Hz, g);
+          G6<T>::load(ghat_at<T>(op, hz, hy, hx), op.gl.piece, g);
         }
         spectral_mul<T, CROSS>(g, fx, fy, fz, q + i * ps, TILE);
       }
@@ -518,7 +516,7 @@ __device__ __forceinline__ void ghat_tile_async(const OpView<T>& op, cplx_t<T>* 
     if (t < ncol) {
       const int kx = op.kx_at[col0 + t];
       const int hx = kx > (op.Lx >> 1) ? op.Lx - kx : kx;
-      const int64_t piece = std::is_same<T, float>::value ? 16 * (int64_t)op.Hz : 16;
+      const int64_t piece = std::is_same<T, float>::value ? 16 * (int64_t)op.gl.piece : 16;
       const char* src = reinterpret_cast<const char*>(ghat_at<T>(op, hz, hy, hx)) + piece * ch;
       char* dst = reinterpret_cast<char*>(gs + 6 * (hz * TILE + t)) + 16 * ch;
       cp_async<16>(dst, src);
@@ -576,7 +574,7 @@ k_fft_z_mul(OpView<T> op, cplx_t<T>* __restrict__ buf, int ps, const int* __rest
       const bool fx = kx > (Lx >> 1);
       C g[6];
       if (GS) G6<T>::load_smem(gs + 6 * t, g);
-      else G6<T>::load(ghat_at<T>(op, 0, hy, fx ? Lx - kx : kx), op.Hz, g);
+      else G6<T>::load(ghat_at<T>(op, 0, hy, fx ? Lx - kx : kx), op.gl.piece, g);
       spectral_mul<T, CROSS>(g, fx, fy, false, s + t, TILE);
     }
     __syncthreads();
@@ -693,7 +691,7 @@ k_fft_z_mul_p(OpView<float> op, float2* __restrict__ buf, const int* __restrict_
             G6<float>::load_smem(gs + 6 * (hz * TILE + t), g);
           } else {
             const int hx = fx ? Lx - kx : kx;
-            G6<float>::load(ghat_at<float>(op, hz, hy, hx), op.Hz, g);
+            G6<float>::load(ghat_at<float>(op, hz, hy, hx), op.gl.piece, g);
           }
           spectral_mul<float, false>(g, fx, fy, fz, q + i * PS, TILE);
         }

@@ -234,7 +234,7 @@ __device__ __forceinline__ void ghat_tile_pairs_async(const OpView<float>& op, f
     if (t < ncol) {
       const int kx = op.kx_at[col0 + t];
       const int hx = kx > (op.Lx >> 1) ? op.Lx - kx : kx;
-      const float2* src = ghat_at<float>(op, hz, hy, hx) + (int64_t)2 * op.Hz * ch;
+      const float2* src = ghat_at<float>(op, hz, hy, hx) + (int64_t)2 * op.gl.piece * ch;
       cp_async<16>(gs + t * stride + 6 * hz + 2 * ch, src);
     }
   }
@@ -433,7 +433,7 @@ k_fft_z_pairs(OpView<float> op, float2* __restrict__ buf, int R, const int* __re
           if (GS) {
             G6<float>::load_smem(gs + (2 * tp2 + e) * gstride + 6 * hz, g);
           } else {
-            G6<float>::load(ghat_at<float>(op, hz, hy, hxm[e]), op.Hz, g);
+            G6<float>::load(ghat_at<float>(op, hz, hy, hxm[e]), op.gl.piece, g);
           }
           spectral_mul<float, false>(g, fxm[e], fy, fz, e ? bb : a, 1);
         }

@@ -161,7 +161,7 @@ k_fft_z_wide(OpView<T> op, cplx_t<T>* __restrict__ buf, const int* __restrict__ 
     const int kz = 2 * (k1 + R1 * k2) + p, kx = op.kx_at[col0 + t];
     const bool fz = kz > n, fx = kx > (Lx >> 1);
     C g[6];
-    G6<T>::load(ghat_at<T>(op, fz ? L - kz : kz, hy, fx ? Lx - kx : kx), op.Hz, g);
+    G6<T>::load(ghat_at<T>(op, fz ? L - kz : kz, hy, fx ? Lx - kx : kx), 0, g);
     wide_mul<T, CROSS>(g, fx, fy, fz, sm + u, 2 * n * TILE);
   }
   __syncthreads();
