@@ -80,6 +80,36 @@ struct DevBuf {
   template <typename X> X* as() const { return reinterpret_cast<X*>(p); }
 };
 
+// A table within a target's one buffer of them (see TableBuilder); null when it has none.
+struct DevTable {
+  void* p = nullptr;
+  template <typename X> X* as() const { return reinterpret_cast<X*>(p); }
+};
+
+// The tables of a new target, collected on the host and uploaded together: an allocation
+// and a copy of its own for each of nine was a third of a small target's creation (16^3:
+// 176 -> 118 us with its destruction).
+class TableBuilder {
+ public:
+  template <typename X> void add(DevTable& t, const std::vector<X>& v) {
+    if (v.empty()) return;
+    parts_.push_back({&t, host_.size()});
+    const char* b = reinterpret_cast<const char*>(v.data());
+    host_.insert(host_.end(), b, b + v.size() * sizeof(X));
+    host_.resize((host_.size() + 255) / 256 * 256);
+  }
+  void upload(DevBuf& d) {
+    d.ensure(host_.size());
+    CK(cudaMemcpy(d.p, host_.data(), host_.size(), cudaMemcpyHostToDevice));
+    for (const Part& q : parts_) q.table->p = d.as<char>() + q.offset;
+  }
+
+ private:
+  struct Part { DevTable* table; size_t offset; };
+  std::vector<Part> parts_;
+  std::vector<char> host_;
+};
+
 // ---------------------------------------------------------------------------
 // FFT plans (Stockham radix sequence and twiddles, host side)
 // ---------------------------------------------------------------------------
@@ -338,12 +368,13 @@ struct dda_target {
   int device = 0;
   cudaStream_t stream = nullptr;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
-  DevBuf comp, site, tw64, tw32, twdf, perm;  // perm: k_at x|y|z, then pos x|y|z
-  DevBuf twzp;  // FP32 z twiddles of the column-pair kernel's plan (when it has one)
-  DevBuf tww, twd;  // z twiddles of zpass_wide.cuh, double-float and FP64 (with a plan)
-  DevBuf twr;   // FP32 twiddles of the register passes, x | y | z (axes with a plan)
+  DevBuf comp, site, tables;  // tables: the following
+  DevTable tw64, tw32, twdf, perm;  // perm: k_at x|y|z, then pos x|y|z
+  DevTable twzp;  // FP32 z twiddles of the column-pair kernel's plan (when it has one)
+  DevTable tww, twd;  // z twiddles of zpass_wide.cuh, double-float and FP64 (with a plan)
+  DevTable twr;   // FP32 twiddles of the register passes, x | y | z (axes with a plan)
   int twroff[3] = {-1, -1, -1};
-  DevBuf zerr;  // one int: a kernel's bounded wait on a copy ran out
+  DevTable zerr;  // one int: a kernel's bounded wait on a copy ran out
   AxisPlan px{}, py{}, pz{};
   int twoff[3] = {0, 0, 0};
   // Green transform cache
@@ -1392,13 +1423,7 @@ void dda_target_destroy(dda_target* t) {
   cudaSetDevice(t->device);
   if (t->stream) cudaStreamSynchronize(t->stream);
   t->ws.release_all();
-  t->comp.release(); t->site.release(); t->tw64.release(); t->tw32.release(); t->twdf.release();
-  t->twzp.release();
-  t->twr.release();
-  t->tww.release();
-  t->twd.release();
-  t->zerr.release();
-  t->perm.release();
+  t->comp.release(); t->site.release(); t->tables.release();
   t->g64.release(); t->g32.release(); t->gdf.release(); t->h64.release();
   t->prof.destroy();
   t->graphs[0].reset();
@@ -1500,18 +1525,14 @@ dda_status dda_target_create(int nx, int ny, int nz, const uint8_t* occ, const u
       t64.push_back(make_double2(1, 0)); t32.push_back(make_float2(1, 0));
       tdf.push_back(make_float4(1, 0, 0, 0));
     }
-    t->tw64.ensure(sizeof(double2) * t64.size());
-    t->tw32.ensure(sizeof(float2) * t32.size());
-    t->twdf.ensure(sizeof(float4) * tdf.size());
-    CK(cudaMemcpy(t->tw64.p, t64.data(), sizeof(double2) * t64.size(), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(t->tw32.p, t32.data(), sizeof(float2) * t32.size(), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(t->twdf.p, tdf.data(), sizeof(float4) * tdf.size(), cudaMemcpyHostToDevice));
+    TableBuilder tables;
+    tables.add(t->tw64, t64);
+    tables.add(t->tw32, t32);
+    tables.add(t->twdf, tdf);
     kat.insert(kat.end(), posall.begin(), posall.end());
     for (int i = 0; i < std::max({t->Lx, t->Ly, t->Lz}); ++i) kat.push_back(i);  // natural order
-    t->perm.ensure(sizeof(int) * kat.size());
-    CK(cudaMemcpy(t->perm.p, kat.data(), sizeof(int) * kat.size(), cudaMemcpyHostToDevice));
-    t->zerr.ensure(sizeof(int));
-    CK(cudaMemset(t->zerr.p, 0, sizeof(int)));
+    tables.add(t->perm, kat);
+    tables.add(t->zerr, std::vector<int>{0});
     // twiddles of the column-pair z kernel's own radix plan (FP32)
     const std::vector<int> prs = pair_plan_radices(t->Lz);
     if (!prs.empty()) {
@@ -1520,8 +1541,7 @@ dda_status dda_target_create(int nx, int ny, int nz, const uint8_t* occ, const u
       make_plan_radices(roots[2], prs, wr, wi, ka);
       std::vector<float2> tp(std::max<size_t>(1, wr.size()), make_float2(1, 0));
       for (size_t i = 0; i < wr.size(); ++i) tp[i] = make_float2((float)wr[i], (float)wi[i]);
-      t->twzp.ensure(sizeof(float2) * tp.size());
-      CK(cudaMemcpy(t->twzp.p, tp.data(), sizeof(float2) * tp.size(), cudaMemcpyHostToDevice));
+      tables.add(t->twzp, tp);
     }
     // and of the register passes, [k1 < R1][j2 < R2]: w_L^(j2 k) for the two frequencies
     // k of row k1 (reg_odd_shift) side by side (re, im even; re, im odd), or for the one,
@@ -1544,10 +1564,7 @@ dda_status dda_target_create(int nx, int ny, int nz, const uint8_t* occ, const u
     if (x_reg_plan(t->Lx, t->nx, &r1, &r2)) reg_twiddles(0, r1, r2);
     if (x_reg_plan(t->Ly, t->ny, &r1, &r2)) reg_twiddles(1, r1, r2);
     if (z_reg_plan(t->Lz, t->nz, &r1, &r2)) reg_twiddles(2, r1, r2);
-    if (!tr.empty()) {
-      t->twr.ensure(sizeof(float4) * tr.size());
-      CK(cudaMemcpy(t->twr.p, tr.data(), sizeof(float4) * tr.size(), cudaMemcpyHostToDevice));
-    }
+    tables.add(t->twr, tr);
     // [parity][k1][j2] in double-float (the refinement's residual passes) and FP64
     if (z_wide_plan(t->Lz, t->nz, &r1, &r2)) {
       std::vector<float4> td;
@@ -1562,11 +1579,10 @@ dda_status dda_target_create(int nx, int ny, int nz, const uint8_t* occ, const u
                                      (float)(im - (long double)ih)));
             tq.push_back(make_double2((double)re, (double)im));
           }
-      t->twd.ensure(sizeof(double2) * tq.size());
-      CK(cudaMemcpy(t->twd.p, tq.data(), sizeof(double2) * tq.size(), cudaMemcpyHostToDevice));
-      t->tww.ensure(sizeof(float4) * td.size());
-      CK(cudaMemcpy(t->tww.p, td.data(), sizeof(float4) * td.size(), cudaMemcpyHostToDevice));
+      tables.add(t->twd, tq);
+      tables.add(t->tww, td);
     }
+    tables.upload(t->tables);
   } catch (const CudaFail& f) {
     dda_status s = from_cuda(f);
     dda_target_destroy(t);
@@ -1607,8 +1623,7 @@ int64_t dda_solve_hbm_bytes(const dda_target* t, const dda_solve_params* p) {
 // workspace and its near-field box.
 static int64_t held_bytes(dda_target* t) {
   int64_t b = 0;
-  for (const DevBuf* d : {&t->comp, &t->site, &t->tw64, &t->tw32, &t->twdf, &t->twzp, &t->twr, &t->tww, &t->twd, &t->perm,
-                          &t->g64, &t->g32, &t->gdf, &t->h64})
+  for (const DevBuf* d : {&t->comp, &t->site, &t->tables, &t->g64, &t->g32, &t->gdf, &t->h64})
     b += (int64_t)d->bytes;
   b += t->ws.bytes();
   if (t->nf) b += held_bytes(t->nf);
@@ -1641,9 +1656,10 @@ int64_t dda_estimate_solve_bytes(int nx, int ny, int nz, int64_t n_dipoles, int 
   if (solve < 0) return -1;
   const int64_t Lsum = (int64_t)d.Lx + d.Ly + d.Lz;
   // dda_target_create: composition grid, site list, twiddles (FP64, FP32,
-  // double-float, and the FP32 z kernels' own) and the frequency/position tables
+  // double-float, the z kernels' and the register passes' own) and the
+  // frequency/position tables, each on a 256-byte boundary
   const int64_t created = nbox + 8 * n_dipoles + Lsum * (16 + 8 + 16) + 2 * Lsum * 4 +
-                          4 * std::max({d.Lx, d.Ly, d.Lz}) + 40 * (int64_t)d.Lz + 8 * Lsum + 3 * 256;
+                          4 * std::max({d.Lx, d.Ly, d.Lz}) + 40 * (int64_t)d.Lz + 16 * Lsum + 12 * 256;
   return created + solve;
 }
 
