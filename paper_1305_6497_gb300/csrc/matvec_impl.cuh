@@ -1027,18 +1027,22 @@ MatvecLaunch plan_matvec(const OpView<T>& op) {
   while (nl < 64 && (size_t)(2 * nl) * (op.Lx + 1) * sizeof(C) <= 36 * 1024) nl <<= 1;
   // small grids: fewer lines per CTA (at least 4) until two CTAs per SM have some
   const int rows = 3 * op.nz * op.ny;
-  constexpr bool wide = std::is_same<T, double>::value;  // double-float follows it
-  while (nl > 4 && (rows / nl < 304 || (wide && op.Lx <= 256 && nl * op.Lx > 800))) nl >>= 1;
+  const bool wide = std::is_same<T, double>::value;  // double-float follows it
+  const bool small = wide && op.Lx <= 160;
+  if (!wide || small)
+    while (nl > 4 && (rows / nl < 304 || (small && nl * op.Lx > 1280))) nl >>= 1;
   L.x_lines = nl;
   // FP32: no more threads than the lines have 8-point butterflies.  FP64 and
-  // double-float lines up to 256 points: two warps and up to 800 points a CTA, so that
-  // many CTAs share an SM and none waits long at its stages' barriers.  Both x passes
-  // with 256 threads and 36 KB a CTA, with a thread per 8 points, and so: FP64 41^3 box
-  // 174, 209, 166 us, 36x41x36 112, 116, 107, 81^3 1015, 1143, 939, 48^3 191, 191, 177;
-  // double-float 41^3 101, 107, 90, 64^3 187, 187, 170.  Longer lines keep 256 (L = 360:
-  // 308 against 310 of a thread per 8 points, double-float 168 against 173).
+  // double-float lines up to 160 points: up to 1280 points a CTA and two warps, four above
+  // 800 points, so that many CTAs share an SM and none waits long at its stages' barriers.
+  // Both x passes with 256 threads and 36 KB a CTA, with a thread per 8 points, and so:
+  // FP64 41^3 box 174, 209, 166 us, 36x41x36 112, 116, 107, 48^3 191, 191, 177; double-
+  // float 41^3 101, 107, 90, 80x60x60 244, 244, 226.  Longer lines keep 36 KB and 256: no
+  // count of lines and threads was as good for all of them (250 points: 4 lines and 128
+  // threads 862 us against 844, double-float 334 against 375; 200 points, 1200 rows: 4
+  // lines and 256 threads 94 against 88).
   L.x_threads = !wide ? std::min(256, std::max(64, (nl * op.Lx / 8 + 31) / 32 * 32))
-                      : op.Lx <= 256 ? 64 : 256;
+                : !small ? 256 : nl * op.Lx > 800 ? 128 : 64;
   L.x_smem = (size_t)op.Lx * (nl + 1) * sizeof(C);
   L.x_reg = std::is_same<T, float>::value && x_reg_plan(op.Lx, op.nx, nullptr, nullptr);
   L.y_reg = std::is_same<T, float>::value && x_reg_plan(op.Ly, op.ny, nullptr, nullptr);
