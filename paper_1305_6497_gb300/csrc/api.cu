@@ -1856,7 +1856,8 @@ dda_status dda_solve(dda_target* t, const dda_solve_params* p, dda_solve_result*
       x_nonzero = true;
     }
     OpView<double> op64 = make_view<double>(t, t->g64.p, w.ainv64.p, t->tw64.p);
-    OpView<float> op32 = make_view<float>(t, t->g32.p, w.ainv32.p, t->tw32.p);
+    OpView<float> op32 =
+        within_solve(make_view<float>(t, t->g32.p, w.ainv32.p, t->tw32.p));
     OpView<df64> opdf = make_view<df64>(t, t->gdf.p, w.ainvdf.p, t->twdf.p);
     // the refinement's residuals r = E - A x: FFT passes in double-float
     // arithmetic (FP64-level accuracy at FP32 rates) unless FP64 is requested
@@ -2400,7 +2401,8 @@ dda_status dda_autotune(dda_target* t, double kd, int n_rhs) {
       if (!v.empty() && schedule_fault(t, prec != 0, v.data())) v.clear();
       if (v.empty()) {
         if (prec == 0) {
-          OpView<float> op = make_view<float>(t, t->g32.p, w.ainv32.p, t->tw32.p);
+          OpView<float> op =
+              within_solve(make_view<float>(t, t->g32.p, w.ainv32.p, t->tw32.p));
           MatvecLaunch L = t->L32;
           CK(autotune_matvec<float>(op, L, n_rhs, w.x32.as<float2>(), w.r32.as<float2>(),
                                     w.scr32.as<float2>(), t->stream));

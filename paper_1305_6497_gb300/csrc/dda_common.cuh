@@ -174,8 +174,9 @@ template <typename T> struct OpView {
   int Hx, Hy, Hz;                 // octant sizes L/2 + 1
   int64_t nbox;                   // nx*ny*nz
   int chain;                      // host, see launch_chained: 0 -- ordinary launches; 1 --
-                                  // the passes of a product are chained; 2 -- and so is
-                                  // its first pass, which a kernel precedes
+                                  // the passes of a product are chained; 3 -- so they are,
+                                  // within a solve; 2 -- and its first pass, which a
+                                  // kernel precedes
   int src_z0, src_z1;             // planes outside [src_z0, src_z1) of the input hold zeros:
                                   // the FP64 x and y passes leave them out
   const uint8_t* comp;            // [nbox] 0 = vacant, else composition 1..ncomp
@@ -216,14 +217,24 @@ template <typename T> struct OpView {
 // 75x60x50 77 and 70; in the graph of a solve, whose launches are closer together, 64^3
 // 18.05 and 17.5 ms, 36x41x36 6.09 and 5.88.  The FP64 and double-float passes are not
 // chained: the 16^3 FP64 solve took 1.56 ms ordinary and 1.73 chained (their CTAs are
-// few and large, and those that wait hold the registers of those that work).
+// few and large, and those that wait hold the registers of those that work).  Nor is
+// the inverse y pass within a solve: behind a z pass of several waves its CTAs cost up
+// to 9% of an iteration (100x75x135 1136 us with it chained, 1035 ordinary, 1044 with no
+// kernel chained; 128^3 1953, 1817, 1830; 96^3 900, 854, 857; 24^3 74.2, 72.7, 72.1; the
+// most it gave was 0.8%, 36x41x36).  A product on its own, launched kernel by kernel,
+// gains from it (16^3 23.6 against 26.6 us, 72^3 85.5 against 89.3).
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 template <class P> __device__ __forceinline__ P* chained(P* p) {
   asm volatile("" : "+l"(p)::"memory");
   return p;
 }
-// A view for the products inside an iteration, which a kernel precedes.
+// A view for the products of a solve, and for those inside an iteration, which a kernel
+// precedes.
+template <typename V> V within_solve(V op) {
+  if (op.chain) op.chain = 3;
+  return op;
+}
 template <typename V> V follows_kernel(V op) {
   if (op.chain) op.chain = 2;
   return op;

@@ -108,8 +108,10 @@ size_t zpair_smem_bytes(int Lz, int tile, bool gs);
 // The two-step register z kernel (FP32, zpass_reg.cuh) covers z length Lz of a box
 // of nz planes: Lz / 2 = R1 R2 for even Lz, Lz = R1 R2 for odd, in the list of plans
 // (R1, R2 returned unless null), and nz such that only the last of a thread's rows can
-// lie beyond the box (of the even lengths up to 512 that leaves out the boxes of 163
-// to 167 planes).
+// lie beyond the box.  Of the boxes up to 256 sites that leaves out sides of up to 6
+// (lengths below 15), 61-63 and 123-125 (125, 250), 121-122 and 241-243 (243, 486),
+// 181-188 (375), 201-203 (405), 244-250 (500) and, with more than one row beyond the
+// box, 163-167 (360; x and y: 163 and 164 only).
 bool z_reg_plan(int Lz, int nz, int* R1, int* R2);
 constexpr int kZRegTile = 8;
 // The register passes of even lengths hold, in row k1 of their exchange, the frequencies

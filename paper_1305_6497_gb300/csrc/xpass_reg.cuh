@@ -18,12 +18,12 @@
 // 32-byte sectors (216 points: 63.4 us where this takes 60.6).
 //
 // What bounds it: HBM on grids larger than L2 (256^3 box: the update of p and its
-// transform move 4.8 GB in 651 us, all of the measured copy rate), load latency on
-// smaller ones.  The kernels that keep lines in shared memory ran a third of the
-// warps, each CTA waiting for its slowest stage.  Forward / inverse pass, two
-// right-hand sides, before and now: 256^3 box 1135 / 1319 -> 651 / 1079 us, 128^3
-// 164 / 202 -> 88 / 123, 64^3 29 / 43 -> 18 / 26, 100x75x135 98 / 121 -> 48 / 85,
-// 16^3 17 / 26 -> 6.5 / 12 us.
+// transform move 4.8 GB in 648 us, all of the measured copy rate, the inverse with its
+// inner products 4.1 GB in 661 us, 0.91 of it), load latency on smaller ones.  The
+// kernels that keep lines in shared memory ran a third of the warps, each CTA waiting for
+// its slowest stage.  Forward / inverse pass, two right-hand sides, before and now: 256^3
+// box 1135 / 1319 -> 648 / 661 us, 128^3 164 / 202 -> 87 / 92, 64^3 29 / 43 -> 17 / 23,
+// 100x75x135 98 / 121 -> 48 / 64, 16^3 17 / 26 -> 7 / 11.5 us.
 #pragma once
 
 #include "reg_step.cuh"

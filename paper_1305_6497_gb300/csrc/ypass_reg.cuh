@@ -8,11 +8,11 @@
 // too few CTAs per SM (136 rows: 53 us against 47, 150: 46 against 42), while
 // above the whole lines win again (256 rows: 66 against 80, 225: 41 against 49).
 //
-// What bounds it: HBM on grids larger than L2 (256^3 box: 4.8 GB in 901 us, 0.79 of
+// What bounds it: HBM on grids larger than L2 (256^3 box: 4.8 GB in 875 us, 0.81 of
 // the measured copy rate), latency on smaller ones.  Forward / inverse pass, two
 // right-hand sides, before (shared-memory stages, compiled or generic plans) and
-// now: 128^3 168 / 203 -> 116 / 105 us, 256^3 1000 / 1013 -> 901 / 939, 100x75x135
-// 179 / 142 -> 70 / 60, 60x45x54 31 / 31 -> 12.5 / 12.3, 64^3 19 / 19 -> 18 / 18.
+// now: 128^3 168 / 203 -> 116 / 106 us, 256^3 1000 / 1013 -> 875 / 936, 100x75x135
+// 179 / 142 -> 69 / 61, 60x45x54 31 / 31 -> 12.3 / 12.2, 64^3 19 / 19 -> 18 / 18.
 #pragma once
 
 #include "xpass_reg.cuh"
@@ -135,8 +135,10 @@ void launch_y_reg(bool inv, const OpView<float>& op, int R, float2* buf, const i
                   cudaStream_t st) {
   using K = YRegCfg<R1, R2, EO>;
   const dim3 g((op.Lx + K::TILE - 1) / K::TILE, 3 * op.nz, R);
-  launch_chained(op.chain, inv ? k_y_reg<R1, R2, EO, true> : k_y_reg<R1, R2, EO, false>, g, K::NT,
-                 K::smem, st, op, buf, active);
+  // the inverse pass of a solve is not chained (see launch_chained)
+  launch_chained(inv ? op.chain == 1 : op.chain != 0,
+                 inv ? k_y_reg<R1, R2, EO, true> : k_y_reg<R1, R2, EO, false>, g, K::NT, K::smem, st,
+                 op, buf, active);
 }
 template <int R1, int R2, bool EO> cudaError_t configure_y_reg() {
   const int smem = (int)YRegCfg<R1, R2, EO>::smem;

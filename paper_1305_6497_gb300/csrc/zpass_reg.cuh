@@ -32,13 +32,13 @@
 // without a conflict, and so do the reads of the Ghat tile (see ROW and GS).
 //
 // What bounds it: instruction issue and the shared-memory pipe (of the 64x64x256
-// brick: 49% and 55% busy, 29% of the DRAM bandwidth, 153 thread instructions per
+// brick: 48% and 53% busy, 29% of the measured copy rate, 154 thread instructions per
 // stored point against 214 of the column-pair kernel).  8 columns per CTA (64-byte
 // rows in global memory) up to n = 96 and 4 above leave room for two to four CTAs.
 // Per launch with two right-hand sides, before (the default one-tile or, where
 // named, the tuned kernel) and now: 256^3 box 8600 (tuned pair kernel 4460) ->
-// 3414 us; 128^3 866 -> 333 us; 64x64x256 582 (tuned 284) -> 202 us; 100x75x135
-// 589 -> 180 us; 48x96x144 319 -> 128 us; 64^3 76 (tuned 54) -> 47 us.
+// 3473 us; 128^3 866 -> 326 us; 64x64x256 582 (tuned 284) -> 206 us; 100x75x135
+// 589 -> 179 us; 48x96x144 319 -> 129 us; 64^3 76 (tuned 54) -> 51 us.
 #pragma once
 
 #include "reg_step.cuh"
@@ -291,8 +291,9 @@ void launch_z_reg(const OpView<float>& op, int R, float2* buf, const int* active
   using K = ZRegCfg<R1, R2, EO>;
   const int tiles = (op.Lx + K::TILE - 1) / K::TILE, hy = op.Ly / 2 + 1;
   // passes per CTA: as many as leave four waves of CTAs (more passes save Ghat
-  // reads, fewer waves lose to the last one: 100x75x135, 2 RHS, 262 us with four
-  // waves, 271 with eight, 301 with one pass per CTA)
+  // reads, fewer waves lose to the last one: two right-hand sides, four waves, eight,
+  // one pass per CTA: 100x75x135 179, 187, 213 us, 128^3 326, 326, 407, 64x64x256 206,
+  // 217, 251)
   int64_t per = (int64_t)tiles * hy * 2 * R / (152 * K::MINB * 4);
   per = per < 1 ? 1 : per > 2 * R ? 2 * R : per;
   const dim3 g(tiles, hy, (unsigned)((2 * R + per - 1) / per));
